@@ -430,6 +430,30 @@ bool make_stage_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t 
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool make_wide_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K) {
+    auto encode = tensor_map_encoder();
+    if (!encode || K % 8 != 0 || (reinterpret_cast<uintptr_t>(base) & 15) != 0) return false;
+    const cuuint64_t dims[2] = {K, rows};
+    const cuuint64_t strides[1] = {K * 2};
+    const cuuint32_t box[2] = {64, 128};
+    const cuuint32_t estr[2] = {1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool make_wide_kv_map(CUtensorMap* map, const void* base, uint64_t rows, uint32_t hd) {
+    auto encode = tensor_map_encoder();
+    if (!encode || hd % 64 != 0 || (reinterpret_cast<uintptr_t>(base) & 15) != 0) return false;
+    const cuuint64_t dims[3] = {64, rows, hd / 64};
+    const cuuint64_t strides[2] = {(cuuint64_t)hd * 2, 128};
+    const cuuint32_t box[3] = {64, 128, hd / 64};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 template <int EPI>
 static cudaError_t launch_f32(const GemvArgs& a, cudaStream_t s) {
     const int pitch = a.kc + 4;

@@ -63,6 +63,10 @@ bool make_stage_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t 
 // K % 64 == 0: 3-D view {64, rows, K / 64}, box of `chunks` chunks (one copy
 // per stage); otherwise 2-D, box {64, 16} (one copy per chunk).
 bool make_weight_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K, uint32_t chunks);
+// Maps of the wide kernels: boxes of 64 columns x 128 rows with the 128-byte
+// swizzle (an operand's stage), and 128 whole cache rows of hd elements.
+bool make_wide_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K);
+bool make_wide_kv_map(CUtensorMap* map, const void* base, uint64_t rows, uint32_t hd);
 int gemv_groups(int N, int dtype);              // output groups (argmax candidates) of a launch
 
 // ----------------------------------------------------------------- chain
@@ -105,6 +109,47 @@ struct ChainArgs {
 size_t chain_counter_ints();
 cudaError_t launch_chain(const ChainArgs& a, cudaStream_t s);
 int sm_count();
+
+// ------------------------------------------------------------------ wide
+// bf16 models: one projection over many rows as a tensor-core GEMM (wide.cu).
+enum WideKind { WK_QKV = 0, WK_RESID = 1, WK_SWIGLU = 2, WK_ARGMAX = 3 };
+struct WideArgs {
+    CUtensorMap amap, wmap;     // make_wide_map of the input rows and of the weights
+    int M, N, K;                // rows, output features (WK_SWIGLU: d_ff), inputs
+    int tiles_m, tiles_n;       // set by launch_wide
+    int d;                      // model width (the norm's)
+    float eps;
+    const float* ss_in;         // [ss_n][ss_ld] sums of squares of the input rows (all kinds but WK_RESID)
+    float* ss_out;              // WK_RESID: the same, one slot per tile of the output
+    int ss_n, ss_ld;
+    float* x;                   // WK_RESID: [M][N] fp32 residual, added to
+    __nv_bfloat16* xg;          // WK_RESID: [M][N] new residual times gain, the next projection's input
+    const __nv_bfloat16* gain;
+    __nv_bfloat16* act;         // WK_SWIGLU: [M][N]
+    __nv_bfloat16* q;           // WK_QKV: [M][hq hd] prepared queries
+    __nv_bfloat16 *kcache, *vcache;   // WK_QKV: this layer's [hk][max_seq][hd]
+    const float* rope;
+    const __nv_bfloat16 *q_norm, *k_norm;
+    int hq, hk, max_seq, p0;    // WK_QKV: row m is at position p0 + m
+    unsigned long long* best;   // WK_ARGMAX: [M] keys, merged by atomicMax
+    int* err;                   // device status word
+};
+int wide_tiles_n(int kind, int N);
+cudaError_t launch_wide(int kind, int hd, const WideArgs& a, cudaStream_t s);
+cudaError_t launch_wide_embed(const __nv_bfloat16* embed, const int32_t* tok, int M, int d, int vocab, float* x,
+                              __nv_bfloat16* xg, const __nv_bfloat16* gain, float* ss, int ss_n, int ss_ld,
+                              cudaStream_t s);
+// Causal attention of M rows at positions p0 .. over the cache (wide_attn.cu).
+struct WideAttnArgs {
+    CUtensorMap qmap;           // make_wide_map of q [rows][hq hd]
+    CUtensorMap kvmap;          // make_wide_kv_map of the whole cache
+    int kv_row_k, kv_row_v;     // first cache row of this layer's K and V
+    int M, p0, hq, hk, max_seq;
+    int blocks;                 // set by launch_wide_attention
+    __nv_bfloat16* out;         // [M][hq hd]
+    int* err;
+};
+cudaError_t launch_wide_attention(int hd, const WideAttnArgs& a, cudaStream_t s);
 
 // ------------------------------------------------------------- attention
 struct AttnArgs {

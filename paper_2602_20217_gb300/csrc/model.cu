@@ -181,7 +181,8 @@ static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 struct Layout {
     size_t kv, rope, x, ss, xg, qkv, attn_out, act, attn_part, gemv_part, counters, logits, amax_val,
         amax_idx, tok, hist, hist_snap, hist_idx, sims, mask, obj, wts, select, chain_ctr, best, tpt_masks,
-        tpt_tok, tpt_info, tpt_out, dyn, samp, slice, qbuf, total;
+        tpt_tok, tpt_info, tpt_out, dyn, samp, slice, qbuf, wide, total;
+    int wide_rows;   // rows of a wide chunk (0: fp32 models, no wide path)
     int n_chunks_max;
     size_t gemv_part_floats;
     int counters_n;
@@ -209,6 +210,37 @@ static bool config_ok(const ks_config* c) {
     if (c->hist_init_rows < 1 || c->hist_init_rows > c->max_rows) return false;
     if (!(c->rms_eps > 0.f) || !(c->rope_theta > 1.0)) return false;
     return true;
+}
+
+// Rows of a wide prefill chunk: enough for the GEMMs to be bound by the
+// tensor cores, few enough for the activations to stay in L2.
+constexpr int kWideChunk = 2048;
+constexpr int kWideMinRows = 64;   // fewer lead rows take the ordinary passes
+static int wide_chunk_rows(const ks_config* c) {
+    return std::min(kWideChunk, (int)align_up((size_t)c->max_seq, 256));
+}
+
+// Buffers of a wide pass over `rows` rows, 256-byte aligned pieces from `base`.
+struct WideLayout {
+    size_t x, xg, q, ao, act, ss, bytes;
+};
+static WideLayout wide_layout(const ks_config* c, int rows, size_t base) {
+    const size_t M = rows, d = c->d_model, hqd = (size_t)c->n_q_heads * c->head_dim;
+    size_t off = base;
+    auto take = [&](size_t bytes) {
+        const size_t o = off;
+        off = align_up(off + bytes, 256);
+        return o;
+    };
+    WideLayout W{};
+    W.x = take(sizeof(float) * M * d);
+    W.xg = take(sizeof(__nv_bfloat16) * M * d);
+    W.q = take(sizeof(__nv_bfloat16) * M * hqd);
+    W.ao = take(sizeof(__nv_bfloat16) * M * hqd);
+    W.act = take(sizeof(__nv_bfloat16) * M * c->d_ff);
+    W.ss = take(sizeof(float) * M * wide_tiles_n(WK_RESID, c->d_model));
+    W.bytes = off - base;
+    return W;
 }
 
 static Layout make_layout(const ks_config* c) {
@@ -246,16 +278,22 @@ static Layout make_layout(const ks_config* c) {
     L.qkv = take(sizeof(float) * (size_t)R * nqkv);
     L.attn_out = take(es * (size_t)R * c->n_q_heads * hd);
     L.act = take(es * (size_t)R * c->d_ff);
-    L.attn_part = take(sizeof(float) * (size_t)R * c->n_q_heads * L.n_chunks_max * (hd + 4));
     L.gemv_part = take(sizeof(float) * std::max<size_t>(gp, 1));
     L.counters = take(sizeof(int) * (size_t)L.counters_n);
-    L.logits = take(sizeof(float) * (size_t)R * c->vocab);
     L.amax_val = take(sizeof(float) * (size_t)gemv_groups(c->vocab, c->dtype) * 16);
     L.amax_idx = take(sizeof(int) * (size_t)gemv_groups(c->vocab, c->dtype) * 16);
     // tokens: rows[R+1] | target[R] | result[R+3] | err | prompt/out[max_seq]
     L.tok = take(sizeof(int) * ((size_t)3 * R + 8 + c->max_seq));
+    // A prefill's wide chunks use the space of what is dead until its last
+    // pass: attention partials, logits, history and its snapshot; only models
+    // of few layers need more than these take.
+    L.wide_rows = c->dtype == KS_DTYPE_BF16 ? wide_chunk_rows(c) : 0;
+    L.wide = off;
+    L.attn_part = take(sizeof(float) * (size_t)R * c->n_q_heads * L.n_chunks_max * (hd + 4));
+    L.logits = take(sizeof(float) * (size_t)R * c->vocab);
     L.hist = take(sizeof(float) * (size_t)(nsub + 1) * L.hist_slots * R * d);
     L.hist_snap = take(sizeof(float) * (size_t)(nsub + 1) * R * d);  // the prefill's history entry
+    off = std::max(off, L.wide + wide_layout(c, L.wide_rows, 0).bytes);
     L.hist_idx = take(sizeof(int) * (size_t)L.hist_slots * R);
     L.sims = take(sizeof(float) * nsub);
     L.mask = take(nsub);
@@ -356,6 +394,9 @@ struct ks_model {
     int64_t h2d = 0, d2h = 0;
     // bf16: TMA maps of every weight matrix and of the three projection inputs
     std::vector<CUtensorMap> map_qkv, map_o, map_gu, map_down;
+    // wide path: operand maps of the weights, of the chunk's inputs and of the cache
+    std::vector<CUtensorMap> wide_qkv, wide_o, wide_gu, wide_down;
+    CUtensorMap wide_xg, wide_q, wide_ao, wide_act, wide_kv;
     CUtensorMap map_lm, map_xg[16], map_xg2[16], map_attn_out[16], map_act[16];  // [R - 1]: boxes of R rows
     KlassTiming timing[kKlasses];
 };
@@ -657,6 +698,73 @@ static ks_status forward(ks_model* m, const int32_t* tok, int R, int p0, const u
     return KS_OK;
 }
 
+// The whole target over M <= wide_rows prompt rows at positions p0..: fills
+// the K/V cache of every layer.  No logits and no history: a prefill's last
+// rows take the ordinary pass (forward).
+static ks_status wide_forward(ks_model* m, const int32_t* tok, int M, int p0) {
+    const ks_config& c = m->cfg;
+    const int d = c.d_model, F = c.d_ff, L = c.n_layers, hd = c.head_dim, hqd = c.n_q_heads * hd;
+    const int nqkv = (c.n_q_heads + 2 * c.n_kv_heads) * hd;
+    cudaStream_t s = m->stream;
+    const WideLayout W = wide_layout(&c, m->lay.wide_rows, m->lay.wide);
+    auto bf = [](const void* p) { return reinterpret_cast<const __nv_bfloat16*>(p); };
+    WideArgs g{};
+    g.M = M;
+    g.d = d;
+    g.eps = c.rms_eps;
+    g.ss_in = g.ss_out = reinterpret_cast<float*>(m->ws + W.ss);
+    g.ss_n = wide_tiles_n(WK_RESID, d);
+    g.ss_ld = m->lay.wide_rows;
+    g.x = reinterpret_cast<float*>(m->ws + W.x);
+    g.xg = reinterpret_cast<__nv_bfloat16*>(m->ws + W.xg);
+    g.act = reinterpret_cast<__nv_bfloat16*>(m->ws + W.act);
+    g.q = reinterpret_cast<__nv_bfloat16*>(m->ws + W.q);
+    g.rope = m->rope;
+    g.hq = c.n_q_heads;
+    g.hk = c.n_kv_heads;
+    g.max_seq = c.max_seq;
+    g.p0 = p0;
+    g.err = m->err;
+    KS_TRY(launch(m, K_EMBED, [&] {
+        return launch_wide_embed(bf(m->embed), tok, M, d, c.vocab, g.x, g.xg, bf(m->attn_norm[0]), g.ss_out, g.ss_n,
+                                 g.ss_ld, s);
+    }, "prompt embed"));
+    auto project = [&](int kind, int klass, const CUtensorMap& in, const CUtensorMap& w, int N, int K) -> ks_status {
+        g.amap = in;
+        g.wmap = w;
+        g.N = N;
+        g.K = K;
+        return launch(m, klass, [&] { return launch_wide(kind, hd, g, s); }, "prompt projection",
+                      2.0 * K * (double)(kind == WK_SWIGLU ? 2 * N : N));
+    };
+    for (int l = 0; l < L; ++l) {
+        g.kcache = reinterpret_cast<__nv_bfloat16*>(kcache(m, l));
+        g.vcache = reinterpret_cast<__nv_bfloat16*>(vcache(m, l));
+        g.q_norm = c.qk_norm ? bf(m->q_norm[l]) : nullptr;
+        g.k_norm = c.qk_norm ? bf(m->k_norm[l]) : nullptr;
+        KS_TRY(project(WK_QKV, K_QKV, m->wide_xg, m->wide_qkv[l], nqkv, d));
+        WideAttnArgs at{};
+        at.qmap = m->wide_q;
+        at.kvmap = m->wide_kv;
+        at.kv_row_k = 2 * l * c.n_kv_heads * c.max_seq;
+        at.kv_row_v = (2 * l + 1) * c.n_kv_heads * c.max_seq;
+        at.M = M;
+        at.p0 = p0;
+        at.hq = c.n_q_heads;
+        at.hk = c.n_kv_heads;
+        at.max_seq = c.max_seq;
+        at.out = reinterpret_cast<__nv_bfloat16*>(m->ws + W.ao);
+        at.err = m->err;
+        KS_TRY(launch(m, K_ATTN, [&] { return launch_wide_attention(hd, at, s); }, "prompt attention"));
+        g.gain = bf(m->mlp_norm[l]);
+        KS_TRY(project(WK_RESID, K_OPROJ, m->wide_ao, m->wide_o[l], d, hqd));
+        KS_TRY(project(WK_SWIGLU, K_GATEUP, m->wide_xg, m->wide_gu[l], F, d));
+        g.gain = bf(l + 1 < L ? m->attn_norm[l + 1] : m->final_norm);
+        KS_TRY(project(WK_RESID, K_DOWN, m->wide_act, m->wide_down[l], d, F));
+    }
+    return KS_OK;
+}
+
 // Wait for the stream, then read the device status word (set when a kernel's
 // bounded wait on an asynchronous copy gave up).
 static ks_status sync(ks_model* m, const char* what) {
@@ -842,6 +950,23 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
             ok = ok && make_stage_map(&m->map_attn_out[b], m->attn_out, R, hqd, b + 1, 4);
             ok = ok && make_stage_map(&m->map_act[b], m->act, R, F, b + 1, 4);
         }
+        m->wide_qkv.resize(L);
+        m->wide_o.resize(L);
+        m->wide_gu.resize(L);
+        m->wide_down.resize(L);
+        for (int l = 0; l < L && ok; ++l) {
+            ok = ok && make_wide_map(&m->wide_qkv[l], m->w_qkv[l], nqkv, d);
+            ok = ok && make_wide_map(&m->wide_o[l], m->w_o[l], d, hqd);
+            ok = ok && make_wide_map(&m->wide_gu[l], m->w_gate_up[l], 2 * (uint64_t)F, d);
+            ok = ok && make_wide_map(&m->wide_down[l], m->w_down[l], d, F);
+        }
+        const WideLayout W = wide_layout(cfg, lay.wide_rows, lay.wide);
+        ok = ok && make_wide_map(&m->wide_xg, b + W.xg, lay.wide_rows, d);
+        ok = ok && make_wide_map(&m->wide_q, b + W.q, lay.wide_rows, hqd);
+        ok = ok && make_wide_map(&m->wide_ao, b + W.ao, lay.wide_rows, hqd);
+        ok = ok && make_wide_map(&m->wide_act, b + W.act, lay.wide_rows, F);
+        ok = ok && make_wide_kv_map(&m->wide_kv, m->kv, 2 * (uint64_t)L * cfg->n_kv_heads * (uint64_t)cfg->max_seq,
+                                    cfg->head_dim);
         if (!ok) {
             set_error("ks_model_create: TMA descriptor encoding failed");
             delete m;
@@ -957,6 +1082,17 @@ ks_status ks_prefill(ks_model* m, const int32_t* tokens, int32_t n, int32_t* nex
     int start = 0;
     int len = first;
     const int init_slot = 0;
+    // bf16: every row but the last chunk's goes through the wide path, in even
+    // chunks of whole tiles
+    const int lead = n - std::min(n, R);
+    if (m->dtype == KS_DTYPE_BF16 && lead >= kWideMinRows) {
+        const int parts = (lead + m->lay.wide_rows - 1) / m->lay.wide_rows;
+        const int rows = std::min(m->lay.wide_rows, (int)align_up((size_t)(lead + parts - 1) / parts, 256));
+        for (; start < lead; start += rows)
+            KS_TRY(wide_forward(m, m->seq + start, std::min(rows, lead - start), start));
+        start = lead;
+        len = R;
+    }
     while (start < n) {
         const bool last = (start + len == n);
         KS_TRY(forward(m, m->seq + start, len, start, nullptr, last ? init_slot : -1, last ? m->target : nullptr));

@@ -1,0 +1,436 @@
+// Projections over many rows (prompt processing) for bf16 models: the same
+// projections as the chain kernel's, as tensor-core GEMMs.
+//
+// Y[m][n] = sum_k A[m][k] W[n][k], M rows at a time (up to the caller's chunk).
+// Streaming the weights once per 16 rows, as the decode path does, left the
+// tensor cores idle: a 4096-token prompt read every weight 256 times.  Two
+// layers of the Llama-3-8B shape over 4096 tokens: 90.4 -> 3.3 ms for the whole
+// prefill; two of the Qwen3-32B shape over 9001: 391 -> 15.7 ms (68 % of the
+// measured bf16 rate over all its GEMM and attention operations).
+//
+// One CTA pair (cta_group::2) works on a 256 x 256 tile: each CTA stages its
+// 128 rows of A and its half of the tile's 256 weight rows (K-major, 64-column
+// stages, 128-byte swizzle) by TMA, so per SM and stage 32 KB feed 256 x 256 x
+// 64 multiply-adds: 64 bytes per clock at the full tensor rate, where a
+// single CTA's 128 x 256 tile would need 96, more than L2 delivers.  The
+// accumulators (128 lanes x 256 columns per CTA) are double buffered in TMEM,
+// so a tile's epilogue runs under the next tile's MMAs.  Grid: one pair per
+// two SMs, persistent; consecutive tiles share the weight rows (rows fastest),
+// so the weights come from HBM once and the activations stay in L2.
+//
+// Per CTA: warp 0 loads, warp 1 issues the MMAs (the pair's first CTA only),
+// warps 2-5 run the epilogue of the kind:
+//   WK_QKV     1/rms, QK-RMSNorm, RoPE; prepared queries to q, keys and values
+//              to the cache (a thread holds one row, so a head's norm and
+//              rotation stay in its registers);
+//   WK_RESID   residual add, the next RMSNorm's input x * gain and the sums of
+//              squares of the tile's columns (via shared memory, so that the
+//              global accesses are whole lines);
+//   WK_SWIGLU  silu(gate) * up: the pair's first CTA stages gate rows, the
+//              second the up rows of the same features;
+//   WK_ARGMAX  the row's best (logit, id) as a 64-bit key, merged by atomicMax
+//              (any order gives the same argmax).
+// Every wait is bounded; a wait that gives up sets the status word and the
+// CTA leaves after its copies have landed.
+#include "common.cuh"
+#include "internal.h"
+#include "umma.cuh"
+
+#include <algorithm>
+#include <climits>
+
+namespace ks {
+
+namespace {
+
+constexpr int kStages = 6;
+constexpr int kTileM = 256, kTileN = 256, kTileK = 64;
+constexpr uint32_t kHalf = 128 * kTileK * 2;               // 128 rows of one operand: 16 KB
+constexpr uint32_t kStageBytes = 2 * kHalf;                // A half, then W half
+constexpr uint32_t kPairBytes = 2 * kStageBytes;           // both CTAs' bytes of a stage
+constexpr int kWideThreads = 192;
+constexpr int kEpiPitch = 36;                              // floats per row of the staging area
+constexpr size_t kEpiBytes = 4 * 32 * kEpiPitch * sizeof(float);
+constexpr size_t kWideSmem = 1024 + (size_t)kStages * kStageBytes + kEpiBytes;
+constexpr uint32_t kIdesc = umma_idesc(256, 256, false);
+constexpr uint32_t kSbo = 1024;                            // 8 rows of 128 bytes
+
+// 1 / rms of row m from the per-tile sums of squares, in tile order.
+KS_DEV float row_scale(const WideArgs& a, int m) {
+    float s = 0.f;
+    for (int q = 0; q < a.ss_n; ++q) s += a.ss_in[(size_t)q * a.ss_ld + m];
+    return rsqrtf(s / (float)a.d + a.eps);
+}
+
+KS_DEV unsigned long long argmax_key(float v, int i) {
+    const uint32_t b = __float_as_uint(v);
+    const uint32_t ord = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+    return ((unsigned long long)ord << 32) | (0xFFFFFFFFu - (uint32_t)i);
+}
+
+KS_DEV void load_chunk(uint32_t (&r)[32], uint32_t addr) {
+    tmem_ld32(r, addr);
+    tmem_wait_ld();
+    tmem_pin(r);
+}
+
+// One head (HD columns at `col`) of this thread's row.
+template <int HD>
+KS_DEV void qkv_head(const WideArgs& a, uint32_t acc, int col, int m, int n, float scale, bool live) {
+    float v[HD];
+#pragma unroll
+    for (int c = 0; c < HD / 32; ++c) {
+        uint32_t r[32];
+        load_chunk(r, acc + col + 32 * c);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[32 * c + i] = __uint_as_float(r[i]) * scale;
+    }
+    if (!live || n >= a.N) return;
+    const int head = n / HD, pos = a.p0 + m;
+    __nv_bfloat16* dst;
+    if (head < a.hq + a.hk) {
+        const __nv_bfloat16* gain = head < a.hq ? a.q_norm : a.k_norm;
+        if (gain != nullptr) {
+            float ss = 0.f;
+#pragma unroll
+            for (int i = 0; i < HD; ++i) ss = fmaf(v[i], v[i], ss);
+            const float inv = rsqrtf(ss / (float)HD + a.eps);
+#pragma unroll
+            for (int i = 0; i < HD; ++i) v[i] = (v[i] * inv) * __bfloat162float(gain[i]);
+        }
+        const float4* rp = reinterpret_cast<const float4*>(a.rope + (size_t)pos * HD);   // (cos, sin) pairs
+#pragma unroll
+        for (int j = 0; j < HD / 2; j += 2) {
+            const float4 cs = rp[j / 2];
+            const float x0 = v[j], y0 = v[j + HD / 2], x1 = v[j + 1], y1 = v[j + 1 + HD / 2];
+            v[j] = x0 * cs.x - y0 * cs.y;
+            v[j + HD / 2] = y0 * cs.x + x0 * cs.y;
+            v[j + 1] = x1 * cs.z - y1 * cs.w;
+            v[j + 1 + HD / 2] = y1 * cs.z + x1 * cs.w;
+        }
+    }
+    if (head < a.hq) {
+        const float qs = 1.4426950408889634f * rsqrtf((float)HD);
+#pragma unroll
+        for (int i = 0; i < HD; ++i) v[i] *= qs;
+        dst = a.q + (size_t)m * a.hq * HD + (size_t)head * HD;
+    } else if (head < a.hq + a.hk) {
+        dst = a.kcache + ((size_t)(head - a.hq) * a.max_seq + pos) * HD;
+    } else {
+        dst = a.vcache + ((size_t)(head - a.hq - a.hk) * a.max_seq + pos) * HD;
+    }
+#pragma unroll
+    for (int i = 0; i < HD; i += 8) {
+        uint4 w;
+        w.x = pack_bf16(v[i], v[i + 1]);
+        w.y = pack_bf16(v[i + 2], v[i + 3]);
+        w.z = pack_bf16(v[i + 4], v[i + 5]);
+        w.w = pack_bf16(v[i + 6], v[i + 7]);
+        *reinterpret_cast<uint4*>(dst + i) = w;
+    }
+}
+
+// Epilogue of one tile by one warp: rows m0 .. m0 + 31 (this thread: m0 +
+// lane), TMEM address `acc` (this warp's lanes, first column of the buffer).
+template <int KIND, int HD>
+KS_DEV void wide_epilogue(const WideArgs& a, uint32_t acc, int m0, int tn, float* stg) {
+    const int lane = threadIdx.x & 31;
+    const int m = m0 + lane;
+    const bool live = m < a.M;
+    if constexpr (KIND == WK_QKV) {
+        const float scale = row_scale(a, live ? m : 0);
+#pragma unroll 1
+        for (int h = 0; h < kTileN / HD; ++h) qkv_head<HD>(a, acc, h * HD, m, tn * kTileN + h * HD, scale, live);
+    } else if constexpr (KIND == WK_SWIGLU) {
+        const float scale = row_scale(a, live ? m : 0);
+        const int n0 = tn * 128;
+#pragma unroll 1
+        for (int c = 0; c < 128; c += 32) {
+            uint32_t g[32], u[32];
+            tmem_ld32(g, acc + c);
+            tmem_ld32(u, acc + 128 + c);
+            tmem_wait_ld();
+            tmem_pin(g);
+            tmem_pin(u);
+            __nv_bfloat16* dst = a.act + (size_t)m * a.N + n0 + c;
+#pragma unroll
+            for (int i = 0; i < 32; i += 8) {
+                uint32_t w[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float g0 = __uint_as_float(g[i + 2 * j]) * scale, g1 = __uint_as_float(g[i + 2 * j + 1]) * scale;
+                    const float u0 = __uint_as_float(u[i + 2 * j]) * scale, u1 = __uint_as_float(u[i + 2 * j + 1]) * scale;
+                    w[j] = pack_bf16(silu(g0) * u0, silu(g1) * u1);
+                }
+                if (live && n0 + c + i < a.N) *reinterpret_cast<uint4*>(dst + i) = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+        }
+    } else if constexpr (KIND == WK_ARGMAX) {
+        const float scale = row_scale(a, live ? m : 0);
+        float bv = -INFINITY;
+        int bi = INT_MAX;
+#pragma unroll 1
+        for (int c = 0; c < kTileN; c += 32) {
+            uint32_t r[32];
+            load_chunk(r, acc + c);
+            const int n = tn * kTileN + c;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const float v = __uint_as_float(r[i]) * scale;
+                if (n + i < a.N && better(v, n + i, bv, bi)) {
+                    bv = v;
+                    bi = n + i;
+                }
+            }
+        }
+        if (live && bi != INT_MAX) atomicMax(&a.best[m], argmax_key(bv, bi));
+    } else {
+        // 32 columns at a time through shared memory: written one row per
+        // thread, read back as whole row pieces of 32 columns
+        float ssq[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) ssq[i] = 0.f;
+        const int sub = lane >> 3, c4 = (lane & 7) * 4;
+#pragma unroll 1
+        for (int c = 0; c < kTileN; c += 32) {
+            uint32_t r[32];
+            load_chunk(r, acc + c);
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 32; i += 4)
+                *reinterpret_cast<uint4*>(stg + lane * kEpiPitch + i) = make_uint4(r[i], r[i + 1], r[i + 2], r[i + 3]);
+            __syncwarp();
+            const int n = tn * kTileN + c + c4;
+            if (n < a.N) {   // N is a multiple of 8
+                const uint2 gw = *reinterpret_cast<const uint2*>(a.gain + n);
+                const float g0 = bf16_lo(gw.x), g1 = bf16_hi(gw.x), g2 = bf16_lo(gw.y), g3 = bf16_hi(gw.y);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int mr = m0 + 4 * i + sub;
+                    if (mr >= a.M) continue;
+                    const float4 v = *reinterpret_cast<const float4*>(stg + (4 * i + sub) * kEpiPitch + c4);
+                    float4* xp = reinterpret_cast<float4*>(a.x + (size_t)mr * a.N + n);
+                    float4 x = *xp;
+                    x.x += v.x;
+                    x.y += v.y;
+                    x.z += v.z;
+                    x.w += v.w;
+                    *xp = x;
+                    *reinterpret_cast<uint2*>(a.xg + (size_t)mr * a.N + n) =
+                        make_uint2(pack_bf16(x.x * g0, x.y * g1), pack_bf16(x.z * g2, x.w * g3));
+                    ssq[i] = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, ssq[i]))));
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) ssq[i] += __shfl_xor_sync(0xffffffffu, ssq[i], o);
+            const int mr = m0 + 4 * i + sub;
+            if ((lane & 7) == 0 && mr < a.M) a.ss_out[(size_t)tn * a.ss_ld + mr] = ssq[i];
+        }
+    }
+}
+
+template <int KIND, int HD>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
+    wide_kernel(const __grid_constant__ WideArgs a) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = reinterpret_cast<unsigned char*>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    float* staging = reinterpret_cast<float*>(smem + (size_t)kStages * kStageBytes);
+    __shared__ __align__(8) uint64_t full[kStages];     // the pair's first CTA: both CTAs' copies have landed
+    __shared__ __align__(8) uint64_t empty[kStages];    // each CTA: the pair's MMAs have read the stage
+    __shared__ __align__(8) uint64_t acc_full[2];       // each CTA: the buffer's accumulators are complete
+    __shared__ __align__(8) uint64_t acc_free[2];       // the pair's first CTA: 8 epilogue warps have read it
+    __shared__ uint32_t tmem_slot;
+    __shared__ uint32_t skip;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t rank = cluster_rank();
+    const int pair = (int)blockIdx.x >> 1, pairs = (int)gridDim.x >> 1;
+    const int tiles = a.tiles_m * a.tiles_n;
+    const int kblocks = (a.K + kTileK - 1) / kTileK;
+
+    if (warp == 1) tmem_alloc<2>(&tmem_slot, 512);
+    if (tid == 0) {
+        for (int i = 0; i < kStages; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&acc_full[i], 1);
+            mbar_init(&acc_free[i], 8);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        // a job whose status word holds an error is void: the pair's first
+        // CTA decides for both (the word can change during the launch)
+        skip = __ldcg(a.err) != 0;
+    }
+    __syncthreads();
+    umma_fence_before();
+    cluster_sync();
+    umma_fence_after();
+    const uint32_t tmem = tmem_slot;
+    if (cluster_load(cluster_addr(&skip, 0)) == 0) {
+        if (warp == 0) {
+            // ------------------------------------------------------ loader
+            if (lane == 0) {
+                bool ok = true;
+                int t = 0;
+                for (int tile = pair; tile < tiles && ok; tile += pairs) {
+                    const int tm = tile % a.tiles_m, tn = tile / a.tiles_m;
+                    const int ra = tm * kTileM + (int)rank * 128;
+                    const int rw = KIND == WK_SWIGLU ? tn * 128 + (int)rank * a.N : tn * kTileN + (int)rank * 128;
+                    for (int kb = 0; kb < kblocks; ++kb, ++t) {
+                        const int st = t % kStages;
+                        if (t >= kStages && !mbar_wait(&empty[st], (uint32_t)((t / kStages - 1) & 1), kWaitLimitNs)) {
+                            ok = false;
+                            break;
+                        }
+                        if (rank == 0) mbar_expect_tx(&full[st], kPairBytes);
+                        const uint32_t bar = cluster_addr(&full[st], 0);
+                        unsigned char* dst = smem + (size_t)st * kStageBytes;
+                        tma_2d_pair(dst, &a.amap, kb * kTileK, ra, bar);
+                        tma_2d_pair(dst + kHalf, &a.wmap, kb * kTileK, rw, bar);
+                    }
+                }
+                if (!ok) {
+                    atomicCAS(a.err, 0, 1);
+                    // copies still in flight land before the pair leaves
+                    if (rank == 0)
+                        for (int q = max(0, t - kStages); q < t; ++q)
+                            mbar_wait(&full[q % kStages], (uint32_t)((q / kStages) & 1), kWaitLimitNs);
+                }
+            }
+        } else if (warp == 1) {
+            // --------------------------------------------------------- MMA
+            if (rank == 0 && lane == 0) {
+                bool ok = true;
+                int t = 0, n = 0;
+                for (int tile = pair; tile < tiles && ok; tile += pairs, ++n) {
+                    const int b = n & 1;
+                    if (n >= 2 && !mbar_wait(&acc_free[b], (uint32_t)((n / 2 - 1) & 1), kWaitLimitNs)) {
+                        ok = false;
+                        break;
+                    }
+                    umma_fence_after();
+                    const uint32_t acc = tmem + (uint32_t)(b * kTileN);
+                    for (int kb = 0; kb < kblocks; ++kb, ++t) {
+                        const int st = t % kStages;
+                        if (!mbar_wait(&full[st], (uint32_t)((t / kStages) & 1), kWaitLimitNs)) {
+                            ok = false;
+                            break;
+                        }
+                        umma_fence_after();
+                        const uint32_t sa = smem_u32(smem + (size_t)st * kStageBytes);
+#pragma unroll
+                        for (int k = 0; k < kTileK / 16; ++k)
+                            umma_ss<2>(acc, umma_desc(sa + 32 * k, 16, kSbo), umma_desc(sa + kHalf + 32 * k, 16, kSbo),
+                                       kIdesc, kb > 0 || k > 0);
+                        umma_commit_pair(&empty[st]);
+                    }
+                    if (ok) umma_commit_pair(&acc_full[b]);
+                }
+                if (!ok) atomicCAS(a.err, 0, 1);
+            }
+        } else {
+            // ---------------------------------------------------- epilogue
+            const int quad = warp & 3;   // the TMEM lanes this warp may read
+            float* stg = staging + (warp - 2) * 32 * kEpiPitch;
+            bool ok = true;
+            int n = 0;
+            for (int tile = pair; tile < tiles; tile += pairs, ++n) {
+                const int b = n & 1;
+                ok = mbar_wait(&acc_full[b], (uint32_t)((n / 2) & 1), kWaitLimitNs);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    ok = false;
+                    break;
+                }
+                umma_fence_after();
+                const int tm = tile % a.tiles_m, tn = tile / a.tiles_m;
+                wide_epilogue<KIND, HD>(a, tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(b * kTileN),
+                                        tm * kTileM + (int)rank * 128 + 32 * quad, tn, stg);
+                umma_fence_before();
+                __syncwarp();
+                if (lane == 0) cluster_arrive(cluster_addr(&acc_free[b], 0));
+            }
+            if (!ok && lane == 0) atomicCAS(a.err, 0, 1);
+        }
+    }
+    __syncthreads();
+    umma_fence_before();
+    cluster_sync();   // neither CTA leaves while the other may still signal it
+    if (warp == 1) tmem_free<2>(tmem, 512);
+}
+
+// Rows of the embedding table as the residual, the first projection's input
+// and the rows' sums of squares (slot 0; the other tiles' slots are zero).
+__global__ void __launch_bounds__(256) wide_embed_kernel(const __nv_bfloat16* embed, const int32_t* tok, int d,
+                                                         int vocab, float* x, __nv_bfloat16* xg,
+                                                         const __nv_bfloat16* gain, float* ss, int ss_n, int ss_ld) {
+    __shared__ float red[9];
+    const int m = blockIdx.x;
+    int t = tok[m];
+    if (t < 0 || t >= vocab) t = 0;
+    const __nv_bfloat16* e = embed + (size_t)t * d;
+    float s = 0.f;
+    for (int k = (int)threadIdx.x * 8; k < d; k += 256 * 8) {   // d is a multiple of 8
+        const uint4 w = *reinterpret_cast<const uint4*>(e + k), g = *reinterpret_cast<const uint4*>(gain + k);
+        const uint32_t ws[4] = {w.x, w.y, w.z, w.w}, gs[4] = {g.x, g.y, g.z, g.w};
+        float v[8];
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            v[2 * i] = bf16_lo(ws[i]);
+            v[2 * i + 1] = bf16_hi(ws[i]);
+            o[i] = pack_bf16(v[2 * i] * bf16_lo(gs[i]), v[2 * i + 1] * bf16_hi(gs[i]));
+            s = fmaf(v[2 * i], v[2 * i], s);
+            s = fmaf(v[2 * i + 1], v[2 * i + 1], s);
+        }
+        float4* xp = reinterpret_cast<float4*>(x + (size_t)m * d + k);
+        xp[0] = make_float4(v[0], v[1], v[2], v[3]);
+        xp[1] = make_float4(v[4], v[5], v[6], v[7]);
+        *reinterpret_cast<uint4*>(xg + (size_t)m * d + k) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+    s = block_sum<8>(s, red);
+    if ((int)threadIdx.x < ss_n) ss[(size_t)threadIdx.x * ss_ld + m] = threadIdx.x == 0 ? s : 0.f;
+}
+
+}  // namespace
+
+int wide_tiles_n(int kind, int N) { return kind == WK_SWIGLU ? (N + 127) / 128 : (N + kTileN - 1) / kTileN; }
+
+cudaError_t launch_wide_embed(const __nv_bfloat16* embed, const int32_t* tok, int M, int d, int vocab, float* x,
+                              __nv_bfloat16* xg, const __nv_bfloat16* gain, float* ss, int ss_n, int ss_ld,
+                              cudaStream_t s) {
+    if (M < 1 || ss_n > 256) return cudaErrorInvalidValue;
+    wide_embed_kernel<<<M, 256, 0, s>>>(embed, tok, d, vocab, x, xg, gain, ss, ss_n, ss_ld);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_wide(int kind, int hd, const WideArgs& args, cudaStream_t s) {
+    if (args.M < 1 || args.N < 1 || args.K < 8 || args.err == nullptr) return cudaErrorInvalidValue;
+    WideArgs a = args;
+    a.tiles_m = (a.M + kTileM - 1) / kTileM;
+    a.tiles_n = wide_tiles_n(kind, a.N);
+    auto run = [&](auto kern) -> cudaError_t {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmem);
+        if (e != cudaSuccess) return e;
+        const int pairs = std::min(sm_count() / 2, a.tiles_m * a.tiles_n);
+        kern<<<2 * pairs, kWideThreads, kWideSmem, s>>>(a);
+        return cudaGetLastError();
+    };
+    switch (kind) {
+        case WK_QKV:
+            if (hd == 128) return run(wide_kernel<WK_QKV, 128>);
+            if (hd == 64) return run(wide_kernel<WK_QKV, 64>);
+            return cudaErrorInvalidValue;
+        case WK_RESID: return run(wide_kernel<WK_RESID, 0>);
+        case WK_SWIGLU: return run(wide_kernel<WK_SWIGLU, 0>);
+        case WK_ARGMAX: return run(wide_kernel<WK_ARGMAX, 0>);
+    }
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace ks

@@ -1,0 +1,303 @@
+// Causal GQA attention for many query rows of one sequence (prompt
+// processing, bf16 models) on the tensor cores.
+//
+// The decode kernel (attn.cu) reads the whole cache once per 16 rows; here a
+// CTA keeps 256 query rows of one head (two tiles of 128) and walks the keys
+// 128 at a time, so K and V tiles are read from L2 once per 256 rows.  Per key
+// tile and query tile:
+//   S = Q K^T          tcgen05.mma, both operands in shared memory, S in TMEM
+//   softmax            one thread per query row: running maximum, P = 2^(S - m)
+//                      in bf16 back into the TMEM columns of S
+//   O += P V           tcgen05.mma with P as the TMEM operand, V as it lies in
+//                      the cache (keys x head_dim: an MN-major operand)
+// The two query tiles alternate: while one is in its softmax, the tensor core
+// works on the other.  O is rescaled only when a row's maximum grew by more
+// than 2^8: the factor 2^(m - m_ref) of the rest stays exact in fp32 and bf16
+// alike (a power of two apart, the relative precision is the same).
+// Queries come prepared (QK-norm, RoPE, log2(e) / sqrt(hd)), the keys and
+// values of these rows are already in the cache.
+//
+// Warps: 0-3 and 4-7 the softmax of query tile 0 and 1, 8 the MMAs, 9 the
+// loads.  TMEM: S0, S1 (128 columns each), O0, O1 (hd columns each).  Longest
+// query blocks first.  Every wait is bounded.
+#include "common.cuh"
+#include "internal.h"
+#include "umma.cuh"
+
+#include <algorithm>
+
+namespace ks {
+
+namespace {
+
+constexpr int kQ = 128;                      // rows of a query tile, keys of a key tile
+constexpr int kChunk = kQ * 128;             // bytes of 128 rows x 64 columns
+constexpr int kRing = 4;                     // K and V tiles in flight
+constexpr int kThreads = 320;
+constexpr float kRescale = 8.f;              // log2 of the growth of a maximum that O is rescaled for
+template <int HD>
+constexpr size_t wide_attn_smem() { return 1024 + (size_t)(2 + kRing) * (HD / 64) * kChunk; }
+
+KS_DEV float fast_exp2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+template <int HD>
+__global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_constant__ WideAttnArgs a) {
+    constexpr int CH = HD / 64;              // 64-column chunks of a tile
+    constexpr uint32_t TB = CH * kChunk;     // bytes of one 128-row tile
+    constexpr uint32_t kIdescS = umma_idesc(128, 128, false);
+    constexpr uint32_t kIdescO = umma_idesc(128, HD, true);
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = reinterpret_cast<unsigned char*>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    unsigned char* qs = smem;
+    unsigned char* ring = smem + 2 * TB;
+    __shared__ __align__(8) uint64_t q_full, kv_full[kRing], kv_free[kRing], s_full[2], p_full[2], o_full[2];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int void_job;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int h = (int)blockIdx.x % a.hq, kvh = h / (a.hq / a.hk);
+    const int q0 = (a.blocks - 1 - (int)blockIdx.x / a.hq) * (2 * kQ);   // first row of this CTA
+    // key tiles of each query tile (a tile without rows has none)
+    int nt[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int first = q0 + i * kQ, last = min(a.M, first + kQ) - 1;
+        nt[i] = first < a.M ? (a.p0 + last) / kQ + 1 : 0;
+    }
+    const int n = max(nt[0], nt[1]);
+
+    if (warp == 8) tmem_alloc<1>(&tmem_slot, 512);
+    if (tid == 0) {
+        void_job = __ldcg(a.err) != 0;
+        mbar_init(&q_full, 1);
+        for (int i = 0; i < kRing; ++i) {
+            mbar_init(&kv_full[i], 1);
+            mbar_init(&kv_free[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&s_full[i], 1);
+            mbar_init(&p_full[i], 4);
+            mbar_init(&o_full[i], 1);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    umma_fence_before();
+    __syncthreads();
+    umma_fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    if (!void_job) {
+        if (warp == 9) {
+            // ---------------------------------------------------------- loads
+            if (lane == 0) {
+                bool ok = true;
+                mbar_expect_tx(&q_full, 2 * TB);
+                for (int i = 0; i < 2; ++i)
+                    for (int c = 0; c < CH; ++c)
+                        tma_2d(qs + i * TB + c * kChunk, &a.qmap, h * HD + 64 * c, q0 + i * kQ, &q_full);
+                int t = 0;
+                for (; t < 2 * n; ++t) {     // K 0, V 0, K 1, V 1, ..
+                    const int st = t % kRing;
+                    if (t >= kRing && !mbar_wait(&kv_free[st], (uint32_t)((t / kRing - 1) & 1), kWaitLimitNs)) {
+                        ok = false;
+                        break;
+                    }
+                    mbar_expect_tx(&kv_full[st], TB);
+                    tma_3d(ring + (size_t)st * TB, &a.kvmap, 0,
+                           ((t & 1) ? a.kv_row_v : a.kv_row_k) + kvh * a.max_seq + (t >> 1) * kQ, 0, &kv_full[st]);
+                }
+                if (!ok) {   // the copies in flight land before the CTA leaves
+                    atomicCAS(a.err, 0, 1);
+                    mbar_wait(&q_full, 0, kWaitLimitNs);
+                    for (int q = max(0, t - kRing); q < t; ++q)
+                        mbar_wait(&kv_full[q % kRing], (uint32_t)((q / kRing) & 1), kWaitLimitNs);
+                }
+            }
+        } else if (warp == 8) {
+            // ----------------------------------------------------------- MMAs
+            if (lane == 0) {
+                bool ok = mbar_wait(&q_full, 0, kWaitLimitNs);
+                auto wait_tile = [&](int t) {
+                    ok = ok && mbar_wait(&kv_full[t % kRing], (uint32_t)((t / kRing) & 1), kWaitLimitNs);
+                    umma_fence_after();
+                };
+                auto scores = [&](int i, int j) {   // S_i = Q_i K_j^T
+                    const uint32_t sa = smem_u32(qs + i * TB), sb = smem_u32(ring + (size_t)((2 * j) % kRing) * TB);
+#pragma unroll
+                    for (int k = 0; k < HD / 16; ++k) {
+                        const uint32_t off = (uint32_t)(k / 4) * kChunk + 32 * (k % 4);
+                        umma_ss<1>(tmem + 128 * i, umma_desc(sa + off, 16, 1024), umma_desc(sb + off, 16, 1024),
+                                   kIdescS, k > 0);
+                    }
+                    umma_commit(&s_full[i]);
+                };
+                wait_tile(0);
+                if (ok) {
+                    for (int i = 0; i < 2; ++i)
+                        if (nt[i] > 0) scores(i, 0);
+                    umma_commit(&kv_free[0]);
+                }
+                for (int j = 0; j < n && ok; ++j) {
+                    wait_tile(2 * j + 1);
+                    if (j + 1 < n) wait_tile(2 * j + 2);
+                    if (!ok) break;
+                    const uint32_t sv = smem_u32(ring + (size_t)((2 * j + 1) % kRing) * TB);
+                    for (int i = 0; i < 2; ++i) {
+                        if (j >= nt[i]) continue;
+                        ok = ok && mbar_wait(&p_full[i], (uint32_t)(j & 1), kWaitLimitNs);
+                        if (!ok) break;
+                        umma_fence_after();
+#pragma unroll
+                        for (int k = 0; k < kQ / 16; ++k)   // 16 keys: 8 P columns, 2 KB of V rows
+                            umma_ts(tmem + 256 + HD * i, tmem + 128 * i + 8 * k,
+                                    umma_desc(sv + 2048 * k, kChunk, 1024), kIdescO, j > 0 || k > 0);
+                        if (j + 1 < nt[i]) scores(i, j + 1);
+                        else umma_commit(&o_full[i]);
+                    }
+                    if (!ok) break;
+                    umma_commit(&kv_free[(2 * j + 1) % kRing]);
+                    if (j + 1 < n) umma_commit(&kv_free[(2 * j + 2) % kRing]);
+                }
+                if (!ok) atomicCAS(a.err, 0, 1);
+            }
+        } else {
+            // -------------------------------------------------------- softmax
+            const int i = warp >> 2, quad = warp & 3;
+            const int row = q0 + i * kQ + 32 * quad + lane;
+            const int pos = a.p0 + row;
+            const uint32_t lanes = tmem + ((uint32_t)(32 * quad) << 16);
+            const uint32_t s_at = lanes + 128 * i, o_at = lanes + 256 + HD * i;
+            float m = -INFINITY, l = 0.f;
+            bool ok = true;
+            for (int j = 0; j < nt[i]; ++j) {
+                ok = mbar_wait(&s_full[i], (uint32_t)(j & 1), kWaitLimitNs);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    ok = false;
+                    break;
+                }
+                umma_fence_after();
+                uint32_t s[4][32];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) tmem_ld32(s[c], s_at + 32 * c);
+                tmem_wait_ld();
+#pragma unroll
+                for (int c = 0; c < 4; ++c) tmem_pin(s[c]);
+                if (kQ * (j + 1) > a.p0 + q0 + i * kQ + 1) {   // some key of the tile lies past the tile's first row
+                    const int seen = pos - kQ * j;             // keys 0 .. seen of the tile
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int q = 0; q < 32; ++q)
+                            if (32 * c + q > seen) s[c][q] = 0xff800000u;   // -inf
+                }
+                float mx[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    mx[c] = __uint_as_float(s[c][0]);
+#pragma unroll
+                    for (int q = 1; q < 32; ++q) mx[c] = fmaxf(mx[c], __uint_as_float(s[c][q]));
+                }
+                const float mnew = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+                if (j == 0) {
+                    m = mnew;    // key 0 is seen by every row
+                } else if (__any_sync(0xffffffffu, mnew > m + kRescale)) {
+                    // only rows that grew change: a row never depends on its neighbours
+                    const float mm = mnew > m + kRescale ? mnew : m, alpha = fast_exp2(m - mm);
+                    m = mm;
+                    l *= alpha;
+#pragma unroll 1
+                    for (int c = 0; c < HD; c += 32) {
+                        uint32_t o[32];
+                        tmem_ld32(o, o_at + c);
+                        tmem_wait_ld();
+                        tmem_pin(o);
+#pragma unroll
+                        for (int q = 0; q < 32; ++q) o[q] = __float_as_uint(__uint_as_float(o[q]) * alpha);
+                        tmem_st32(o_at + c, o);
+                    }
+                }
+                float sum[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    sum[c] = 0.f;
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) {
+                        const float p = fast_exp2(__uint_as_float(s[c][q]) - m);
+                        sum[c] += p;
+                        s[c][q] = __float_as_uint(p);
+                    }
+                }
+                l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {   // bf16 pairs: P columns 32 c .. 32 c + 31
+                    uint32_t pk[32];
+#pragma unroll
+                    for (int q = 0; q < 32; ++q)
+                        pk[q] = pack_bf16(__uint_as_float(s[2 * c + q / 16][2 * (q % 16)]),
+                                          __uint_as_float(s[2 * c + q / 16][2 * (q % 16) + 1]));
+                    tmem_st32(s_at + 32 * c, pk);
+                }
+                tmem_wait_st();
+                umma_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&p_full[i]);
+            }
+            if (ok && nt[i] > 0) {
+                ok = mbar_wait(&o_full[i], 0, kWaitLimitNs);
+                ok = __all_sync(0xffffffffu, ok);
+                if (ok) {
+                    umma_fence_after();
+                    const float inv = 1.f / l;
+                    __nv_bfloat16* dst = a.out + (size_t)row * a.hq * HD + h * HD;
+#pragma unroll 1
+                    for (int c = 0; c < HD; c += 32) {
+                        uint32_t o[32];
+                        tmem_ld32(o, o_at + c);
+                        tmem_wait_ld();
+                        tmem_pin(o);
+                        if (row < a.M) {
+#pragma unroll
+                            for (int q = 0; q < 32; q += 8) {
+                                uint32_t w[4];
+#pragma unroll
+                                for (int e = 0; e < 4; ++e)
+                                    w[e] = pack_bf16(__uint_as_float(o[q + 2 * e]) * inv,
+                                                     __uint_as_float(o[q + 2 * e + 1]) * inv);
+                                *reinterpret_cast<uint4*>(dst + c + q) = make_uint4(w[0], w[1], w[2], w[3]);
+                            }
+                        }
+                        __syncwarp();
+                    }
+                }
+            }
+            if (!ok && lane == 0) atomicCAS(a.err, 0, 1);
+        }
+    }
+    umma_fence_before();
+    __syncthreads();
+    if (warp == 8) tmem_free<1>(tmem, 512);
+}
+
+}  // namespace
+
+cudaError_t launch_wide_attention(int hd, const WideAttnArgs& args, cudaStream_t s) {
+    if (args.M < 1 || args.p0 < 0 || args.err == nullptr || args.hq % args.hk) return cudaErrorInvalidValue;
+    WideAttnArgs a = args;
+    a.blocks = (a.M + 2 * kQ - 1) / (2 * kQ);
+    auto run = [&](auto kern, size_t smem) -> cudaError_t {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<a.hq * a.blocks, kThreads, smem, s>>>(a);
+        return cudaGetLastError();
+    };
+    if (hd == 128) return run(wide_attn_kernel<128>, wide_attn_smem<128>());
+    if (hd == 64) return run(wide_attn_kernel<64>, wide_attn_smem<64>());
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace ks
