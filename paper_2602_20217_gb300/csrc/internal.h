@@ -136,6 +136,8 @@ struct WideArgs {
 };
 int wide_tiles_n(int kind, int N);
 cudaError_t launch_wide(int kind, int hd, const WideArgs& a, cudaStream_t s);
+// tokens[m] = the argmax that key best[m] stands for (0 for no key)
+cudaError_t launch_wide_tokens(const unsigned long long* best, int M, int32_t* tokens, cudaStream_t s);
 cudaError_t launch_wide_embed(const __nv_bfloat16* embed, const int32_t* tok, int M, int d, int vocab, float* x,
                               __nv_bfloat16* xg, const __nv_bfloat16* gain, float* ss, int ss_n, int ss_ld,
                               cudaStream_t s);

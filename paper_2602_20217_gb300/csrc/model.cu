@@ -143,15 +143,24 @@ __global__ void __launch_bounds__(kTop1Threads) top1_kernel(const float* logits,
     *ticket = 0;
 }
 
+// Sum of squares of the block's 256 features as one slot of a wide pass.
+KS_DEV void wide_ss(float v, float* ss, int ss_ld, int row) {
+    __shared__ float red[9];
+    const float s = block_sum<8>(v * v, red);
+    if (threadIdx.x == 0) ss[(size_t)blockIdx.y * ss_ld + row] = s;
+}
+
 // TPT stage, Eq. 4 inputs: row b of a batch is overall row q = row0 + b, i.e.
 // candidate j = q / r (j == K: the full layer set) on history row i = q % r.
 // Its draft state is X^(2L) minus X^(s) - X^(s-1) for every sublayer s the
 // candidate skips, in order s = 1 .. 2L; written as the LM head's input: the
-// fp32 residual, its bf16 x * final gain, and the 16-feature sums of squares.
+// fp32 residual, its bf16 x * final gain, and the 16-feature sums of squares;
+// for a wide LM head (ss_ld > 0) x is not needed and the sums are the wide
+// pass's, one slot per 256 features.
 template <typename WT>
 __global__ void __launch_bounds__(256) tpt_states_kernel(const float* hist, long long plane, const int32_t* hidx,
                                                          int r, int row0, int nsub, const uint8_t* masks, int K,
-                                                         int d, const WT* gain, float* x, float* ss,
+                                                         int d, const WT* gain, float* x, float* ss, int ss_ld,
                                                          __nv_bfloat16* xg) {
     const int b = blockIdx.x;
     const int q = row0 + b;
@@ -165,8 +174,12 @@ __global__ void __launch_bounds__(256) tpt_states_kernel(const float* hist, long
         if (mask)
             for (int sl = 1; sl <= nsub; ++sl)
                 if (!mask[sl - 1]) h -= base[(size_t)sl * plane] - base[(size_t)(sl - 1) * plane];
-        x[(size_t)b * d + k] = h;
+        if (x) x[(size_t)b * d + k] = h;
         if (xg) xg[(size_t)b * d + k] = __float2bfloat16_rn(h * to_float(gain[k]));
+    }
+    if (ss_ld > 0) {
+        wide_ss(h, ss, ss_ld, b);
+        return;
     }
     float sq = h * h;   // lanes 0-15 and 16-31 of each warp form one 16-feature group
 #pragma unroll
@@ -396,7 +409,7 @@ struct ks_model {
     std::vector<CUtensorMap> map_qkv, map_o, map_gu, map_down;
     // wide path: operand maps of the weights, of the chunk's inputs and of the cache
     std::vector<CUtensorMap> wide_qkv, wide_o, wide_gu, wide_down;
-    CUtensorMap wide_xg, wide_q, wide_ao, wide_act, wide_kv;
+    CUtensorMap wide_lm, wide_xg, wide_q, wide_ao, wide_act, wide_kv;
     CUtensorMap map_lm, map_xg[16], map_xg2[16], map_attn_out[16], map_act[16];  // [R - 1]: boxes of R rows
     KlassTiming timing[kKlasses];
 };
@@ -960,6 +973,7 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
             ok = ok && make_wide_map(&m->wide_gu[l], m->w_gate_up[l], 2 * (uint64_t)F, d);
             ok = ok && make_wide_map(&m->wide_down[l], m->w_down[l], d, F);
         }
+        ok = ok && make_wide_map(&m->wide_lm, m->lm_head, cfg->vocab, d);
         const WideLayout W = wide_layout(cfg, lay.wide_rows, lay.wide);
         ok = ok && make_wide_map(&m->wide_xg, b + W.xg, lay.wide_rows, d);
         ok = ok && make_wide_map(&m->wide_q, b + W.q, lay.wide_rows, hqd);
@@ -1497,6 +1511,51 @@ static ks_status lm_head_rows(ks_model* m, int R, int32_t* tokens) {
     return launch(m, K_LMHEAD, [&] { return launch_gemv(m->dtype, EPI_LMHEAD, g, s); }, "tpt lm-head");
 }
 
+// LM head argmax of many rows (bf16 models): buffers in the space of the
+// attention partials and logits, which no pass is using then.
+struct WideHead {
+    __nv_bfloat16* xg;            // [rows][d] x * final gain
+    float* ss;                    // [slots][rows] sums of squares
+    unsigned long long* best;     // [rows]
+    int rows;                     // room
+};
+static WideHead wide_head(ks_model* m) {
+    const size_t d = m->cfg.d_model, slots = wide_tiles_n(WK_RESID, m->cfg.d_model);
+    const size_t room = m->lay.hist - m->lay.wide;
+    WideHead H{};
+    H.rows = (int)std::min<size_t>((room - 1024) / (2 * d + 4 * slots + 8) / 8 * 8, 4096);
+    char* b = m->ws + m->lay.wide;
+    H.best = reinterpret_cast<unsigned long long*>(b);
+    b += align_up(8 * (size_t)H.rows, 256);
+    H.ss = reinterpret_cast<float*>(b);
+    b += align_up(4 * slots * H.rows, 256);
+    H.xg = reinterpret_cast<__nv_bfloat16*>(b);
+    return H;
+}
+// rows <= H.rows, xg and ss in place; the tokens go to tokens[0..rows).
+static ks_status wide_head_rows(ks_model* m, const WideHead& H, int rows, int32_t* tokens) {
+    const ks_config& c = m->cfg;
+    WideArgs g{};
+    if (!make_wide_map(&g.amap, H.xg, rows, c.d_model)) {
+        set_error("lm-head: TMA descriptor encoding failed");
+        return KS_ERR_CUDA;
+    }
+    g.wmap = m->wide_lm;
+    g.M = rows;
+    g.N = c.vocab;
+    g.K = g.d = c.d_model;
+    g.eps = c.rms_eps;
+    g.ss_in = H.ss;
+    g.ss_n = wide_tiles_n(WK_RESID, c.d_model);
+    g.ss_ld = H.rows;
+    g.best = H.best;
+    g.err = m->err;
+    KS_CUDA(cudaMemsetAsync(H.best, 0, sizeof(unsigned long long) * rows, m->stream), "lm-head keys");
+    KS_TRY(launch(m, K_LMHEAD, [&] { return launch_wide(WK_ARGMAX, c.head_dim, g, m->stream); }, "wide lm-head",
+                  2.0 * c.vocab * (double)c.d_model));
+    return launch(m, K_ACCEPT, [&] { return launch_wide_tokens(H.best, rows, tokens, m->stream); }, "lm-head tokens");
+}
+
 static ks_status history_sims(ks_model* m, int* rows_out);
 
 // The TPT stage on the device (results stay in tpt_* and mask_dev).
@@ -1514,17 +1573,33 @@ static ks_status tpt_stage(ks_model* m, const ks_latency* lat, int K, int D, int
     const int total = (K + 1) * r;
     const int64_t plane = (int64_t)m->lay.hist_slots * c.max_rows * d;
     const bool bf = m->dtype == KS_DTYPE_BF16;
-    for (int row0 = 0; row0 < total; row0 += c.max_rows) {
+    int done = 0;
+    // More rows than one pass of the decode kernel takes: the LM head reads
+    // its weights once for all of them instead of once per max_rows.
+    if (bf && total > c.max_rows) {
+        const WideHead H = wide_head(m);
+        for (; H.rows > c.max_rows && done < total; done += std::min(H.rows, total - done)) {
+            const int B = std::min(H.rows, total - done);
+            KS_TRY(launch(m, K_EMBED, [&]() -> cudaError_t {
+                tpt_states_kernel<__nv_bfloat16><<<dim3(B, (d + 255) / 256), 256, 0, m->stream>>>(
+                    hist_plane(m, 0), plane, m->hist_idx, r, done, nsub, m->tpt_masks, K, d,
+                    reinterpret_cast<const __nv_bfloat16*>(m->final_norm), nullptr, H.ss, H.rows, H.xg);
+                return cudaGetLastError();
+            }, "tpt states"));
+            KS_TRY(wide_head_rows(m, H, B, m->tpt_tok + done));
+        }
+    }
+    for (int row0 = done; row0 < total; row0 += c.max_rows) {
         const int B = std::min(c.max_rows, total - row0);
         KS_TRY(launch(m, K_EMBED, [&]() -> cudaError_t {
             if (bf)
                 tpt_states_kernel<__nv_bfloat16><<<dim3(B, (d + 255) / 256), 256, 0, m->stream>>>(
                     hist_plane(m, 0), plane, m->hist_idx, r, row0, nsub, m->tpt_masks, K, d,
-                    reinterpret_cast<const __nv_bfloat16*>(m->final_norm), m->x, m->ss, m->xg);
+                    reinterpret_cast<const __nv_bfloat16*>(m->final_norm), m->x, m->ss, 0, m->xg);
             else
                 tpt_states_kernel<float><<<dim3(B, (d + 255) / 256), 256, 0, m->stream>>>(
                     hist_plane(m, 0), plane, m->hist_idx, r, row0, nsub, m->tpt_masks, K, d,
-                    reinterpret_cast<const float*>(m->final_norm), m->x, m->ss, nullptr);
+                    reinterpret_cast<const float*>(m->final_norm), m->x, m->ss, 0, nullptr);
             return cudaGetLastError();
         }, "tpt states"));
         KS_TRY(lm_head_rows(m, B, m->tpt_tok + row0));

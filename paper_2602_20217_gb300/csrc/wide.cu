@@ -29,7 +29,8 @@
 //   WK_SWIGLU  silu(gate) * up: the pair's first CTA stages gate rows, the
 //              second the up rows of the same features;
 //   WK_ARGMAX  the row's best (logit, id) as a 64-bit key, merged by atomicMax
-//              (any order gives the same argmax).
+//              (any order gives the same argmax): the LM head of the layer
+//              selection's candidate states, whose logits nobody reads.
 // Every wait is bounded; a wait that gives up sets the status word and the
 // CTA leaves after its copies have landed.
 #include "common.cuh"
@@ -397,7 +398,19 @@ __global__ void __launch_bounds__(256) wide_embed_kernel(const __nv_bfloat16* em
     if ((int)threadIdx.x < ss_n) ss[(size_t)threadIdx.x * ss_ld + m] = threadIdx.x == 0 ? s : 0.f;
 }
 
+__global__ void __launch_bounds__(256) wide_tokens_kernel(const unsigned long long* best, int M, int32_t* tokens) {
+    const int m = blockIdx.x * 256 + threadIdx.x;
+    if (m >= M) return;
+    const unsigned long long key = best[m];
+    tokens[m] = key == 0ull ? 0 : (int)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull));
+}
+
 }  // namespace
+
+cudaError_t launch_wide_tokens(const unsigned long long* best, int M, int32_t* tokens, cudaStream_t s) {
+    wide_tokens_kernel<<<(M + 255) / 256, 256, 0, s>>>(best, M, tokens);
+    return cudaGetLastError();
+}
 
 int wide_tiles_n(int kind, int N) { return kind == WK_SWIGLU ? (N + 127) / 128 : (N + kTileN - 1) / kTileN; }
 
