@@ -23,31 +23,80 @@ namespace ks {
 
 namespace {
 
-constexpr int kCosThreads = 256;
+constexpr int kCosThreads = 1024;
 
 // mean over the r rows of cos(A_r, B_r); A: a state's contiguous rows, B: the
-// history plane's rows hidx[0..r).  One CTA per state, fixed reduction order.
-__global__ void __launch_bounds__(kCosThreads) dp_cos_kernel(const float* A, long long a_stride, const float* B,
-                                                             const int32_t* hidx, int r, int d, float* sig) {
-    const float* a = A + (size_t)blockIdx.x * a_stride;
-    __shared__ float red[3][kCosThreads / 32 + 1];
+// history plane's rows hidx[0..r).  blockIdx.y picks the execute candidates
+// (0) or the previous states (1).  One CTA per state, a row per warp (32 rows
+// in flight; with a whole CTA and three block sums per row this took 177 us
+// for 13 states of 28 rows of 4096), the row terms added in row order.
+__global__ void __launch_bounds__(kCosThreads) dp_cos_kernel(const float* A0, const float* A1, long long a_stride,
+                                                             const float* B, const int32_t* hidx, int r, int d,
+                                                             float* sig0, float* sig1) {
+    const float* a = (blockIdx.y ? A1 : A0) + (size_t)blockIdx.x * a_stride;
+    float* sig = blockIdx.y ? sig1 : sig0;
+    __shared__ float term[kCosThreads / 32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float acc = 0.f;
-    for (int row = 0; row < r; ++row) {
-        const float* x = a + (size_t)row * d;
-        const float* y = B + (size_t)hidx[row] * d;
-        float xy = 0.f, xx = 0.f, yy = 0.f;
-        for (int k = threadIdx.x; k < d; k += kCosThreads) {
-            const float u = x[k], v = y[k];
-            xy = fmaf(u, v, xy);
-            xx = fmaf(u, u, xx);
-            yy = fmaf(v, v, yy);
+    for (int r0 = 0; r0 < r; r0 += kCosThreads / 32) {
+        const int row = r0 + warp;
+        if (row < r) {
+            const float4* x = reinterpret_cast<const float4*>(a + (size_t)row * d);
+            const float4* y = reinterpret_cast<const float4*>(B + (size_t)hidx[row] * d);
+            float xy = 0.f, xx = 0.f, yy = 0.f;
+#pragma unroll 4
+            for (int k = lane; k < d / 4; k += 32) {   // d is a multiple of 8
+                const float4 u = x[k], v = y[k];
+                xy = fmaf(u.x, v.x, fmaf(u.y, v.y, fmaf(u.z, v.z, fmaf(u.w, v.w, xy))));
+                xx = fmaf(u.x, u.x, fmaf(u.y, u.y, fmaf(u.z, u.z, fmaf(u.w, u.w, xx))));
+                yy = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, yy))));
+            }
+            xy = warp_sum(xy);
+            xx = warp_sum(xx);
+            yy = warp_sum(yy);
+            if (lane == 0) term[warp] = xy / (sqrtf(xx) * sqrtf(yy));
         }
-        xy = block_sum<kCosThreads / 32>(xy, red[0]);
-        xx = block_sum<kCosThreads / 32>(xx, red[1]);
-        yy = block_sum<kCosThreads / 32>(yy, red[2]);
-        acc += xy / (sqrtf(xx) * sqrtf(yy));
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int i = 0; i < min(kCosThreads / 32, r - r0); ++i) acc += term[i];
+        __syncthreads();
     }
     if (threadIdx.x == 0) sig[blockIdx.x] = acc / (float)r;
+}
+
+// Input of a wide pass: row q of `rows`, features 256 y .. (blockIdx.y).
+KS_DEV void wide_row(float v, int q, int k, int d, const __nv_bfloat16* gain, __nv_bfloat16* xg, float* ss, int ss_ld) {
+    __shared__ float red[9];
+    if (k < d) xg[(size_t)q * d + k] = __float2bfloat16_rn(v * __bfloat162float(gain[k]));
+    const float s = block_sum<8>(v * v, red);
+    if (threadIdx.x == 0) ss[(size_t)blockIdx.y * ss_ld + q] = s;
+}
+
+// grid (n r, ceil(d / 256)): row q belongs to state j0 + q / r.  Invalid
+// states become zeros: their values are never used, but they share key tiles
+// with the others, where 0 * NaN would not vanish.
+__global__ void __launch_bounds__(256) dp_prep_kernel(const float* G, int j0, const int* valid, int r, int d,
+                                                      const __nv_bfloat16* gain, float* E, __nv_bfloat16* xg,
+                                                      float* ss, int ss_ld) {
+    const int q = blockIdx.x, k = blockIdx.y * 256 + threadIdx.x;
+    const size_t at = ((size_t)j0 * r + q) * d + k;
+    const bool ok = valid[j0 + q / r] == 0;
+    float v = 0.f;
+    if (k < d) {
+        if (ok) v = G[at];
+        E[at] = v;
+    }
+    wide_row(v, q, k, d, gain, xg, ss, ss_ld);
+}
+
+__global__ void __launch_bounds__(256) dp_head_kernel(const float* G, const int* js, int n_cand, int row0, int r,
+                                                      int d, const __nv_bfloat16* gain, __nv_bfloat16* xg, float* ss,
+                                                      int ss_ld) {
+    const int q = blockIdx.x, k = blockIdx.y * 256 + threadIdx.x;
+    const int c = (row0 + q) / r, i = row0 + q - c * r;
+    const int j = c < n_cand ? js[c] : 0;
+    const float v = k < d ? G[((size_t)j * r + i) * d + k] : 0.f;
+    wide_row(v, q, k, d, gain, xg, ss, ss_ld);
 }
 
 // One thread per skipped weight j.  valid_*: 0 valid, 1 invalid (the value
@@ -80,23 +129,19 @@ __global__ void dp_select_kernel(int J, int w, float tau, const int* valid_prev,
     src[j] = s;
 }
 
-// grid (J, ceil(d / 256)): row block of state j from its source
+// grid (J, r): one row of state j from its source
 __global__ void __launch_bounds__(256) dp_gather_kernel(const int* src, const int* valid_cur, const float* E,
                                                         const float* G_prev, long long stride, const float* X,
                                                         const int32_t* hidx, int r, int d, float* G_cur) {
     const int j = blockIdx.x;
     if (valid_cur[j]) return;
-    const int k = blockIdx.y * 256 + threadIdx.x;
-    if (k >= d) return;
+    const int row = blockIdx.y;
     const int s = src[j];
-    float* out = G_cur + (size_t)j * stride;
-    for (int row = 0; row < r; ++row) {
-        float v;
-        if (s < 0) v = X[(size_t)hidx[row] * d + k];
-        else if (s & 1) v = G_prev[(size_t)(s >> 1) * stride + (size_t)row * d + k];
-        else v = E[(size_t)(s >> 1) * stride + (size_t)row * d + k];
-        out[(size_t)row * d + k] = v;
-    }
+    const float* in = s < 0 ? X + (size_t)hidx[row] * d
+                            : (s & 1 ? G_prev : E) + (size_t)(s >> 1) * stride + (size_t)row * d;
+    const float4* from = reinterpret_cast<const float4*>(in);
+    float4* out = reinterpret_cast<float4*>(G_cur + (size_t)j * stride + (size_t)row * d);
+    for (int k = threadIdx.x; k < d / 4; k += 256) out[k] = from[k];   // d is a multiple of 8
 }
 
 // one thread per candidate: candidate c is terminal state js[c]
@@ -128,10 +173,22 @@ __global__ void dp_candidates_kernel(int J, const int* valid, int* js, int* n_ca
 
 }  // namespace
 
-cudaError_t launch_dp_cos(const float* A, long long stride, int n, const float* B, const int32_t* hidx, int r, int d,
-                          float* sig, cudaStream_t s) {
+cudaError_t launch_dp_cos(const float* A0, const float* A1, long long stride, int n, const float* B,
+                          const int32_t* hidx, int r, int d, float* sig0, float* sig1, cudaStream_t s) {
     if (n < 1) return cudaSuccess;
-    dp_cos_kernel<<<n, kCosThreads, 0, s>>>(A, stride, B, hidx, r, d, sig);
+    dp_cos_kernel<<<dim3(n, 2), kCosThreads, 0, s>>>(A0, A1, stride, B, hidx, r, d, sig0, sig1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_dp_prep(const float* G, int j0, int n, const int* valid, int r, int d, const __nv_bfloat16* gain,
+                           float* E, __nv_bfloat16* xg, float* ss, int ss_ld, cudaStream_t s) {
+    dp_prep_kernel<<<dim3(n * r, (d + 255) / 256), 256, 0, s>>>(G, j0, valid, r, d, gain, E, xg, ss, ss_ld);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_dp_head(const float* G, const int* js, int n_cand, int row0, int rows, int r, int d,
+                           const __nv_bfloat16* gain, __nv_bfloat16* xg, float* ss, int ss_ld, cudaStream_t s) {
+    dp_head_kernel<<<dim3(rows, (d + 255) / 256), 256, 0, s>>>(G, js, n_cand, row0, r, d, gain, xg, ss, ss_ld);
     return cudaGetLastError();
 }
 
@@ -145,7 +202,7 @@ cudaError_t launch_dp_select(int J, int w, float tau, const int* valid_prev, con
 cudaError_t launch_dp_gather(int J, const int* src, const int* valid_cur, const float* E, const float* G_prev,
                              long long stride, const float* X, const int32_t* hidx, int r, int d, float* G_cur,
                              cudaStream_t s) {
-    dp_gather_kernel<<<dim3(J, (d + 255) / 256), 256, 0, s>>>(src, valid_cur, E, G_prev, stride, X, hidx, r, d,
+    dp_gather_kernel<<<dim3(J, r), 256, 0, s>>>(src, valid_cur, E, G_prev, stride, X, hidx, r, d,
                                                               G_cur);
     return cudaGetLastError();
 }

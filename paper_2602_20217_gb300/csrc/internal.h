@@ -117,6 +117,9 @@ struct WideArgs {
     CUtensorMap amap, wmap;     // make_wide_map of the input rows and of the weights
     int M, N, K;                // rows, output features (WK_SWIGLU: d_ff), inputs
     int tiles_m, tiles_n;       // set by launch_wide
+    int slices;                 // set by launch_wide: K-slices of a tile
+    float* part;                // kWidePartFloats partial sums of K-sliced tiles
+    int* ticket;                // kWideTickets arrivals, zero between launches
     int d;                      // model width (the norm's)
     float eps;
     const float* ss_in;         // [ss_n][ss_ld] sums of squares of the input rows (all kinds but WK_RESID)
@@ -130,10 +133,17 @@ struct WideArgs {
     __nv_bfloat16 *kcache, *vcache;   // WK_QKV: this layer's [hk][max_seq][hd]
     const float* rope;
     const __nv_bfloat16 *q_norm, *k_norm;
-    int hq, hk, max_seq, p0;    // WK_QKV: row m is at position p0 + m
+    int hq, hk, max_seq, p0;    // WK_QKV: row m is at position p0 + m and in cache row p0 + m
+    int state_rows;             // > 0: independent states of that many rows, row m at position p0 + m % state_rows;
+                                // kcache / vcache hold the rows' own K/V, [hk][max_seq][hd] with row m
     unsigned long long* best;   // WK_ARGMAX: [M] keys, merged by atomicMax
     int* err;                   // device status word
 };
+// K-sliced launches have at most kWideUnits (tile, slice) units, one per CTA
+// pair: 256 x 256 partial sums each, and 8 row groups of 32 per tile.
+constexpr int kWideUnits = 76;
+constexpr size_t kWidePartFloats = (size_t)kWideUnits * 256 * 256;
+constexpr int kWideTickets = kWideUnits * 8;
 int wide_tiles_n(int kind, int N);
 cudaError_t launch_wide(int kind, int hd, const WideArgs& a, cudaStream_t s);
 // tokens[m] = the argmax that key best[m] stands for (0 for no key)
@@ -142,11 +152,15 @@ cudaError_t launch_wide_embed(const __nv_bfloat16* embed, const int32_t* tok, in
                               __nv_bfloat16* xg, const __nv_bfloat16* gain, float* ss, int ss_n, int ss_ld,
                               cudaStream_t s);
 // Causal attention of M rows at positions p0 .. over the cache (wide_attn.cu).
+// state_rows > 0: the rows are independent states of state_rows rows; each row
+// sees the cache below p0 and its own state's rows up to itself.
 struct WideAttnArgs {
     CUtensorMap qmap;           // make_wide_map of q [rows][hq hd]
     CUtensorMap kvmap;          // make_wide_kv_map of the whole cache
+    CUtensorMap kxmap, vxmap;   // states: make_wide_kv_map of the rows' own K and V, [hk][own_ld] rows
     int kv_row_k, kv_row_v;     // first cache row of this layer's K and V
     int M, p0, hq, hk, max_seq;
+    int state_rows, own_ld;
     int blocks;                 // set by launch_wide_attention
     __nv_bfloat16* out;         // [M][hq hd]
     int* err;
@@ -245,8 +259,15 @@ cudaError_t launch_spec_accept(const AcceptSampleArgs& a, cudaStream_t s);
 
 // ------------------------------------------------ hidden-state DP (dp.cu)
 constexpr int kDpMaxStates = 128;   // skipped weights 0 .. 127 (the TPT grid kernel's candidate limit)
-cudaError_t launch_dp_cos(const float* A, long long stride, int n, const float* B, const int32_t* hidx, int r, int d,
-                          float* sig, cudaStream_t s);
+cudaError_t launch_dp_cos(const float* A0, const float* A1, long long stride, int n, const float* B,
+                          const int32_t* hidx, int r, int d, float* sig0, float* sig1, cudaStream_t s);
+// E, xg and ss (wide pass layout) of the rows of n states from j0: a copy of the
+// state, its bf16 x * gain and sums of squares; invalid states give zeros.
+cudaError_t launch_dp_prep(const float* G, int j0, int n, const int* valid, int r, int d, const __nv_bfloat16* gain,
+                           float* E, __nv_bfloat16* xg, float* ss, int ss_ld, cudaStream_t s);
+// The same LM head input for rows row0 .. row0 + rows of the candidates js[] (state 0 after the last).
+cudaError_t launch_dp_head(const float* G, const int* js, int n_cand, int row0, int rows, int r, int d,
+                           const __nv_bfloat16* gain, __nv_bfloat16* xg, float* ss, int ss_ld, cudaStream_t s);
 cudaError_t launch_dp_select(int J, int w, float tau, const int* valid_prev, const float* sig_e, const float* sig_s,
                              int* valid_cur, float* sig_cur, uint8_t* choice, int* src, cudaStream_t s);
 cudaError_t launch_dp_gather(int J, const int* src, const int* valid_cur, const float* E, const float* G_prev,

@@ -194,7 +194,7 @@ static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 struct Layout {
     size_t kv, rope, x, ss, xg, qkv, attn_out, act, attn_part, gemv_part, counters, logits, amax_val,
         amax_idx, tok, hist, hist_snap, hist_idx, sims, mask, obj, wts, select, chain_ctr, best, tpt_masks,
-        tpt_tok, tpt_info, tpt_out, dyn, samp, slice, qbuf, wide, total;
+        tpt_tok, tpt_info, tpt_out, dyn, samp, slice, qbuf, wide, wide_part, wide_ticket, total;
     int wide_rows;   // rows of a wide chunk (0: fp32 models, no wide path)
     int n_chunks_max;
     size_t gemv_part_floats;
@@ -256,6 +256,41 @@ static WideLayout wide_layout(const ks_config* c, int rows, size_t base) {
     return W;
 }
 
+// Buffers of the hidden-state DP's wide sublayer evaluations, from `base`: the
+// rows' input, their own K and V ([hk][rows][hd], which stay finite past the
+// rows in use: key tiles are read whole), and the attention's or the MLP's
+// intermediate rows.  rows is a multiple of the 128-key tiles.
+struct DpWideLayout {
+    size_t xg, ss, kx, vx, q, ao, act, bytes;
+};
+static DpWideLayout dp_wide_layout(const ks_config* c, int rows, size_t base) {
+    const size_t M = rows, d = c->d_model, hqd = (size_t)c->n_q_heads * c->head_dim;
+    size_t off = base;
+    auto take = [&](size_t bytes) {
+        const size_t o = off;
+        off = align_up(off + bytes, 256);
+        return o;
+    };
+    DpWideLayout W{};
+    W.xg = take(sizeof(__nv_bfloat16) * M * d);
+    W.ss = take(sizeof(float) * M * wide_tiles_n(WK_RESID, c->d_model));
+    W.kx = take(sizeof(__nv_bfloat16) * M * c->n_kv_heads * c->head_dim);
+    W.vx = take(sizeof(__nv_bfloat16) * M * c->n_kv_heads * c->head_dim);
+    W.q = W.act = off;
+    W.ao = W.q + align_up(sizeof(__nv_bfloat16) * M * hqd, 256);
+    off = std::max(W.ao + align_up(sizeof(__nv_bfloat16) * M * hqd, 256),
+                   W.act + align_up(sizeof(__nv_bfloat16) * M * c->d_ff, 256));
+    W.bytes = off - base;
+    return W;
+}
+constexpr int kDpWideRows = 512;   // rows there is always room for
+// the largest row count that fits `bytes`
+static int dp_wide_rows(const ks_config* c, size_t bytes) {
+    int rows = 0;
+    while (rows < 4096 && dp_wide_layout(c, rows + 128, 0).bytes <= bytes) rows += 128;
+    return rows;
+}
+
 static Layout make_layout(const ks_config* c) {
     Layout L{};
     const size_t es = c->dtype == KS_DTYPE_BF16 ? 2 : 4;
@@ -304,6 +339,7 @@ static Layout make_layout(const ks_config* c) {
     L.wide = off;
     L.attn_part = take(sizeof(float) * (size_t)R * c->n_q_heads * L.n_chunks_max * (hd + 4));
     L.logits = take(sizeof(float) * (size_t)R * c->vocab);
+    if (L.wide_rows) off = std::max(off, L.wide + dp_wide_layout(c, kDpWideRows, 0).bytes);   // the DP's, beside the history
     L.hist = take(sizeof(float) * (size_t)(nsub + 1) * L.hist_slots * R * d);
     L.hist_snap = take(sizeof(float) * (size_t)(nsub + 1) * R * d);  // the prefill's history entry
     off = std::max(off, L.wide + wide_layout(c, L.wide_rows, 0).bytes);
@@ -330,6 +366,9 @@ static Layout make_layout(const ks_config* c) {
     L.slice = take(sizeof(float) * 2 * kChainSliceMaxItems * 512 + sizeof(int) * 2 * kChainSliceMaxItems);
     // bf16 attention: the pass's prepared queries [hk][G R][hd]
     L.qbuf = take(sizeof(__nv_bfloat16) * (size_t)R * c->n_q_heads * hd);
+    // wide path: partial sums of K-sliced tiles and their arrivals (zero between launches)
+    L.wide_part = take(L.wide_rows ? sizeof(float) * kWidePartFloats : 0);
+    L.wide_ticket = take(sizeof(int) * kWideTickets);
     L.total = off;
     return L;
 }
@@ -738,6 +777,8 @@ static ks_status wide_forward(ks_model* m, const int32_t* tok, int M, int p0) {
     g.max_seq = c.max_seq;
     g.p0 = p0;
     g.err = m->err;
+    g.part = reinterpret_cast<float*>(m->ws + m->lay.wide_part);
+    g.ticket = reinterpret_cast<int*>(m->ws + m->lay.wide_ticket);
     KS_TRY(launch(m, K_EMBED, [&] {
         return launch_wide_embed(bf(m->embed), tok, M, d, c.vocab, g.x, g.xg, bf(m->attn_norm[0]), g.ss_out, g.ss_n,
                                  g.ss_ld, s);
@@ -1034,6 +1075,8 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
     if (e != cudaSuccess) return fail(e, "token reset");
     e = cudaMemsetAsync(m->slice_ticket, 0, sizeof(int) * 2 * kChainSliceMaxItems, m->stream);
     if (e != cudaSuccess) return fail(e, "slice reset");
+    e = cudaMemsetAsync(b + lay.wide_ticket, 0, sizeof(int) * kWideTickets, m->stream);
+    if (e != cudaSuccess) return fail(e, "ticket reset");
     e = cudaMemsetAsync(b + lay.dyn, 0, sizeof(float) * ((size_t)R + kTop1Ctas) + sizeof(int), m->stream);
     if (e != cudaSuccess) return fail(e, "dynamic-exit reset");
     e = cudaStreamSynchronize(m->stream);
@@ -1550,6 +1593,8 @@ static ks_status wide_head_rows(ks_model* m, const WideHead& H, int rows, int32_
     g.ss_ld = H.rows;
     g.best = H.best;
     g.err = m->err;
+    g.part = reinterpret_cast<float*>(m->ws + m->lay.wide_part);
+    g.ticket = reinterpret_cast<int*>(m->ws + m->lay.wide_ticket);
     KS_CUDA(cudaMemsetAsync(H.best, 0, sizeof(unsigned long long) * rows, m->stream), "lm-head keys");
     KS_TRY(launch(m, K_LMHEAD, [&] { return launch_wide(WK_ARGMAX, c.head_dim, g, m->stream); }, "wide lm-head",
                   2.0 * c.vocab * (double)c.d_model));
@@ -1762,6 +1807,86 @@ static void dp_weights(const ks_latency& lat, int64_t n, int nsub, std::vector<i
     for (int i = 0; i < nsub; ++i) w[i] = (i % 2 == 0) ? wa : wm;
 }
 
+// Sublayer i of states 1 .. S - 1 (r rows each at positions p0..) from G to E,
+// every state's rows in one pass per batch of `per` states: the sublayer's
+// weights stream once per batch instead of once per state and max_rows rows.
+// The states' own K/V stay in the pass's buffers; the cache is only read.
+static ks_status dp_wide_sublayer(ks_model* m, int i, int S, int r, int p0, int rows, const float* G, const int* valid,
+                                  float* E, CUtensorMap (&maps)[6]) {
+    const ks_config& c = m->cfg;
+    const int d = c.d_model, F = c.d_ff, hd = c.head_dim, hqd = c.n_q_heads * hd, l = (i - 1) / 2;
+    cudaStream_t s = m->stream;
+    const DpWideLayout W = dp_wide_layout(&c, rows, m->lay.wide);
+    auto bf = [](const void* p) { return reinterpret_cast<const __nv_bfloat16*>(p); };
+    auto at = [&](size_t o) { return reinterpret_cast<__nv_bfloat16*>(m->ws + o); };
+    const bool attn = i % 2 == 1;
+    const int per = rows / r;
+    WideArgs g{};
+    g.d = d;
+    g.eps = c.rms_eps;
+    g.ss_in = g.ss_out = reinterpret_cast<float*>(m->ws + W.ss);
+    g.ss_n = wide_tiles_n(WK_RESID, d);
+    g.ss_ld = rows;
+    g.xg = at(W.xg);
+    g.act = at(W.act);
+    g.q = at(W.q);
+    g.kcache = at(W.kx);
+    g.vcache = at(W.vx);
+    g.rope = m->rope;
+    g.q_norm = c.qk_norm ? bf(m->q_norm[l]) : nullptr;
+    g.k_norm = c.qk_norm ? bf(m->k_norm[l]) : nullptr;
+    g.hq = c.n_q_heads;
+    g.hk = c.n_kv_heads;
+    g.max_seq = rows;
+    g.p0 = p0;
+    g.state_rows = r;
+    g.err = m->err;
+    g.part = reinterpret_cast<float*>(m->ws + m->lay.wide_part);
+    g.ticket = reinterpret_cast<int*>(m->ws + m->lay.wide_ticket);
+    g.gain = bf(attn ? m->attn_norm[l] : m->mlp_norm[l]);   // the residual kind's x * gain is not used
+    auto project = [&](int kind, int klass, const CUtensorMap& in, const CUtensorMap& w, int N, int K) -> ks_status {
+        g.amap = in;
+        g.wmap = w;
+        g.N = N;
+        g.K = K;
+        return launch(m, klass, [&] { return launch_wide(kind, hd, g, s); }, "dp projection",
+                      2.0 * K * (double)(kind == WK_SWIGLU ? 2 * N : N));
+    };
+    for (int j0 = 1; j0 < S; j0 += per) {
+        const int n = std::min(per, S - j0);
+        g.M = n * r;
+        g.x = E + (size_t)j0 * r * d;
+        KS_TRY(launch(m, K_EMBED, [&] {
+            return launch_dp_prep(G, j0, n, valid, r, d, g.gain, E, g.xg, g.ss_out, rows, s);
+        }, "dp states"));
+        if (attn) {
+            KS_TRY(project(WK_QKV, K_QKV, maps[0], m->wide_qkv[l], (c.n_q_heads + 2 * c.n_kv_heads) * hd, d));
+            WideAttnArgs a{};
+            a.qmap = maps[1];
+            a.kvmap = m->wide_kv;
+            a.kxmap = maps[2];
+            a.vxmap = maps[3];
+            a.kv_row_k = 2 * l * c.n_kv_heads * c.max_seq;
+            a.kv_row_v = (2 * l + 1) * c.n_kv_heads * c.max_seq;
+            a.M = g.M;
+            a.p0 = p0;
+            a.hq = c.n_q_heads;
+            a.hk = c.n_kv_heads;
+            a.max_seq = c.max_seq;
+            a.state_rows = r;
+            a.own_ld = rows;
+            a.out = at(W.ao);
+            a.err = m->err;
+            KS_TRY(launch(m, K_ATTN, [&] { return launch_wide_attention(hd, a, s); }, "dp attention"));
+            KS_TRY(project(WK_RESID, K_OPROJ, maps[4], m->wide_o[l], d, hqd));
+        } else {
+            KS_TRY(project(WK_SWIGLU, K_GATEUP, maps[0], m->wide_gu[l], F, d));
+            KS_TRY(project(WK_RESID, K_DOWN, maps[5], m->wide_down[l], d, F));
+        }
+    }
+    return KS_OK;
+}
+
 ks_status ks_select_dp(ks_model* m, const ks_latency* lat, float tau, int32_t max_gamma, int32_t max_states,
                        int32_t max_rows, void* scratch, size_t scratch_bytes, uint8_t* mask_out, int32_t* gamma_out,
                        double* tpt_out, int32_t* n_candidates, int32_t* js_out, double* alphas_out,
@@ -1830,6 +1955,25 @@ ks_status ks_select_dp(ks_model* m, const ks_latency* lat, float tau, int32_t ma
             return launch_dp_gather(S, D.src, vp, D.E, Gp, stride, hist_plane(m, 0), m->hist_idx, r, d, Gp, s);
         }, "dp init"));
     }
+    // bf16 models with more state rows than one decode pass takes: wide passes
+    // over batches of whole states
+    const int wide_rows = m->dtype == KS_DTYPE_BF16 ? dp_wide_rows(&c, m->lay.hist - m->lay.wide) : 0;
+    const bool wide = (S - 1) * r > c.max_rows && wide_rows >= r;
+    CUtensorMap maps[6];
+    if (wide) {
+        const DpWideLayout W = dp_wide_layout(&c, wide_rows, m->lay.wide);
+        const int hqd = c.n_q_heads * c.head_dim;
+        char* b = m->ws;
+        if (!make_wide_map(&maps[0], b + W.xg, wide_rows, d) || !make_wide_map(&maps[1], b + W.q, wide_rows, hqd) ||
+            !make_wide_kv_map(&maps[2], b + W.kx, (uint64_t)c.n_kv_heads * wide_rows, c.head_dim) ||
+            !make_wide_kv_map(&maps[3], b + W.vx, (uint64_t)c.n_kv_heads * wide_rows, c.head_dim) ||
+            !make_wide_map(&maps[4], b + W.ao, wide_rows, hqd) ||
+            !make_wide_map(&maps[5], b + W.act, wide_rows, c.d_ff)) {
+            set_error("ks_select_dp: TMA descriptor encoding failed");
+            return KS_ERR_CUDA;
+        }
+        KS_CUDA(cudaMemsetAsync(b + W.kx, 0, W.q - W.kx, s), "dp kv init");
+    }
     const size_t kv_row = (size_t)c.head_dim * m->es;
     const size_t kv_plane = (size_t)c.n_kv_heads * r * kv_row;
     std::vector<uint8_t> one(nsub, 0);
@@ -1842,13 +1986,14 @@ ks_status ks_select_dp(ks_model* m, const ks_latency* lat, float tau, int32_t ma
         char* vcach = reinterpret_cast<char*>(vcache(m, l));
         char* kvs = reinterpret_cast<char*>(D.kv);
         const size_t seq_pitch = (size_t)c.max_seq * kv_row;
-        if (attn) {   // the target's K/V at the history positions, restored after every state
+        if (wide) KS_TRY(dp_wide_sublayer(m, i, S, r, p0, wide_rows, Gp, vp, D.E, maps));
+        if (attn && !wide) {   // the target's K/V at the history positions, restored after every state
             KS_CUDA(cudaMemcpy2DAsync(kvs, r * kv_row, kc + (size_t)p0 * kv_row, seq_pitch, r * kv_row, c.n_kv_heads,
                                       cudaMemcpyDeviceToDevice, s), "dp kv save");
             KS_CUDA(cudaMemcpy2DAsync(kvs + kv_plane, r * kv_row, vcach + (size_t)p0 * kv_row, seq_pitch, r * kv_row,
                                       c.n_kv_heads, cudaMemcpyDeviceToDevice, s), "dp kv save");
         }
-        for (int j = 1; j < S; ++j) {
+        for (int j = 1; j < S && !wide; ++j) {
             for (int c0 = 0; c0 < r; c0 += c.max_rows) {
                 const int R = std::min(c.max_rows, r - c0);
                 KS_CUDA(cudaMemcpyAsync(m->x, Gp + (size_t)j * stride + (size_t)c0 * d, sizeof(float) * R * d,
@@ -1865,10 +2010,9 @@ ks_status ks_select_dp(ks_model* m, const ks_latency* lat, float tau, int32_t ma
             }
         }
         const float* X = hist_plane(m, i);
-        KS_TRY(launch(m, K_ACCEPT, [&] { return launch_dp_cos(D.E, stride, S, X, m->hist_idx, r, d, D.sig_e, s); },
-                      "dp cosines"));
-        KS_TRY(launch(m, K_ACCEPT, [&] { return launch_dp_cos(Gp, stride, S, X, m->hist_idx, r, d, D.sig_s, s); },
-                      "dp cosines"));
+        KS_TRY(launch(m, K_ACCEPT, [&] {
+            return launch_dp_cos(D.E, Gp, stride, S, X, m->hist_idx, r, d, D.sig_e, D.sig_s, s);
+        }, "dp cosines"));
         KS_TRY(launch(m, K_ACCEPT, [&] {
             return launch_dp_select(S, w[i - 1], tau, vp, D.sig_e, D.sig_s, vc, D.sig, D.choices + (size_t)(i - 1) * S,
                                     D.src, s);
@@ -1896,7 +2040,20 @@ ks_status ks_select_dp(ks_model* m, const ks_latency* lat, float tau, int32_t ma
         return launch_dp_backtrack(D.js, n_cand, nsub, S, D.choices, D.w, D.masks, s);
     }, "dp backtrack"));
     // Eq. 4 inputs: the LM head's argmax of every terminal state's rows and of X^(2L)
-    for (int cnd = 0; cnd <= n_cand; ++cnd) {
+    const int total = (n_cand + 1) * r;
+    int done = 0;
+    if (m->dtype == KS_DTYPE_BF16 && total > c.max_rows) {   // all rows in one wide LM head pass (or few)
+        const WideHead H = wide_head(m);
+        for (; H.rows > c.max_rows && done < total; done += std::min(H.rows, total - done)) {
+            const int rows = std::min(H.rows, total - done);
+            KS_TRY(launch(m, K_EMBED, [&] {
+                return launch_dp_head(Gp, D.js, n_cand, done, rows, r, d,
+                                      reinterpret_cast<const __nv_bfloat16*>(m->final_norm), H.xg, H.ss, H.rows, s);
+            }, "dp prediction rows"));
+            KS_TRY(wide_head_rows(m, H, rows, D.pred + done));
+        }
+    }
+    for (int cnd = 0; cnd <= n_cand && done < total; ++cnd) {
         for (int c0 = 0; c0 < r; c0 += c.max_rows) {
             const int R = std::min(c.max_rows, r - c0);
             if (cnd < n_cand) {

@@ -31,6 +31,11 @@
 //   WK_ARGMAX  the row's best (logit, id) as a 64-bit key, merged by atomicMax
 //              (any order gives the same argmax): the LM head of the layer
 //              selection's candidate states, whose logits nobody reads.
+// When there are at most half as many tiles as pairs (a few hundred rows at
+// d_model features) a tile's K range is cut into slices, one pair each: every
+// slice leaves its sums in global memory, and per group of 32 rows the slice
+// that arrives last (a ticket) adds them in slice order, puts the total back
+// into its TMEM columns and runs the epilogue.  No pair waits for another.
 // Every wait is bounded; a wait that gives up sets the status word and the
 // CTA leaves after its copies have landed.
 #include "common.cuh"
@@ -75,6 +80,65 @@ KS_DEV void load_chunk(uint32_t (&r)[32], uint32_t addr) {
     tmem_pin(r);
 }
 
+// K-sliced tile: this warp's 32 rows x 256 columns go to the slice's slab;
+// true for the slice that arrives last, whose TMEM columns then hold the sum
+// of all slices in slice order.  Slab: [column / 4][row] float4, so that a
+// warp's accesses are whole lines.
+KS_DEV bool merge_slices(const WideArgs& a, uint32_t acc, int tile, int slice, int group) {
+    const int lane = threadIdx.x & 31;
+    const size_t slab = 32 * kTileN;
+    float* base = a.part + ((size_t)tile * a.slices * 8 + group) * slab;   // slice q at + q * 8 slabs
+    float4* mine = reinterpret_cast<float4*>(base + (size_t)slice * 8 * slab);
+#pragma unroll 1
+    for (int c = 0; c < kTileN; c += 32) {
+        uint32_t r[32];
+        load_chunk(r, acc + c);
+#pragma unroll
+        for (int i = 0; i < 32; i += 4)
+            __stcg(&mine[((c + i) / 4) * 32 + lane],
+                   make_float4(__uint_as_float(r[i]), __uint_as_float(r[i + 1]), __uint_as_float(r[i + 2]),
+                               __uint_as_float(r[i + 3])));
+    }
+    __threadfence();
+    __syncwarp();
+    int last = 0;
+    if (lane == 0) {
+        int* tk = a.ticket + tile * 8 + group;
+        last = atomicAdd(tk, 1) == a.slices - 1;
+        if (last) *tk = 0;   // every slice has arrived: zero for the next launch
+    }
+    if (!__shfl_sync(0xffffffffu, last, 0)) return false;
+    __threadfence();
+#pragma unroll 1
+    for (int c = 0; c < kTileN; c += 32) {
+        float4 t[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) t[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int q = 0; q < a.slices; ++q) {
+            const float4* src = reinterpret_cast<const float4*>(base + (size_t)q * 8 * slab);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float4 v = __ldcg(&src[(c / 4 + i) * 32 + lane]);
+                t[i].x += v.x;
+                t[i].y += v.y;
+                t[i].z += v.z;
+                t[i].w += v.w;
+            }
+        }
+        uint32_t r[32];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            r[4 * i] = __float_as_uint(t[i].x);
+            r[4 * i + 1] = __float_as_uint(t[i].y);
+            r[4 * i + 2] = __float_as_uint(t[i].z);
+            r[4 * i + 3] = __float_as_uint(t[i].w);
+        }
+        tmem_st32(acc + c, r);
+    }
+    tmem_wait_st();
+    return true;
+}
+
 // One head (HD columns at `col`) of this thread's row.
 template <int HD>
 KS_DEV void qkv_head(const WideArgs& a, uint32_t acc, int col, int m, int n, float scale, bool live) {
@@ -87,7 +151,8 @@ KS_DEV void qkv_head(const WideArgs& a, uint32_t acc, int col, int m, int n, flo
         for (int i = 0; i < 32; ++i) v[32 * c + i] = __uint_as_float(r[i]) * scale;
     }
     if (!live || n >= a.N) return;
-    const int head = n / HD, pos = a.p0 + m;
+    const int head = n / HD, pos = a.p0 + (a.state_rows > 0 ? m % a.state_rows : m);
+    const int kv_row = a.state_rows > 0 ? m : pos;
     __nv_bfloat16* dst;
     if (head < a.hq + a.hk) {
         const __nv_bfloat16* gain = head < a.hq ? a.q_norm : a.k_norm;
@@ -116,9 +181,9 @@ KS_DEV void qkv_head(const WideArgs& a, uint32_t acc, int col, int m, int n, flo
         for (int i = 0; i < HD; ++i) v[i] *= qs;
         dst = a.q + (size_t)m * a.hq * HD + (size_t)head * HD;
     } else if (head < a.hq + a.hk) {
-        dst = a.kcache + ((size_t)(head - a.hq) * a.max_seq + pos) * HD;
+        dst = a.kcache + ((size_t)(head - a.hq) * a.max_seq + kv_row) * HD;
     } else {
-        dst = a.vcache + ((size_t)(head - a.hq - a.hk) * a.max_seq + pos) * HD;
+        dst = a.vcache + ((size_t)(head - a.hq - a.hk) * a.max_seq + kv_row) * HD;
     }
 #pragma unroll
     for (int i = 0; i < HD; i += 8) {
@@ -251,7 +316,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
     const uint32_t rank = cluster_rank();
     const int pair = (int)blockIdx.x >> 1, pairs = (int)gridDim.x >> 1;
     const int tiles = a.tiles_m * a.tiles_n;
+    const int units = tiles * a.slices;                 // unit u: tile u % tiles, K-slice u / tiles
     const int kblocks = (a.K + kTileK - 1) / kTileK;
+    auto first_kb = [&](int slice) { return (int)((long long)kblocks * slice / a.slices); };
 
     if (warp == 1) tmem_alloc<2>(&tmem_slot, 512);
     if (tid == 0) {
@@ -279,11 +346,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
             if (lane == 0) {
                 bool ok = true;
                 int t = 0;
-                for (int tile = pair; tile < tiles && ok; tile += pairs) {
+                for (int u = pair; u < units && ok; u += pairs) {
+                    const int tile = u % tiles, slice = u / tiles;
                     const int tm = tile % a.tiles_m, tn = tile / a.tiles_m;
                     const int ra = tm * kTileM + (int)rank * 128;
                     const int rw = KIND == WK_SWIGLU ? tn * 128 + (int)rank * a.N : tn * kTileN + (int)rank * 128;
-                    for (int kb = 0; kb < kblocks; ++kb, ++t) {
+                    for (int kb = first_kb(slice), ke = first_kb(slice + 1); kb < ke; ++kb, ++t) {
                         const int st = t % kStages;
                         if (t >= kStages && !mbar_wait(&empty[st], (uint32_t)((t / kStages - 1) & 1), kWaitLimitNs)) {
                             ok = false;
@@ -309,15 +377,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
             if (rank == 0 && lane == 0) {
                 bool ok = true;
                 int t = 0, n = 0;
-                for (int tile = pair; tile < tiles && ok; tile += pairs, ++n) {
+                for (int u = pair; u < units && ok; u += pairs, ++n) {
                     const int b = n & 1;
+                    const int k0 = first_kb(u / tiles), ke = first_kb(u / tiles + 1);
                     if (n >= 2 && !mbar_wait(&acc_free[b], (uint32_t)((n / 2 - 1) & 1), kWaitLimitNs)) {
                         ok = false;
                         break;
                     }
                     umma_fence_after();
                     const uint32_t acc = tmem + (uint32_t)(b * kTileN);
-                    for (int kb = 0; kb < kblocks; ++kb, ++t) {
+                    for (int kb = k0; kb < ke; ++kb, ++t) {
                         const int st = t % kStages;
                         if (!mbar_wait(&full[st], (uint32_t)((t / kStages) & 1), kWaitLimitNs)) {
                             ok = false;
@@ -328,7 +397,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
 #pragma unroll
                         for (int k = 0; k < kTileK / 16; ++k)
                             umma_ss<2>(acc, umma_desc(sa + 32 * k, 16, kSbo), umma_desc(sa + kHalf + 32 * k, 16, kSbo),
-                                       kIdesc, kb > 0 || k > 0);
+                                       kIdesc, kb > k0 || k > 0);
                         umma_commit_pair(&empty[st]);
                     }
                     if (ok) umma_commit_pair(&acc_full[b]);
@@ -341,8 +410,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
             float* stg = staging + (warp - 2) * 32 * kEpiPitch;
             bool ok = true;
             int n = 0;
-            for (int tile = pair; tile < tiles; tile += pairs, ++n) {
+            for (int u = pair; u < units; u += pairs, ++n) {
                 const int b = n & 1;
+                const int tile = u % tiles;
                 ok = mbar_wait(&acc_full[b], (uint32_t)((n / 2) & 1), kWaitLimitNs);
                 if (!__all_sync(0xffffffffu, ok)) {
                     ok = false;
@@ -350,8 +420,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
                 }
                 umma_fence_after();
                 const int tm = tile % a.tiles_m, tn = tile / a.tiles_m;
-                wide_epilogue<KIND, HD>(a, tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(b * kTileN),
-                                        tm * kTileM + (int)rank * 128 + 32 * quad, tn, stg);
+                const uint32_t acc = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(b * kTileN);
+                if (a.slices == 1 || merge_slices(a, acc, tile, u / tiles, (int)rank * 4 + quad))
+                    wide_epilogue<KIND, HD>(a, acc, tm * kTileM + (int)rank * 128 + 32 * quad, tn, stg);
                 umma_fence_before();
                 __syncwarp();
                 if (lane == 0) cluster_arrive(cluster_addr(&acc_free[b], 0));
@@ -427,10 +498,14 @@ cudaError_t launch_wide(int kind, int hd, const WideArgs& args, cudaStream_t s) 
     WideArgs a = args;
     a.tiles_m = (a.M + kTileM - 1) / kTileM;
     a.tiles_n = wide_tiles_n(kind, a.N);
+    // K-slices: as many as there are pairs for, each at least 8 stages long
+    const int tiles = a.tiles_m * a.tiles_n, kblocks = (a.K + kTileK - 1) / kTileK;
+    const int pairs_max = std::min(sm_count() / 2, kWideUnits);
+    a.slices = a.part != nullptr && a.ticket != nullptr ? std::max(1, std::min(pairs_max / tiles, kblocks / 8)) : 1;
     auto run = [&](auto kern) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmem);
         if (e != cudaSuccess) return e;
-        const int pairs = std::min(sm_count() / 2, a.tiles_m * a.tiles_n);
+        const int pairs = std::min(sm_count() / 2, tiles * a.slices);
         kern<<<2 * pairs, kWideThreads, kWideSmem, s>>>(a);
         return cudaGetLastError();
     };

@@ -14,6 +14,10 @@
 // works on the other.  O is rescaled only when a row's maximum grew by more
 // than 2^8: the factor 2^(m - m_ref) of the rest stays exact in fp32 and bf16
 // alike (a power of two apart, the relative precision is the same).
+// STATES: the rows are several states of r rows (the hidden-state DP's); all
+// see the cache's keys below p0, and each row its own state's rows up to
+// itself, so the key tiles are the cache's and then those of the block's own
+// K/V rows under a band mask.
 // Queries come prepared (QK-norm, RoPE, log2(e) / sqrt(hd)), the keys and
 // values of these rows are already in the cache.
 //
@@ -44,7 +48,7 @@ KS_DEV float fast_exp2(float x) {
     return y;
 }
 
-template <int HD>
+template <int HD, bool STATES>
 __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_constant__ WideAttnArgs a) {
     constexpr int CH = HD / 64;              // 64-column chunks of a tile
     constexpr uint32_t TB = CH * kChunk;     // bytes of one 128-row tile
@@ -64,10 +68,12 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
     const int q0 = (a.blocks - 1 - (int)blockIdx.x / a.hq) * (2 * kQ);   // first row of this CTA
     // key tiles of each query tile (a tile without rows has none)
     int nt[2];
+    const int n_cache = STATES ? (a.p0 + kQ - 1) / kQ : 1 << 30;                // key tiles from the cache
+    const int own0 = STATES ? (q0 - q0 % a.state_rows) / kQ : 0;                // first tile of own rows
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         const int first = q0 + i * kQ, last = min(a.M, first + kQ) - 1;
-        nt[i] = first < a.M ? (a.p0 + last) / kQ + 1 : 0;
+        nt[i] = first >= a.M ? 0 : STATES ? n_cache + last / kQ - own0 + 1 : (a.p0 + last) / kQ + 1;
     }
     const int n = max(nt[0], nt[1]);
 
@@ -108,7 +114,10 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
                         break;
                     }
                     mbar_expect_tx(&kv_full[st], TB);
-                    tma_3d(ring + (size_t)st * TB, &a.kvmap, 0,
+                    if (STATES && (t >> 1) >= n_cache)
+                        tma_3d(ring + (size_t)st * TB, (t & 1) ? &a.vxmap : &a.kxmap, 0,
+                               kvh * a.own_ld + (own0 + (t >> 1) - n_cache) * kQ, 0, &kv_full[st]);
+                    else tma_3d(ring + (size_t)st * TB, &a.kvmap, 0,
                            ((t & 1) ? a.kv_row_v : a.kv_row_k) + kvh * a.max_seq + (t >> 1) * kQ, 0, &kv_full[st]);
                 }
                 if (!ok) {   // the copies in flight land before the CTA leaves
@@ -187,13 +196,26 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
                 tmem_wait_ld();
 #pragma unroll
                 for (int c = 0; c < 4; ++c) tmem_pin(s[c]);
-                if (kQ * (j + 1) > a.p0 + q0 + i * kQ + 1) {   // some key of the tile lies past the tile's first row
-                    const int seen = pos - kQ * j;             // keys 0 .. seen of the tile
+                // keys lo .. hi of the tile are seen; tiles that every row sees whole need no mask
+                int lo = 0, hi = pos - kQ * j;
+                bool masked = kQ * (j + 1) > a.p0 + q0 + i * kQ + 1;
+                if (STATES) {
+                    if (j < n_cache) {
+                        hi = a.p0 - 1 - kQ * j;
+                        masked = kQ * (j + 1) > a.p0;
+                    } else {
+                        const int base = (own0 + j - n_cache) * kQ;
+                        lo = row - row % a.state_rows - base;
+                        hi = row - base;
+                        masked = true;
+                    }
+                }
+                if (masked) {
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
 #pragma unroll
                         for (int q = 0; q < 32; ++q)
-                            if (32 * c + q > seen) s[c][q] = 0xff800000u;   // -inf
+                            if (32 * c + q > hi || (STATES && 32 * c + q < lo)) s[c][q] = 0xff800000u;   // -inf
                 }
                 float mx[4];
 #pragma unroll
@@ -204,7 +226,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
                 }
                 const float mnew = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
                 if (j == 0) {
-                    m = mnew;    // key 0 is seen by every row
+                    m = mnew;
                 } else if (__any_sync(0xffffffffu, mnew > m + kRescale)) {
                     // only rows that grew change: a row never depends on its neighbours
                     const float mm = mnew > m + kRescale ? mnew : m, alpha = fast_exp2(m - mm);
@@ -221,13 +243,15 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
                         tmem_st32(o_at + c, o);
                     }
                 }
+                // a state's row may have seen no key yet: P is then 0
+                const float ref = STATES && m == -INFINITY ? 0.f : m;
                 float sum[4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     sum[c] = 0.f;
 #pragma unroll
                     for (int q = 0; q < 32; ++q) {
-                        const float p = fast_exp2(__uint_as_float(s[c][q]) - m);
+                        const float p = fast_exp2(__uint_as_float(s[c][q]) - ref);
                         sum[c] += p;
                         s[c][q] = __float_as_uint(p);
                     }
@@ -295,8 +319,13 @@ cudaError_t launch_wide_attention(int hd, const WideAttnArgs& args, cudaStream_t
         kern<<<a.hq * a.blocks, kThreads, smem, s>>>(a);
         return cudaGetLastError();
     };
-    if (hd == 128) return run(wide_attn_kernel<128>, wide_attn_smem<128>());
-    if (hd == 64) return run(wide_attn_kernel<64>, wide_attn_smem<64>());
+    const bool st = a.state_rows > 0;
+    if (hd == 128)
+        return st ? run(wide_attn_kernel<128, true>, wide_attn_smem<128>())
+                  : run(wide_attn_kernel<128, false>, wide_attn_smem<128>());
+    if (hd == 64)
+        return st ? run(wide_attn_kernel<64, true>, wide_attn_smem<64>())
+                  : run(wide_attn_kernel<64, false>, wide_attn_smem<64>());
     return cudaErrorInvalidValue;
 }
 
