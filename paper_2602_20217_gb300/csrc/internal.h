@@ -117,13 +117,15 @@ struct WideArgs {
     CUtensorMap amap, wmap;     // make_wide_map of the input rows and of the weights
     int M, N, K;                // rows, output features (WK_SWIGLU: d_ff), inputs
     int tiles_m, tiles_n;       // set by launch_wide
-    int slices;                 // set by launch_wide: K-slices of a tile
-    float* part;                // kWidePartFloats partial sums of K-sliced tiles
+    int full, tail, share;      // set by launch_wide: whole tiles, tiles cut along K, stages per pair of the latter
+    float* part;                // kWidePartFloats partial sums of the cut tiles (null: none is cut)
     int* ticket;                // kWideTickets arrivals, zero between launches
+    float* capture;             // WK_RESID: rows from capture_from on are also written here, [row - capture_from][N]
+    int capture_from;
     int d;                      // model width (the norm's)
     float eps;
     const float* ss_in;         // [ss_n][ss_ld] sums of squares of the input rows (all kinds but WK_RESID)
-    float* ss_out;              // WK_RESID: the same, one slot per tile of the output
+    float* ss_out;              // WK_RESID: the same of its output, one slot per 128 features (or null)
     int ss_n, ss_ld;
     float* x;                   // WK_RESID: [M][N] fp32 residual, added to
     __nv_bfloat16* xg;          // WK_RESID: [M][N] new residual times gain, the next projection's input
@@ -139,18 +141,20 @@ struct WideArgs {
     unsigned long long* best;   // WK_ARGMAX: [M] keys, merged by atomicMax
     int* err;                   // device status word
 };
-// K-sliced launches have at most kWideUnits (tile, slice) units, one per CTA
-// pair: 256 x 256 partial sums each, and 8 row groups of 32 per tile.
-constexpr int kWideUnits = 76;
-constexpr size_t kWidePartFloats = (size_t)kWideUnits * 256 * 256;
-constexpr int kWideTickets = kWideUnits * 8;
+// At most kWidePairs CTA pairs work on a launch's cut tiles, of which there
+// are fewer than pairs: one 256 x 256 slab per (pair, tile) part, 16 groups of
+// 32 rows x 128 columns per tile.
+constexpr int kWidePairs = 76;
+constexpr size_t kWidePartFloats = (size_t)2 * kWidePairs * 256 * 256;
+constexpr int kWideTickets = kWidePairs * 16;
 int wide_tiles_n(int kind, int N);
+inline int wide_ss_slots(int d) { return 2 * ((d + 255) / 256); }   // of a WK_RESID launch's ss_out
 cudaError_t launch_wide(int kind, int hd, const WideArgs& a, cudaStream_t s);
 // tokens[m] = the argmax that key best[m] stands for (0 for no key)
 cudaError_t launch_wide_tokens(const unsigned long long* best, int M, int32_t* tokens, cudaStream_t s);
 cudaError_t launch_wide_embed(const __nv_bfloat16* embed, const int32_t* tok, int M, int d, int vocab, float* x,
                               __nv_bfloat16* xg, const __nv_bfloat16* gain, float* ss, int ss_n, int ss_ld,
-                              cudaStream_t s);
+                              float* capture, int capture_from, cudaStream_t s);
 // Causal attention of M rows at positions p0 .. over the cache (wide_attn.cu).
 // state_rows > 0: the rows are independent states of state_rows rows; each row
 // sees the cache below p0 and its own state's rows up to itself.

@@ -228,7 +228,6 @@ static bool config_ok(const ks_config* c) {
 // Rows of a wide prefill chunk: enough for the GEMMs to be bound by the
 // tensor cores, few enough for the activations to stay in L2.
 constexpr int kWideChunk = 2048;
-constexpr int kWideMinRows = 64;   // fewer lead rows take the ordinary passes
 static int wide_chunk_rows(const ks_config* c) {
     return std::min(kWideChunk, (int)align_up((size_t)c->max_seq, 256));
 }
@@ -251,7 +250,7 @@ static WideLayout wide_layout(const ks_config* c, int rows, size_t base) {
     W.q = take(sizeof(__nv_bfloat16) * M * hqd);
     W.ao = take(sizeof(__nv_bfloat16) * M * hqd);
     W.act = take(sizeof(__nv_bfloat16) * M * c->d_ff);
-    W.ss = take(sizeof(float) * M * wide_tiles_n(WK_RESID, c->d_model));
+    W.ss = take(sizeof(float) * M * wide_ss_slots(c->d_model));
     W.bytes = off - base;
     return W;
 }
@@ -332,17 +331,17 @@ static Layout make_layout(const ks_config* c) {
     L.amax_idx = take(sizeof(int) * (size_t)gemv_groups(c->vocab, c->dtype) * 16);
     // tokens: rows[R+1] | target[R] | result[R+3] | err | prompt/out[max_seq]
     L.tok = take(sizeof(int) * ((size_t)3 * R + 8 + c->max_seq));
-    // A prefill's wide chunks use the space of what is dead until its last
-    // pass: attention partials, logits, history and its snapshot; only models
-    // of few layers need more than these take.
+    // A prefill's wide chunks use the space of what is dead until they are
+    // done: attention partials, logits and history; only models of few layers
+    // need more than these take.
     L.wide_rows = c->dtype == KS_DTYPE_BF16 ? wide_chunk_rows(c) : 0;
     L.wide = off;
     L.attn_part = take(sizeof(float) * (size_t)R * c->n_q_heads * L.n_chunks_max * (hd + 4));
     L.logits = take(sizeof(float) * (size_t)R * c->vocab);
     if (L.wide_rows) off = std::max(off, L.wide + dp_wide_layout(c, kDpWideRows, 0).bytes);   // the DP's, beside the history
     L.hist = take(sizeof(float) * (size_t)(nsub + 1) * L.hist_slots * R * d);
-    L.hist_snap = take(sizeof(float) * (size_t)(nsub + 1) * R * d);  // the prefill's history entry
     off = std::max(off, L.wide + wide_layout(c, L.wide_rows, 0).bytes);
+    L.hist_snap = take(sizeof(float) * (size_t)(nsub + 1) * R * d);  // the prefill's history entry
     L.hist_idx = take(sizeof(int) * (size_t)L.hist_slots * R);
     L.sims = take(sizeof(float) * nsub);
     L.mask = take(nsub);
@@ -751,9 +750,9 @@ static ks_status forward(ks_model* m, const int32_t* tok, int R, int p0, const u
 }
 
 // The whole target over M <= wide_rows prompt rows at positions p0..: fills
-// the K/V cache of every layer.  No logits and no history: a prefill's last
-// rows take the ordinary pass (forward).
-static ks_status wide_forward(ks_model* m, const int32_t* tok, int M, int p0) {
+// the K/V cache of every layer; the hidden states of the rows at positions
+// from `keep` on go to the history snapshot, [2L+1][max_rows][d].  No logits.
+static ks_status wide_forward(ks_model* m, const int32_t* tok, int M, int p0, int keep) {
     const ks_config& c = m->cfg;
     const int d = c.d_model, F = c.d_ff, L = c.n_layers, hd = c.head_dim, hqd = c.n_q_heads * hd;
     const int nqkv = (c.n_q_heads + 2 * c.n_kv_heads) * hd;
@@ -765,7 +764,7 @@ static ks_status wide_forward(ks_model* m, const int32_t* tok, int M, int p0) {
     g.d = d;
     g.eps = c.rms_eps;
     g.ss_in = g.ss_out = reinterpret_cast<float*>(m->ws + W.ss);
-    g.ss_n = wide_tiles_n(WK_RESID, d);
+    g.ss_n = wide_ss_slots(d);
     g.ss_ld = m->lay.wide_rows;
     g.x = reinterpret_cast<float*>(m->ws + W.x);
     g.xg = reinterpret_cast<__nv_bfloat16*>(m->ws + W.xg);
@@ -779,9 +778,11 @@ static ks_status wide_forward(ks_model* m, const int32_t* tok, int M, int p0) {
     g.err = m->err;
     g.part = reinterpret_cast<float*>(m->ws + m->lay.wide_part);
     g.ticket = reinterpret_cast<int*>(m->ws + m->lay.wide_ticket);
+    g.capture_from = keep - p0;   // before this chunk: negative
+    auto plane = [&](int i) { return keep - p0 < M ? m->hist_snap + (size_t)i * c.max_rows * d : nullptr; };
     KS_TRY(launch(m, K_EMBED, [&] {
         return launch_wide_embed(bf(m->embed), tok, M, d, c.vocab, g.x, g.xg, bf(m->attn_norm[0]), g.ss_out, g.ss_n,
-                                 g.ss_ld, s);
+                                 g.ss_ld, plane(0), g.capture_from, s);
     }, "prompt embed"));
     auto project = [&](int kind, int klass, const CUtensorMap& in, const CUtensorMap& w, int N, int K) -> ks_status {
         g.amap = in;
@@ -811,9 +812,11 @@ static ks_status wide_forward(ks_model* m, const int32_t* tok, int M, int p0) {
         at.err = m->err;
         KS_TRY(launch(m, K_ATTN, [&] { return launch_wide_attention(hd, at, s); }, "prompt attention"));
         g.gain = bf(m->mlp_norm[l]);
+        g.capture = plane(2 * l + 1);
         KS_TRY(project(WK_RESID, K_OPROJ, m->wide_ao, m->wide_o[l], d, hqd));
         KS_TRY(project(WK_SWIGLU, K_GATEUP, m->wide_xg, m->wide_gu[l], F, d));
         g.gain = bf(l + 1 < L ? m->attn_norm[l + 1] : m->final_norm);
+        g.capture = plane(2 * l + 2);
         KS_TRY(project(WK_RESID, K_DOWN, m->wide_act, m->wide_down[l], d, F));
     }
     return KS_OK;
@@ -998,11 +1001,11 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
         ok = ok && make_weight_map(&m->map_kv, m->kv,
                                    2 * (uint64_t)L * cfg->n_kv_heads * (uint64_t)cfg->max_seq, cfg->head_dim,
                                    cfg->head_dim / 64);
-        for (int b = 0; b < R; ++b) {
-            ok = ok && make_stage_map(&m->map_xg[b], m->xg, R, d, b + 1, 4);
-            ok = ok && make_stage_map(&m->map_xg2[b], m->xg, R, d, b + 1, 2);
-            ok = ok && make_stage_map(&m->map_attn_out[b], m->attn_out, R, hqd, b + 1, 4);
-            ok = ok && make_stage_map(&m->map_act[b], m->act, R, F, b + 1, 4);
+        for (int r = 0; r < R; ++r) {
+            ok = ok && make_stage_map(&m->map_xg[r], m->xg, R, d, r + 1, 4);
+            ok = ok && make_stage_map(&m->map_xg2[r], m->xg, R, d, r + 1, 2);
+            ok = ok && make_stage_map(&m->map_attn_out[r], m->attn_out, R, hqd, r + 1, 4);
+            ok = ok && make_stage_map(&m->map_act[r], m->act, R, F, r + 1, 4);
         }
         m->wide_qkv.resize(L);
         m->wide_o.resize(L);
@@ -1109,6 +1112,8 @@ static void reset_history(ks_model* m, int lastlen) {
     m->hist_next = 1;
 }
 
+static ks_status lm_head_rows(ks_model* m, int R, int32_t* tokens);
+
 ks_status ks_prefill(ks_model* m, const int32_t* tokens, int32_t n, int32_t* next_token) {
     if (!m || !tokens || !next_token) {
         set_error("ks_prefill: null argument");
@@ -1134,30 +1139,45 @@ ks_status ks_prefill(ks_model* m, const int32_t* tokens, int32_t n, int32_t* nex
     KS_CUDA(cudaMemcpyAsync(m->seq, m->h_buf, sizeof(int32_t) * n, cudaMemcpyHostToDevice, m->stream), "prompt upload");
     m->h2d += sizeof(int32_t) * n;
     const int R = c.max_rows;
-    // chunks aligned to the end so the last chunk holds the last R rows
-    const int first = n - R * ((n - 1) / R);
-    int start = 0;
-    int len = first;
-    const int init_slot = 0;
-    // bf16: every row but the last chunk's goes through the wide path, in even
-    // chunks of whole tiles
-    const int lead = n - std::min(n, R);
-    if (m->dtype == KS_DTYPE_BF16 && lead >= kWideMinRows) {
-        const int parts = (lead + m->lay.wide_rows - 1) / m->lay.wide_rows;
-        const int rows = std::min(m->lay.wide_rows, (int)align_up((size_t)(lead + parts - 1) / parts, 256));
-        for (; start < lead; start += rows)
-            KS_TRY(wide_forward(m, m->seq + start, std::min(rows, lead - start), start));
-        start = lead;
-        len = R;
-    }
-    while (start < n) {
-        const bool last = (start + len == n);
-        KS_TRY(forward(m, m->seq + start, len, start, nullptr, last ? init_slot : -1, last ? m->target : nullptr));
-        start += len;
-        len = R;
-    }
-    // pending = argmax of the last prompt row
+    // the last rows leave their history and logits; pending = argmax of the last
     const int lastlen = (n <= R) ? n : R;
+    const size_t row_bytes = sizeof(float) * (size_t)R * c.d_model;   // a plane's rows of one history entry
+    // A wide pass costs about what three passes of 9 to 16 rows or four of up
+    // to 8 cost (four Llama-3-8B layers: 820 us at any length up to 256 against
+    // 1385, 1780, 2724 us at 32, 33 and 64 tokens in passes of 16).
+    const int passes = (n + R - 1) / R;
+    const bool wide = m->dtype == KS_DTYPE_BF16 && passes * (R > 8 ? 3 : 2) > 7;
+    if (wide) {
+        // even wide chunks of whole tiles; the last rows' states go to the
+        // snapshot of the history entry, from where the LM head takes them
+        const int parts = (n + m->lay.wide_rows - 1) / m->lay.wide_rows;
+        const int rows = std::min(m->lay.wide_rows, (int)align_up((size_t)(n + parts - 1) / parts, 256));
+        for (int start = 0; start < n; start += rows)
+            KS_TRY(wide_forward(m, m->seq + start, std::min(rows, n - start), start, n - lastlen));
+        KS_CUDA(cudaMemcpy2DAsync(m->hist, row_bytes * m->lay.hist_slots, m->hist_snap, row_bytes, row_bytes,
+                                  m->nsub + 1, cudaMemcpyDeviceToDevice, m->stream),
+                "history entry");
+        const int d = c.d_model;
+        KS_CUDA(cudaMemcpyAsync(m->x, m->hist_snap + (size_t)m->nsub * R * d, sizeof(float) * lastlen * d,
+                                cudaMemcpyDeviceToDevice, m->stream),
+                "last rows");
+        KS_TRY(launch(m, K_EMBED, [&]() -> cudaError_t {
+            rows_prep_kernel<__nv_bfloat16><<<dim3(lastlen, (d + 255) / 256), 256, 0, m->stream>>>(
+                m->x, d, m->ss, m->xg, reinterpret_cast<const __nv_bfloat16*>(m->final_norm), nullptr);
+            return cudaGetLastError();
+        }, "last rows"));
+        KS_TRY(lm_head_rows(m, lastlen, m->target));
+        m->last_pass_rows = lastlen;
+    } else {
+        // chunks aligned to the end so the last chunk holds the last R rows
+        int start = 0, len = n - R * ((n - 1) / R);
+        while (start < n) {
+            const bool last = (start + len == n);
+            KS_TRY(forward(m, m->seq + start, len, start, nullptr, last ? 0 : -1, last ? m->target : nullptr));
+            start += len;
+            len = R;
+        }
+    }
     KS_CUDA(cudaMemcpyAsync(m->rows, m->target + (lastlen - 1), sizeof(int32_t), cudaMemcpyDeviceToDevice, m->stream),
             "pending");
     KS_CUDA(cudaMemcpyAsync(m->h_buf, m->rows, sizeof(int32_t), cudaMemcpyDeviceToHost, m->stream), "pending");
@@ -1171,10 +1191,10 @@ ks_status ks_prefill(ks_model* m, const int32_t* tokens, int32_t n, int32_t* nex
     m->prompt_pending = m->pending;
     m->prompt_rows = lastlen;
     // keep the prefill's history entry (slot 0 of every plane) for ks_rewind
-    const size_t row_bytes = sizeof(float) * (size_t)c.max_rows * c.d_model;
-    KS_CUDA(cudaMemcpy2DAsync(m->hist_snap, row_bytes, m->hist, row_bytes * m->lay.hist_slots, row_bytes,
-                              m->nsub + 1, cudaMemcpyDeviceToDevice, m->stream),
-            "history snapshot");
+    if (!wide)
+        KS_CUDA(cudaMemcpy2DAsync(m->hist_snap, row_bytes, m->hist, row_bytes * m->lay.hist_slots, row_bytes,
+                                  m->nsub + 1, cudaMemcpyDeviceToDevice, m->stream),
+                "history snapshot");
     reset_history(m, lastlen);
     return KS_OK;
 }
@@ -1824,8 +1844,9 @@ static ks_status dp_wide_sublayer(ks_model* m, int i, int S, int r, int p0, int 
     WideArgs g{};
     g.d = d;
     g.eps = c.rms_eps;
-    g.ss_in = g.ss_out = reinterpret_cast<float*>(m->ws + W.ss);
-    g.ss_n = wide_tiles_n(WK_RESID, d);
+    float* ss = reinterpret_cast<float*>(m->ws + W.ss);
+    g.ss_in = ss;
+    g.ss_n = wide_tiles_n(WK_RESID, d);   // one slot per 256 features, as dp_prep leaves them
     g.ss_ld = rows;
     g.xg = at(W.xg);
     g.act = at(W.act);
@@ -1857,7 +1878,7 @@ static ks_status dp_wide_sublayer(ks_model* m, int i, int S, int r, int p0, int 
         g.M = n * r;
         g.x = E + (size_t)j0 * r * d;
         KS_TRY(launch(m, K_EMBED, [&] {
-            return launch_dp_prep(G, j0, n, valid, r, d, g.gain, E, g.xg, g.ss_out, rows, s);
+            return launch_dp_prep(G, j0, n, valid, r, d, g.gain, E, g.xg, ss, rows, s);
         }, "dp states"));
         if (attn) {
             KS_TRY(project(WK_QKV, K_QKV, maps[0], m->wide_qkv[l], (c.n_q_heads + 2 * c.n_kv_heads) * hd, d));

@@ -94,12 +94,21 @@ KS_DEV void tmem_ld32(uint32_t (&r)[32], uint32_t addr) {
           "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(addr));
 }
+KS_DEV void tmem_ld16(uint32_t (&r)[16], uint32_t addr) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(addr));
+}
 KS_DEV void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // Ties the registers of a tmem_ld32 to this point (after the wait): volatile
 // statements keep their order, so no use can move before the wait.
-KS_DEV void tmem_pin(uint32_t (&r)[32]) {
+template <int N>
+KS_DEV void tmem_pin(uint32_t (&r)[N]) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) asm volatile("" : "+r"(r[i]));
+    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
 }
 KS_DEV void tmem_st32(uint32_t addr, const uint32_t (&r)[32]) {
     asm volatile(
