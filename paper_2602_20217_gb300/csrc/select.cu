@@ -1,7 +1,7 @@
 // a4 and a5 of the hot path: history cosines and knapsack mask selection.
 //
-// ks_cosine  - Sec. 2's matrix cosine, one CTA per pair; each warp takes rows
-//              in turn, the row terms are summed in row order by one thread.
+// ks_cosine  - Sec. 2's matrix cosine, a cluster of CTAs per pair; each warp
+//              takes rows in turn, one thread sums the row terms in row order.
 // ks_select_mask - Sec. 3.4 integer weight normalisation (App. C latency
 //              model) and the exact 0/1 knapsack of Sec. 3.3 over the 2L
 //              sublayers: items processed in order 1..2L, all capacities of
@@ -13,40 +13,78 @@
 #include "../../include/knapspec.h"
 #include "common.cuh"
 #include "internal.h"
+#include "umma.cuh"
 
+#include <algorithm>
+#include <climits>
 #include <cmath>
 
 namespace ks {
 
+// A cluster of kCosCtas CTAs per pair, a row per warp at a time: one CTA per
+// pair left most of the chip idle (64 pairs on 152 SMs, a load in flight per
+// lane; 64 pairs of 25 rows of 4096 fp32: 35.8 us, now 12.2 us with 16-byte
+// loads, eight of each side in flight).  The warps' row terms meet in the
+// first CTA's shared memory and one thread adds them in row order.
+constexpr int kCosCtas = 4;
 constexpr int kCosThreads = 256;
 
-template <typename T>
-__global__ void __launch_bounds__(kCosThreads) cosine_kernel(const T* X, const T* Y, int rows, int d,
-                                                             int64_t pair_stride, const int32_t* row_index,
-                                                             float* out) {
+// VEC: elements per load, 16 bytes' worth or 1 (rows that are not 16-byte aligned)
+template <typename T, int VEC>
+__global__ void __cluster_dims__(kCosCtas, 1, 1) __launch_bounds__(kCosThreads)
+    cosine_kernel(const T* X, const T* Y, int rows, int d, int64_t pair_stride, const int32_t* row_index, float* out) {
     extern __shared__ float rowcos[];
-    const int p = blockIdx.x;
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");   // this CTA runs: its shared memory may be written
+    const int64_t p = blockIdx.x / kCosCtas;
+    const uint32_t rank = cluster_rank();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const T* Xp = X + (size_t)p * pair_stride;
-    const T* Yp = Y + (size_t)p * pair_stride;
-    for (int i = warp; i < rows; i += kCosThreads / 32) {
+    const T* Xp = X + p * pair_stride;
+    const T* Yp = Y + p * pair_stride;
+    bool waited = false;
+    for (int i = (int)rank + kCosCtas * warp; i < rows; i += kCosCtas * (kCosThreads / 32)) {
         const int64_t ri = row_index ? row_index[i] : i;
         const T* x = Xp + ri * d;
         const T* y = Yp + ri * d;
         float xy = 0.f, xx = 0.f, yy = 0.f;
-        for (int k = lane; k < d; k += 32) {
-            const float a = to_float(x[k]), b = to_float(y[k]);
+        auto add = [&](float a, float b) {
             xy = fmaf(a, b, xy);
             xx = fmaf(a, a, xx);
             yy = fmaf(b, b, yy);
+        };
+        if constexpr (VEC == 1) {
+#pragma unroll 8
+            for (int k = lane; k < d; k += 32) add(to_float(x[k]), to_float(y[k]));
+        } else {
+            const uint4* xv = reinterpret_cast<const uint4*>(x);
+            const uint4* yv = reinterpret_cast<const uint4*>(y);
+#pragma unroll 8
+            for (int k = lane; k < d / VEC; k += 32) {
+                const uint4 u = xv[k], v = yv[k];
+                const uint32_t a[4] = {u.x, u.y, u.z, u.w}, b[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if constexpr (VEC == 4) {
+                        add(__uint_as_float(a[e]), __uint_as_float(b[e]));
+                    } else {
+                        add(bf16_lo(a[e]), bf16_lo(b[e]));
+                        add(bf16_hi(a[e]), bf16_hi(b[e]));
+                    }
+                }
+            }
         }
         xy = warp_sum(xy);
         xx = warp_sum(xx);
         yy = warp_sum(yy);
-        if (lane == 0) rowcos[i] = xy / (sqrtf(xx) * sqrtf(yy));
+        if (!waited) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        waited = true;
+        if (lane == 0) {
+            const float c = xy / (sqrtf(xx) * sqrtf(yy));
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(&rowcos[i], 0)), "f"(c) : "memory");
+        }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    if (!waited) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    cluster_sync();   // the row terms are in the first CTA
+    if (rank == 0 && threadIdx.x == 0) {
         float s = 0.f;
         for (int i = 0; i < rows; ++i) s += rowcos[i];
         out[p] = s / (float)rows;
@@ -57,21 +95,29 @@ cudaError_t launch_cosine(const void* X, const void* Y, int dtype, int64_t n_pai
                           int64_t pair_stride, const int32_t* row_index, float* out, cudaStream_t s) {
     const size_t smem = sizeof(float) * (size_t)rows;
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
-    if (dtype == KS_DTYPE_BF16)
-        cosine_kernel<__nv_bfloat16><<<(unsigned)n_pairs, kCosThreads, smem, s>>>(
-            reinterpret_cast<const __nv_bfloat16*>(X), reinterpret_cast<const __nv_bfloat16*>(Y), rows, d,
-            pair_stride, row_index, out);
-    else
-        cosine_kernel<float><<<(unsigned)n_pairs, kCosThreads, smem, s>>>(
-            reinterpret_cast<const float*>(X), reinterpret_cast<const float*>(Y), rows, d, pair_stride,
-            row_index, out);
-    return cudaGetLastError();
+    const int vec = dtype == KS_DTYPE_BF16 ? 8 : 4;   // elements of 16 bytes
+    // every row of every pair starts on a 16-byte boundary
+    const bool aligned = d % vec == 0 && pair_stride % vec == 0 &&
+                         ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 15) == 0;
+    constexpr int64_t kMost = 1 << 28;   // pairs of a launch: the grid's limit
+    auto run = [&](auto kern, auto x, auto y) {
+        for (int64_t p = 0; p < n_pairs; p += kMost)
+            kern<<<(unsigned)((n_pairs - p < kMost ? n_pairs - p : kMost) * kCosCtas), kCosThreads, smem, s>>>(
+                x + p * pair_stride, y + p * pair_stride, rows, d, pair_stride, row_index, out + p);
+        return cudaGetLastError();
+    };
+    if (dtype == KS_DTYPE_BF16) {
+        auto x = reinterpret_cast<const __nv_bfloat16*>(X), y = reinterpret_cast<const __nv_bfloat16*>(Y);
+        return aligned ? run(cosine_kernel<__nv_bfloat16, 8>, x, y) : run(cosine_kernel<__nv_bfloat16, 1>, x, y);
+    }
+    auto x = reinterpret_cast<const float*>(X), y = reinterpret_cast<const float*>(Y);
+    return aligned ? run(cosine_kernel<float, 4>, x, y) : run(cosine_kernel<float, 1>, x, y);
 }
 
 // ----------------------------------------------------------------- knapsack
 constexpr int kMaxItems = 256;
 constexpr int kMaxTpt = 128;   // ks_select_tpt passes at most KS_TPT_MAX_CANDIDATES; the DP stage more
-constexpr int kKnapThreads = 512;
+constexpr int kKnapMaxThreads = 1024;
 
 struct KnapArgs {
     int kind;                 // 0 latency model, 1 explicit units
@@ -87,104 +133,154 @@ struct KnapArgs {
     int32_t* weights_out;
     int32_t* budget_out;      // optional: the budget used
     long long* best;          // scratch [2][cap + 1]
-    uint8_t* take;            // scratch [n_items][cap + 1]
+    uint32_t* take;           // scratch: choice bits, [n_items][words of cap + 1]
     int cap;                  // capacity of the scratch tables
+    int shared_cap;           // capacity of the tables in shared memory
     int n_frontier;           // > 0: also backtrack the optima of budgets floor(sum w (j + 1) / n_frontier)
     uint8_t* frontier;        // [n_frontier][n_items] masks of those budgets
 };
 
-__global__ void __launch_bounds__(kKnapThreads) knapsack_kernel(const KnapArgs a) {
-    __shared__ int w[kMaxItems];
-    __shared__ long long q[kMaxItems];
-    __shared__ int B;
-    __shared__ long long SW;
-    const int tid = threadIdx.x;
-    const int N = a.n_items;
-    if (tid == 0) {
-        int wa = 1, wm = 1;
-        if (a.kind == 0) {
-            // Sec. 3.4: Delta = min(t_Attn(n), t_MLP), w = round(t / Delta), >= 1
-            // explicit _rn intrinsics: no FMA contraction, the same two
-            // roundings as c2 * n + c3 evaluated left to right
-            const double ta = __dadd_rn(__dmul_rn(a.c2, (double)a.n), a.c3);
-            const double tm = a.c1;
-            const double delta = fmin(ta, tm);
-            wa = (int)llround(__ddiv_rn(ta, delta));
-            wm = (int)llround(__ddiv_rn(tm, delta));
-            if (wa < 1) wa = 1;
-            if (wm < 1) wm = 1;
-        }
-        long long sum = 0;
-        for (int i = 0; i < N; ++i) {
-            // 0-based item i is sublayer i + 1: even i -> Attn, odd i -> MLP
-            w[i] = (a.kind == 0) ? ((i % 2 == 0) ? wa : wm) : a.units[i];
-            sum += w[i];
-        }
-        SW = sum;
-        long long b = a.budget;
-        if (a.budget_frac >= 0.0) b = (long long)floor(__dmul_rn(a.budget_frac, (double)sum));
-        if (b > a.cap) b = a.cap;
-        if (b < 0) b = 0;
-        B = (int)b;
-        if (a.budget_out) *a.budget_out = (int)b;
+// The tables of a budget up to `cap`: two rows of int64 values and a choice
+// bit per (item, capacity).
+__host__ __device__ constexpr int knap_words(int cap) { return (cap + 32) / 32; }
+__host__ __device__ constexpr size_t knap_table_bytes(int n_items, int cap) {
+    return sizeof(long long) * 2 * ((size_t)cap + 1) + sizeof(uint32_t) * (size_t)n_items * knap_words(cap);
+}
+
+// Items N - 1 .. 0 from capacity c; two items' words are read together (the
+// second at both capacities that the first may leave).
+KS_DEV void knap_backtrack(const uint32_t* take, int W, const int* w, int N, int c, uint8_t* mask) {
+    int i = N - 1;
+    for (; i >= 1; i -= 2) {
+        const int w1 = w[i], c1 = max(c - w1, 0);
+        const uint32_t t1 = (take[(size_t)i * W + (c >> 5)] >> (c & 31)) & 1u;
+        const uint32_t skip = (take[(size_t)(i - 1) * W + (c >> 5)] >> (c & 31)) & 1u;
+        const uint32_t took = (take[(size_t)(i - 1) * W + (c1 >> 5)] >> (c1 & 31)) & 1u;
+        const uint32_t t0 = t1 ? took : skip;
+        c -= (t1 ? w1 : 0) + (t0 ? w[i - 1] : 0);
+        mask[i] = (uint8_t)t1;
+        mask[i - 1] = (uint8_t)t0;
     }
-    for (int i = tid; i < N; i += blockDim.x) {
-        // q_i = round((1 - sigma_i) * 2^30), half away from zero, in double
-        const double v = __dmul_rn(__dsub_rn(1.0, (double)a.sims[i]), 1073741824.0);
-        q[i] = llround(v);
-    }
-    __syncthreads();
-    const int cap1 = B + 1;
-    long long* cur = a.best;
-    long long* nxt = a.best + (a.cap + 1);
-    for (int c = tid; c < cap1; c += blockDim.x) cur[c] = 0;
-    __syncthreads();
-    for (int i = 0; i < N; ++i) {
-        const int wi = w[i];
-        const long long qi = q[i];
-        uint8_t* tk = a.take + (size_t)i * (a.cap + 1);
-        for (int c = tid; c < cap1; c += blockDim.x) {
-            long long v = cur[c];
-            uint8_t t = 0;
-            if (c >= wi) {
-                const long long cand = cur[c - wi] + qi;
-                if (cand > v) {
-                    v = cand;
-                    t = 1;
-                }
+    if (i == 0) mask[0] = (uint8_t)((take[c >> 5] >> (c & 31)) & 1u);
+}
+
+// The dynamic program over items 0 .. N - 1, two items a step: v1 is the value
+// with item i decided, at c and at c - w(i + 1), and v2 the value with item
+// i + 1 decided on top; each is taken only on strict improvement, exactly as
+// one item at a time.  Two table reads more per capacity, half the barriers.
+// Returns the row that holds the final values.
+KS_DEV const long long* knap_solve(long long* cur, long long* nxt, uint32_t* take, int W, const int* w,
+                                   const long long* q, int N, int cap1) {
+    const int tid = threadIdx.x, T = blockDim.x;
+    const int rounds = (cap1 + T - 1) / T;   // every warp does each round: the ballots are whole
+    int w0 = w[0], w1 = N > 1 ? w[1] : 0;
+    long long q0 = q[0], q1 = N > 1 ? q[1] : 0;
+    for (int i = 0; i < N; i += 2) {
+        const bool two = i + 1 < N;
+        // the next pair's, while this one is worked on
+        const int w2 = i + 2 < N ? w[i + 2] : 0, w3 = i + 3 < N ? w[i + 3] : 0;
+        const long long q2 = i + 2 < N ? q[i + 2] : 0, q3 = i + 3 < N ? q[i + 3] : 0;
+#pragma unroll 1
+        for (int k = 0; k < rounds; ++k) {
+            const int c = tid + k * T;
+            const bool in = c < cap1;
+            auto at = [&](int x) { return in && x >= 0 ? cur[x] : 0; };
+            const long long a0 = at(c), a1 = at(c - w0) + q0, b0 = at(c - w1), b1 = at(c - w1 - w0) + q0;
+            const bool t0 = in && c >= w0 && a1 > a0;
+            const long long v1 = t0 ? a1 : a0;
+            const bool s0 = c >= w1 + w0 && b1 > b0;
+            const long long with1 = (s0 ? b1 : b0) + q1;
+            const bool t1 = in && two && c >= w1 && with1 > v1;
+            if (in) nxt[c] = t1 ? with1 : v1;
+            const uint32_t m0 = __ballot_sync(0xffffffffu, t0), m1 = __ballot_sync(0xffffffffu, t1);
+            if ((tid & 31) == 0 && in) {
+                take[(size_t)i * W + (c >> 5)] = m0;
+                if (two) take[(size_t)(i + 1) * W + (c >> 5)] = m1;
             }
-            nxt[c] = v;
-            tk[c] = t;
         }
         __syncthreads();
         long long* tmp = cur;
         cur = nxt;
         nxt = tmp;
+        w0 = w2;
+        w1 = w3;
+        q0 = q2;
+        q1 = q3;
     }
-    if (tid == 0) {
-        int c = B;
-        for (int i = N - 1; i >= 0; --i) {
-            const uint8_t t = a.take[(size_t)i * (a.cap + 1) + c];
-            a.mask[i] = t;
-            if (t) c -= w[i];
+    return cur;
+}
+
+// One CTA.  The tables are in shared memory whenever the budget fits (with
+// them in global memory and a barrier per item, a 64-layer model's 128 items
+// at 153 units took 50 us, most of it round trips; now 18); larger budgets
+// use the caller's scratch (256 items at 16000 units: 1941 -> 880 us).
+__global__ void __launch_bounds__(kKnapMaxThreads) knapsack_kernel(const KnapArgs a) {
+    extern __shared__ __align__(16) unsigned char tables[];
+    __shared__ int w[kMaxItems];
+    __shared__ long long q[kMaxItems];
+    __shared__ long long part[kKnapMaxThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int N = a.n_items;
+    int wa = 1, wm = 1;
+    if (a.kind == 0) {
+        // Sec. 3.4: Delta = min(t_Attn(n), t_MLP), w = round(t / Delta), >= 1
+        // explicit _rn intrinsics: no FMA contraction, the same two
+        // roundings as c2 * n + c3 evaluated left to right
+        const double ta = __dadd_rn(__dmul_rn(a.c2, (double)a.n), a.c3);
+        const double tm = a.c1;
+        const double delta = fmin(ta, tm);
+        wa = max(1, (int)llround(__ddiv_rn(ta, delta)));
+        wm = max(1, (int)llround(__ddiv_rn(tm, delta)));
+    }
+    long long sum = 0;
+    for (int i = tid; i < N; i += blockDim.x) {
+        // 0-based item i is sublayer i + 1: even i -> Attn, odd i -> MLP
+        const int wi = (a.kind == 0) ? ((i % 2 == 0) ? wa : wm) : a.units[i];
+        w[i] = wi;
+        sum += wi;
+        // q_i = round((1 - sigma_i) * 2^30), half away from zero, in double
+        q[i] = llround(__dmul_rn(__dsub_rn(1.0, (double)a.sims[i]), 1073741824.0));
+        if (a.weights_out) a.weights_out[i] = wi;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) part[warp] = sum;
+    __syncthreads();
+    long long SW = 0;
+    for (int i = 0; i < (int)blockDim.x / 32; ++i) SW += part[i];
+    long long b = a.budget;
+    if (a.budget_frac >= 0.0) b = (long long)floor(__dmul_rn(a.budget_frac, (double)SW));
+    if (b > a.cap) b = a.cap;
+    if (b < 0) b = 0;
+    const int B = (int)b, cap1 = B + 1;
+    if (tid == 0 && a.budget_out) *a.budget_out = B;
+    // frontier and mask backtracks: one thread each from the shared tables' bits
+    auto finish = [&](const long long* values, const uint32_t* take, int W) {
+        if (tid == 0) {
+            knap_backtrack(take, W, w, N, B, a.mask);
+            if (a.objective) *a.objective = (double)values[B] / 1073741824.0;
         }
-        if (a.objective) *a.objective = (double)cur[B] / 1073741824.0;
-    }
-    // The TPT stage's candidate set: the optimum of each frontier budget,
-    // backtracked from the same table (the DP up to capacity c does not
-    // depend on larger capacities).
-    for (int j = tid; j < a.n_frontier; j += blockDim.x) {
-        int c = (int)((SW * (long long)(j + 1)) / a.n_frontier);
-        if (c > B) c = B;
-        uint8_t* fm = a.frontier + (size_t)j * N;
-        for (int i = N - 1; i >= 0; --i) {
-            const uint8_t t = a.take[(size_t)i * (a.cap + 1) + c];
-            fm[i] = t;
-            if (t) c -= w[i];
+        // The TPT stage's candidate set: the optimum of each frontier budget,
+        // backtracked from the same table (the DP up to capacity c does not
+        // depend on larger capacities).  One candidate per warp.
+        for (int j = warp; j < a.n_frontier; j += (int)blockDim.x / 32) {
+            if (lane != 0) continue;
+            int c = (int)((SW * (long long)(j + 1)) / a.n_frontier);
+            if (c > B) c = B;
+            knap_backtrack(take, W, w, N, c, a.frontier + (size_t)j * N);
         }
+    };
+    if (B <= a.shared_cap) {
+        long long* row = reinterpret_cast<long long*>(tables);
+        uint32_t* take = reinterpret_cast<uint32_t*>(row + 2 * cap1);
+        for (int c = tid; c < cap1; c += blockDim.x) row[c] = 0;
+        __syncthreads();
+        finish(knap_solve(row, row + cap1, take, knap_words(B), w, q, N, cap1), take, knap_words(B));
+    } else {
+        for (int c = tid; c < cap1; c += blockDim.x) a.best[c] = 0;
+        __syncthreads();
+        finish(knap_solve(a.best, a.best + (a.cap + 1), a.take, knap_words(B), w, q, N, cap1), a.take, knap_words(B));
     }
-    if (a.weights_out)
-        for (int i = tid; i < N; i += blockDim.x) a.weights_out[i] = w[i];
 }
 
 size_t select_scratch_bytes(int n_items, int cap) {
@@ -215,10 +311,39 @@ cudaError_t launch_select(const ks_latency* lat, const float* sims, int64_t n, i
     a.budget_out = budget_out;
     a.cap = cap;
     a.best = reinterpret_cast<long long*>(scratch);
-    a.take = reinterpret_cast<uint8_t*>(scratch) + sizeof(long long) * 2 * ((size_t)cap + 1);
+    a.take = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(scratch) + sizeof(long long) * 2 * ((size_t)cap + 1));
     a.n_frontier = n_frontier;
     a.frontier = frontier;
-    knapsack_kernel<<<1, kKnapThreads, 0, s>>>(a);
+    // The budget as the kernel computes it (its weights' sum; one more unit in
+    // case a rounding differs here), for the launch only: the kernel checks
+    // what fits.
+    long long b = budget;
+    if (budget_frac >= 0.0) {
+        double sum = 0.0;
+        if (lat->kind == 1) {
+            for (int i = 0; i < n_items; ++i) sum += lat->units[i];
+        } else {
+            const double ta = lat->c2 * (double)n + lat->c3, tm = lat->c1, dl = std::fmin(ta, tm);
+            sum = 0.5 * n_items * (std::fmax(1.0, std::round(ta / dl)) + std::fmax(1.0, std::round(tm / dl)));
+        }
+        b = (long long)std::fmin(std::floor(budget_frac * sum) + 1.0, 65536.0);
+    }
+    const int want = (int)std::max<long long>(0, std::min<long long>(b, cap));
+    size_t smem = 0;
+    a.shared_cap = -1;
+    if (knap_table_bytes(n_items, want) <= 200 * 1024) {
+        a.shared_cap = want;
+        smem = knap_table_bytes(n_items, want);
+    }
+    // a capacity per thread below 512 (128 items at 153 units: 18.4 us, with
+    // two per thread 22.5), above that two (64 items at 1000: 20.5 against 23.6)
+    const int threads = std::min(kKnapMaxThreads, (want / (want < 512 ? 1 : 2) + 32) / 32 * 32);
+    if (smem > 40 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(knapsack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   200 * 1024);
+        if (e != cudaSuccess) return e;
+    }
+    knapsack_kernel<<<1, threads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -242,56 +367,89 @@ struct TptArgs {
     double* out;              // [0] TPT, [1 + j] alpha of candidate j
 };
 
+// One CTA: a warp per candidate counts its matches and its sublayers, then a
+// thread per (candidate, gamma) evaluates Eq. 3 with the grid search's order
+// kept by the tie rule (the first of the largest values in candidate order,
+// gamma ascending, which is what replacing on strictly larger finds).  One
+// thread doing all of it in sequence took 50 us for 8 candidates at D = 10,
+// 90 for 13 of the hidden-state DP.
 __global__ void __launch_bounds__(256) tpt_kernel(const TptArgs a) {
-    __shared__ double alpha[kMaxTpt];
+    __shared__ double alpha[kMaxTpt], draft[kMaxTpt];
+    __shared__ double best_v[8];
+    __shared__ int best_i[8];
     __shared__ int sel;
-    const int tid = threadIdx.x;
-    for (int j = tid; j < a.K; j += blockDim.x) {
-        int cnt = 0;
-        for (int i = 0; i < a.r; ++i) cnt += a.tokens[(size_t)j * a.r + i] == a.tokens[(size_t)a.K * a.r + i];
-        alpha[j] = __ddiv_rn((double)cnt, (double)a.r);
-        a.out[1 + j] = alpha[j];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double ta = 0.0, tm = 0.0;
+    if (a.kind == 0) {
+        ta = __dadd_rn(__dmul_rn(a.c2, (double)a.n), a.c3);
+        tm = a.c1;
+    }
+    const int32_t* full = a.tokens + (size_t)a.K * a.r;
+    for (int j = warp; j < a.K; j += 8) {
+        int cnt = 0, na = 0, nm = 0;
+        long long units = 0;   // whole numbers below 2^53: exact as the double sum is
+        for (int i = lane; i < a.r; i += 32) cnt += a.tokens[(size_t)j * a.r + i] == full[i];
+        const uint8_t* m = a.frontier + (size_t)j * a.n_items;
+        for (int i = lane; i < a.n_items; i += 32)
+            if (m[i]) {
+                (i % 2 == 0 ? na : nm)++;
+                if (a.kind == 1) units += a.units[i];
+            }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+            na += __shfl_xor_sync(0xffffffffu, na, o);
+            nm += __shfl_xor_sync(0xffffffffu, nm, o);
+            units += __shfl_xor_sync(0xffffffffu, units, o);
+        }
+        if (lane == 0) {
+            alpha[j] = __ddiv_rn((double)cnt, (double)a.r);
+            a.out[1 + j] = alpha[j];
+            draft[j] = a.kind == 0 ? __dadd_rn(__dmul_rn((double)na, ta), __dmul_rn((double)nm, tm)) : (double)units;
+        }
+    }
+    long long all = 0;
+    if (a.kind == 1)
+        for (int i = lane; i < a.n_items; i += 32) all += a.units[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
+    const double tt = a.kind == 0 ? __dmul_rn((double)a.n_layers, __dadd_rn(ta, tm)) : (double)all;
+    __syncthreads();
+    double bv = 0.0;
+    int bi = INT_MAX;
+    auto take = [&](double v, int i) {
+        if (v > bv || (v == bv && i < bi && bi != INT_MAX)) {
+            bv = v;
+            bi = i;
+        }
+    };
+    for (int q = tid; q < a.K * a.D; q += 256) {
+        const int j = q / a.D, gamma = q - j * a.D + 1;
+        double e = 1.0, p = 1.0;
+        for (int g = 1; g <= gamma; ++g) {
+            p = __dmul_rn(p, alpha[j]);
+            e = __dadd_rn(e, p);   // Eq. 1 summed term by term
+        }
+        take(__ddiv_rn(e, __dadd_rn(__dmul_rn((double)gamma, draft[j]), tt)), q);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        take(ov, oi);
+    }
+    if (lane == 0) {
+        best_v[warp] = bv;
+        best_i[warp] = bi;
     }
     __syncthreads();
     if (tid == 0) {
-        double ta = 0.0, tm = 0.0, tt = 0.0;
-        if (a.kind == 0) {
-            ta = __dadd_rn(__dmul_rn(a.c2, (double)a.n), a.c3);
-            tm = a.c1;
-            tt = __dmul_rn((double)a.n_layers, __dadd_rn(ta, tm));
-        } else {
-            for (int i = 0; i < a.n_items; ++i) tt = __dadd_rn(tt, (double)a.units[i]);
-        }
-        int bj = -1, bg = 0;
-        double bv = 0.0;
-        for (int j = 0; j < a.K; ++j) {
-            const uint8_t* m = a.frontier + (size_t)j * a.n_items;
-            double td = 0.0;
-            if (a.kind == 0) {
-                int na = 0, nm = 0;
-                for (int i = 0; i < a.n_items; ++i)
-                    if (m[i]) (i % 2 == 0 ? na : nm)++;
-                td = __dadd_rn(__dmul_rn((double)na, ta), __dmul_rn((double)nm, tm));
-            } else {
-                for (int i = 0; i < a.n_items; ++i)
-                    if (m[i]) td = __dadd_rn(td, (double)a.units[i]);
-            }
-            double e = 1.0, p = 1.0;
-            for (int g = 1; g <= a.D; ++g) {
-                p = __dmul_rn(p, alpha[j]);
-                e = __dadd_rn(e, p);   // Eq. 1 summed term by term
-                const double v = __ddiv_rn(e, __dadd_rn(__dmul_rn((double)g, td), tt));
-                if (v > bv) {
-                    bv = v;
-                    bj = j;
-                    bg = g;
-                }
-            }
-        }
-        a.info[0] = bj;
-        a.info[1] = bg;
+        for (int k = 1; k < 8; ++k) take(best_v[k], best_i[k]);
+        const bool found = bi != INT_MAX;   // false only where the times overflow
+        a.info[0] = found ? bi / a.D : -1;
+        a.info[1] = found ? bi % a.D + 1 : 0;
         a.out[0] = bv;
-        sel = bj;
+        sel = found ? bi / a.D : 0;
     }
     __syncthreads();
     for (int i = tid; i < a.n_items; i += blockDim.x) a.mask_out[i] = a.frontier[(size_t)sel * a.n_items + i];
