@@ -602,14 +602,19 @@ __global__ void __launch_bounds__(128, kAttnCtasPerSm) attn_bf16_kernel(const __
 }
 
 // ----------------------------------------------------------- fp32 kernel
-// One warp per query row at a time; K/V read from the cache (L2).  Used for
-// fp32 models.
+// One warp per query row, K/V read from the cache (L2).  Used for fp32
+// models.  The rows of a (KV head, chunk) are spread over CTAs (blockIdx.z);
+// each CTA writes the chunk's new K/V rows itself before it reads them (the
+// same values everywhere), so none waits for another.  Latency-bound: with all
+// rows of a chunk in one CTA and scalar loads the tiny workload's 5-row verify
+// took 91 us on 6 CTAs; 16-byte loads of K, several V rows in flight and a
+// warp per row take 12.
 template <int HD>
 __global__ void __launch_bounds__(128) attn_f32_kernel(const AttnArgs a) {
     if (a.stop && *a.stop) return;   // a draft pass after the dynamic exit
     constexpr int NPL = HD / 32;
     constexpr int C = 2048;  // largest chunk of the schedule
-    extern __shared__ float fsm[];
+    extern __shared__ __align__(16) float fsm[];
     float* qsh = fsm;                    // [4][HD]
     float* psh = fsm + kAttnWarps * HD;  // [4][C]
     const int h = blockIdx.x, c = my_chunk(a);
@@ -619,6 +624,8 @@ __global__ void __launch_bounds__(128) attn_f32_kernel(const AttnArgs a) {
     const int cs = attn_chunk_start(c);
     const int ce = min(attn_chunk_start(c + 1), a.p0 + a.R);
 
+    grid_launch_dependents();   // the merge may launch: it waits for this grid
+    grid_dependency_wait();     // the projections of this pass
     write_new_kv<float, NPL>(a, h, cs, ce);
     __syncthreads();
 
@@ -628,47 +635,56 @@ __global__ void __launch_bounds__(128) attn_f32_kernel(const AttnArgs a) {
     const float* qn = reinterpret_cast<const float*>(a.q_norm);
     float* q_w = qsh + warp * HD;
     float* p_w = psh + warp * C;
-    for (int m = warp; m < M; m += kAttnWarps) {
-        const int r = m / G, gq = m - r * G;
-        const int pos = a.p0 + r;
-        float q[NPL];
-        head_vector<float, NPL>(a.qkv + (size_t)r * a.qkv_ld + (h * G + gq) * HD, qn, a.eps, a.rope, pos, q);
+    const int m = (int)blockIdx.z * kAttnWarps + warp;
+    if (m >= M) return;
+    const int r = m / G, gq = m - r * G;
+    const int pos = a.p0 + r;
+    float q[NPL];
+    head_vector<float, NPL>(a.qkv + (size_t)r * a.qkv_ld + (h * G + gq) * HD, qn, a.eps, a.rope, pos, q);
 #pragma unroll
-        for (int i = 0; i < NPL; ++i) q_w[lane + 32 * i] = q[i] * qscale;
-        __syncwarp();
-        const int kend = min(ce, pos + 1);
-        float mx = -INFINITY;
-        for (int j = lane; j < ce - cs; j += 32) {
-            const int key = cs + j;
-            float sc = -INFINITY;
-            if (key < kend) {
-                sc = 0.f;
-                const float* kr = kc + (size_t)key * HD;
-                for (int d = 0; d < HD; ++d) sc = fmaf(q_w[d], kr[d], sc);
+    for (int i = 0; i < NPL; ++i) q_w[lane + 32 * i] = q[i] * qscale;
+    __syncwarp();
+    const int kend = min(ce, pos + 1);
+    float mx = -INFINITY;
+    for (int j = lane; j < ce - cs; j += 32) {
+        const int key = cs + j;
+        float sc = -INFINITY;
+        if (key < kend) {
+            sc = 0.f;
+            const float4* kr = reinterpret_cast<const float4*>(kc + (size_t)key * HD);
+#pragma unroll 8
+            for (int d = 0; d < HD / 4; ++d) {
+                const float4 k4 = kr[d], q4 = reinterpret_cast<const float4*>(q_w)[d];
+                sc = fmaf(q4.w, k4.w, fmaf(q4.z, k4.z, fmaf(q4.y, k4.y, fmaf(q4.x, k4.x, sc))));
             }
-            p_w[j] = sc;
-            mx = fmaxf(mx, sc);
         }
-        mx = warp_max(mx);
-        float l = 0.f;
-        for (int j = lane; j < ce - cs; j += 32) {
-            const float p = (mx == -INFINITY || p_w[j] == -INFINITY) ? 0.f : exp2f(p_w[j] - mx);
-            p_w[j] = p;
-            l += p;
-        }
-        l = warp_sum(l);
-        __syncwarp();
-        float* dst = a.part + (((size_t)r * a.hq + h * G + gq) * a.n_chunks_max + c) * (HD + kPartPad);
-        for (int d = lane; d < HD; d += 32) {
-            float acc = 0.f;
-            for (int j = 0; j < kend - cs; ++j) acc = fmaf(p_w[j], vc[(size_t)(cs + j) * HD + d], acc);
-            dst[kPartPad + d] = acc;
-        }
-        if (lane == 0) {
-            dst[0] = mx;
-            dst[1] = l;
-        }
-        __syncwarp();
+        p_w[j] = sc;
+        mx = fmaxf(mx, sc);
+    }
+    mx = warp_max(mx);
+    float l = 0.f;
+    for (int j = lane; j < ce - cs; j += 32) {
+        const float p = (mx == -INFINITY || p_w[j] == -INFINITY) ? 0.f : exp2f(p_w[j] - mx);
+        p_w[j] = p;
+        l += p;
+    }
+    l = warp_sum(l);
+    __syncwarp();
+    float* dst = a.part + (((size_t)r * a.hq + h * G + gq) * a.n_chunks_max + c) * (HD + kPartPad);
+    float acc[NPL];
+#pragma unroll
+    for (int i = 0; i < NPL; ++i) acc[i] = 0.f;
+#pragma unroll 16
+    for (int j = 0; j < kend - cs; ++j) {
+        const float p = p_w[j];
+#pragma unroll
+        for (int i = 0; i < NPL; ++i) acc[i] = fmaf(p, vc[(size_t)(cs + j) * HD + lane + 32 * i], acc[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < NPL; ++i) dst[kPartPad + lane + 32 * i] = acc[i];
+    if (lane == 0) {
+        dst[0] = mx;
+        dst[1] = l;
     }
 }
 
@@ -820,7 +836,6 @@ cudaError_t launch_attn_prep(const AttnArgs& a, cudaStream_t s) {
 cudaError_t launch_attention(int dtype, const AttnArgs& a, cudaStream_t s) {
     const int nch = attn_num_chunks(a.p0 + a.R);
     if (nch > a.n_chunks_max || a.p0 + a.R > a.max_seq) return cudaErrorInvalidValue;
-    dim3 grid(a.hk, nch);
     if (dtype == 1) {
         if (a.q == nullptr || a.err == nullptr) return cudaErrorInvalidValue;
         // query rows per round: 8 NQ (24 at most); each round is its own CTA,
@@ -852,8 +867,16 @@ cudaError_t launch_attention(int dtype, const AttnArgs& a, cudaStream_t s) {
     auto run = [&](auto kern) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        kern<<<grid, 128, smem, s>>>(a);
-        return cudaGetLastError();
+        const int rows = (a.hq / a.hk) * a.R;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(a.hk, nch, (rows + kAttnWarps - 1) / kAttnWarps);
+        cfg.blockDim = dim3(128);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1] = {pdl_attr()};
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kern, a);
     };
     if (a.hd == 128) return run(attn_f32_kernel<128>);
     if (a.hd == 64) return run(attn_f32_kernel<64>);
@@ -865,22 +888,19 @@ cudaError_t launch_attn_merge(int dtype, const AttnArgs& a, cudaStream_t s) {
     const int nch = attn_num_chunks(a.p0 + a.R);
     const size_t smem = sizeof(float) * (size_t)nch;
     if (nch > a.n_chunks_max || smem > 48 * 1024) return cudaErrorInvalidValue;
-    if (dtype == 1) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = grid;
-        cfg.blockDim = dim3(kMergeWarps * 32);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1] = {pdl_attr()};
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (a.hd == 128) return cudaLaunchKernelEx(&cfg, attn_merge_kernel<__nv_bfloat16, 128>, a);
-        return cudaLaunchKernelEx(&cfg, attn_merge_kernel<__nv_bfloat16, 64>, a);
-    } else {
-        if (a.hd == 128) attn_merge_kernel<float, 128><<<grid, kMergeWarps * 32, smem, s>>>(a);
-        else attn_merge_kernel<float, 64><<<grid, kMergeWarps * 32, smem, s>>>(a);
-    }
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kMergeWarps * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1] = {pdl_attr()};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (dtype == 1)
+        return a.hd == 128 ? cudaLaunchKernelEx(&cfg, attn_merge_kernel<__nv_bfloat16, 128>, a)
+                           : cudaLaunchKernelEx(&cfg, attn_merge_kernel<__nv_bfloat16, 64>, a);
+    return a.hd == 128 ? cudaLaunchKernelEx(&cfg, attn_merge_kernel<float, 128>, a)
+                       : cudaLaunchKernelEx(&cfg, attn_merge_kernel<float, 64>, a);
 }
 
 }  // namespace ks

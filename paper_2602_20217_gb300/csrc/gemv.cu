@@ -1,20 +1,23 @@
 // Skinny GEMM kernel for fp32 models (the tiny parity workload), plus the
-// TMA descriptor helper used by the bf16 chain kernel.
+// TMA descriptor helpers of the bf16 kernels.
 //
 // Y[r][n] = sum_k W[n][k] A[r][k] for R <= 16 rows: the per-token
 // projections of the Attn and MLP sublayers and the LM head (Sec. 2 decoder;
-// every pass of a1 / a2).  One CTA per (64-feature group, K slice); each
-// warp computes 16 features with CUDA-core dot products and hands its results
-// over in the mma fragment layout the bf16 path uses, so both share one set
-// of epilogues: plain store (QKV), residual add with optional history capture
-// and partial sums of squares (W_o, W_down), SwiGLU (gate and up rows paired
-// in one warp), LM head logits with a per-row argmax (ties to the lowest id).
-// K slices are added in slice order by the last CTA of a group (an atomic
-// ticket, no waiting): results depend only on (N, K), never on R.  The
-// optional RMSNorm prologue builds each row's sum of squares from the
-// per-16-feature partials that the residual's producer wrote, in group order.
+// every pass of a1 / a2).  A CTA has 16 features, each of its eight warps two
+// (with SwiGLU two gate and two up rows): the lanes stride over K, every row of
+// the pass is accumulated from the same weights in registers, and a butterfly
+// adds the lanes.  The weights of a 512-column chunk are loaded while its
+// activations are staged, the first chunk's before the previous launch is done
+// (programmatic dependent launch).  What bounds it is latency (the tiny workload's
+// matrices are 0.3 to 1.4 MB in L2): one feature after the other per warp, 64 per
+// CTA, with K slices and a last-CTA reduction took 23 to 39 us a launch; this
+// takes 4 to 6.  Results depend only on K, never on R, so rows agree bit
+// for bit between passes of any size.  The optional RMSNorm prologue builds
+// each row's sum of squares from the per-16-feature partials that the
+// residual's producer wrote, in group order.
 #include "common.cuh"
 #include "internal.h"
+#include "tma.cuh"
 
 #include <cudaTypedefs.h>
 
@@ -22,15 +25,14 @@
 
 namespace ks {
 
-constexpr int kGemvWarps = 4;
-constexpr int kRowsPerCta = 16 * kGemvWarps;  // output features per group (CTA or work item)
+constexpr int kGemvWarps = 8;
+constexpr int kGemvThreads = 32 * kGemvWarps;
+constexpr int kFeatures = 2 * kGemvWarps;     // output features per CTA (one sum-of-squares group)
+constexpr int kGemvChunk = 512;               // columns staged at a time
 constexpr int kMaxRows = 16;
-// counters: [0] next work item, [1] finished CTAs, [2 + g] ticket of group g
+static_assert(kFeatures == kSsGroup, "a CTA writes one sum-of-squares group");
 
-__host__ __device__ __forceinline__ int div_up(int a, int b) { return (a + b - 1) / b; }
-
-int gemv_grid_x(int N) { return div_up(N, kRowsPerCta); }
-int gemv_groups(int N, int dtype) { return dtype == 1 ? div_up(N, 16) : div_up(N, kRowsPerCta); }
+int gemv_groups(int N) { return (N + kFeatures - 1) / kFeatures; }
 
 int sm_count() {
     static int n = 0;
@@ -40,218 +42,6 @@ int sm_count() {
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
     }
     return n;
-}
-
-
-void gemv_plan(GemvArgs& a, int epi) {
-    // Depends on (N, K, dtype) only, never on R: the split decides the
-    // summation order, which must be the same for 1 row and gamma + 1 rows.
-    const int gx = gemv_grid_x(a.N);
-    if (a.dtype == 1) {
-        // bf16 streaming kernel: 16-row work items over the full K (the four
-        // consumer warps of a CTA split K inside each stage), no global split
-        a.kc = a.K;
-        a.ksplit = 1;
-        return;
-    }
-    int s = 1;
-    if (epi != EPI_LMHEAD) {
-        s = div_up(5 * 152, gx);
-        if (s > 16) s = 16;
-        if (s < 1) s = 1;
-    }
-    int kc = div_up(div_up(a.K, s), 64) * 64;
-    if (kc < 64) kc = 64;
-    a.kc = kc;
-    a.ksplit = div_up(a.K, kc);
-}
-
-size_t gemv_partial_floats(int N, int K, int R, int epi, int dtype) {
-    GemvArgs a{};
-    a.N = N;
-    a.K = K;
-    a.dtype = dtype;
-    gemv_plan(a, epi);
-    if (a.ksplit <= 1) return 0;
-    return (size_t)a.ksplit * R * N * (epi == EPI_SWIGLU ? 2 : 1);
-}
-
-// --------------------------------------------------------------- prologue
-// Stage A[r][kbeg .. kbeg + kc) for r < R into shared memory (pitch elements
-// per row), applying RMSNorm when norm_gain is set.  Elements past K are 0.
-template <typename WT>
-KS_DEV void stage_activations(const GemvArgs& a, WT* act, int pitch, int kbeg, float* red) {
-    const int tid = threadIdx.x;
-    const int R = a.R;
-    const int kc = a.kc;
-    __syncthreads();  // the previous user of act / red is done
-    if (a.norm_gain != nullptr) {
-        // inv_rms[r] from the producer's per-64-feature partial sums of
-        // squares, added in group order (the same for every CTA and every R)
-        const float* x = reinterpret_cast<const float*>(a.in);
-        const WT* gain = reinterpret_cast<const WT*>(a.norm_gain);
-        if (tid < R) {
-            float s = 0.f;
-            for (int g = 0; g < a.ss_groups; ++g) s += a.ss_in[g * kMaxRows + tid];
-            red[tid] = rsqrtf(s / (float)a.K + a.eps);
-        }
-        __syncthreads();
-        for (int idx = tid; idx < R * kc; idx += blockDim.x) {
-            const int r = idx / kc, k = idx - r * kc;
-            const int kg = kbeg + k;
-            float v = 0.f;
-            if (kg < a.K) v = (x[(size_t)r * a.in_ld + kg] * red[r]) * to_float(gain[kg]);
-            act[r * pitch + k] = from_float<WT>(v);
-        }
-    } else {
-        const WT* in = reinterpret_cast<const WT*>(a.in);
-        for (int idx = tid; idx < R * kc; idx += blockDim.x) {
-            const int r = idx / kc, k = idx - r * kc;
-            const int kg = kbeg + k;
-            act[r * pitch + k] = kg < a.K ? in[(size_t)r * a.in_ld + kg] : from_float<WT>(0.f);
-        }
-    }
-    __syncthreads();
-}
-
-// -------------------------------------------------------------- fp32 rows
-// fp32: the warp computes its 16 rows one at a time (lanes stride over k in
-// float4 steps, butterfly sum), then redistributes the results into the same
-// fragment layout the bf16 path produces.
-template <int NT, bool PAIR>
-KS_DEV void fma_rows(const float* W, int K, int N, int n_base, int kbeg, const float* act,
-                     int pitch, int R, int kc, int kvalid, float* tile /* [2][16][16] per warp */,
-                     float (&acc)[NT][4], float (&accu)[NT][4]) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    for (int half = 0; half < (PAIR ? 2 : 1); ++half) {
-        for (int j = 0; j < 16; ++j) {
-            const int n = n_base + j;
-            float s[kMaxRows];
-#pragma unroll
-            for (int r = 0; r < kMaxRows; ++r) s[r] = 0.f;
-            if (n < N) {
-                const float* wr = W + (size_t)(n + half * N) * K + kbeg;
-                for (int k = 4 * lane; k < kvalid; k += 128) {
-                    const float4 w = *reinterpret_cast<const float4*>(wr + k);
-#pragma unroll
-                    for (int r = 0; r < kMaxRows; ++r) {
-                        if (r < R) {
-                            const float4 x = *reinterpret_cast<const float4*>(act + r * pitch + k);
-                            s[r] = fmaf(w.x, x.x, s[r]);
-                            s[r] = fmaf(w.y, x.y, s[r]);
-                            s[r] = fmaf(w.z, x.z, s[r]);
-                            s[r] = fmaf(w.w, x.w, s[r]);
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < kMaxRows; ++r) {
-                const float v = warp_sum(s[r]);
-                if (lane == 0) tile[(half * 16 + j) * 16 + r] = v;
-            }
-        }
-    }
-    __syncwarp();
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-        const int c = nt * 8 + 2 * t;
-        acc[nt][0] = tile[g * 16 + c];
-        acc[nt][1] = tile[g * 16 + c + 1];
-        acc[nt][2] = tile[(g + 8) * 16 + c];
-        acc[nt][3] = tile[(g + 8) * 16 + c + 1];
-        if (PAIR) {
-            accu[nt][0] = tile[(16 + g) * 16 + c];
-            accu[nt][1] = tile[(16 + g) * 16 + c + 1];
-            accu[nt][2] = tile[(16 + g + 8) * 16 + c];
-            accu[nt][3] = tile[(16 + g + 8) * 16 + c + 1];
-        }
-    }
-}
-
-// --------------------------------------------------------------- epilogue
-template <typename WT, int EPI>
-KS_DEV void apply_epilogue(const GemvArgs& a, int n, int r, float v, float vu) {
-    if (EPI == EPI_STORE) {
-        a.out[(size_t)r * a.out_ld + n] = v;
-    } else if (EPI == EPI_RESID) {
-        float* x = a.resid + (size_t)r * a.resid_ld + n;
-        const float nx = *x + v;
-        *x = nx;
-        if (a.capture) a.capture[(size_t)r * a.capture_ld + n] = nx;
-        if (a.xg_out)
-            a.xg_out[(size_t)r * a.resid_ld + n] =
-                __float2bfloat16_rn(nx * to_float(reinterpret_cast<const __nv_bfloat16*>(a.next_gain)[n]));
-    } else if (EPI == EPI_SWIGLU) {
-        WT* act = reinterpret_cast<WT*>(a.act);
-        act[(size_t)r * a.act_ld + n] = from_float<WT>(silu(v) * vu);
-    }
-}
-
-// After a residual update of features [64 b, 64 b + 64): per row, the sum of
-// squares of the new residual over those features, for the next RMSNorm.
-// Lane l adds features l and l + 32, then a butterfly: a fixed order.
-// Barrier of the 128 threads that own the output fragments: the whole CTA in
-// the fp32 kernel, the four consumer warps (named barrier 1) in the streaming
-// kernel, whose producer warp never joins.
-template <bool CONSUMERS>
-KS_DEV void out_sync() {
-    if (CONSUMERS) asm volatile("bar.sync 1, 128;" ::: "memory");
-    else __syncthreads();
-}
-
-template <bool CONSUMERS = false>
-KS_DEV void residual_sumsq(const GemvArgs& a, int group) {
-    out_sync<CONSUMERS>();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int n0 = group * kRowsPerCta;
-    // 16-feature partials: lanes 0-15 and 16-31 each reduce one half-warp
-    for (int r = warp; r < a.R; r += kGemvWarps) {
-        const float* x = a.resid + (size_t)r * a.resid_ld;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int n = n0 + 32 * h + lane;
-            float s = (n < a.N) ? x[n] * x[n] : 0.f;
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if ((lane & 15) == 0) {
-                const int q = (n0 + 32 * h + lane) / kSsGroup;
-                if (q * kSsGroup < a.N) a.ss_out[q * kMaxRows + r] = s;
-            }
-        }
-    }
-}
-
-// LM head: after the logits of features [64 g, 64 g + 64) are in global memory,
-// each row's best (value, index) of the group -> amax[g][r].
-template <bool CONSUMERS = false>
-KS_DEV void group_argmax(const GemvArgs& a, int group) {
-    out_sync<CONSUMERS>();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int n0 = group * kRowsPerCta;
-    for (int r = warp; r < a.R; r += kGemvWarps) {
-        const float* lg = a.logits + (size_t)r * a.logits_ld;
-        float bv = -INFINITY;
-        int bi = INT_MAX;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int n = n0 + lane + 32 * h;
-            if (n < a.N) {
-                const float v = lg[n];
-                if (better(v, n, bv, bi)) { bv = v; bi = n; }
-            }
-        }
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (better(ov, oi, bv, bi)) { bv = ov; bi = oi; }
-        }
-        if (lane == 0) {
-            a.amax_val[group * kMaxRows + r] = bv;
-            a.amax_idx[group * kMaxRows + r] = bi;
-        }
-    }
 }
 
 // LM head, last CTA of the launch: per row, the best candidate over groups.
@@ -275,94 +65,151 @@ KS_DEV void final_argmax(const GemvArgs& a, int groups) {
     }
 }
 
-// ---------------------------------------------------- fp32 register kernel
-// One CTA per (64-feature group, K slice); used for fp32 models only.
-template <int NT, int EPI>
-__global__ void __launch_bounds__(128) gemv_f32_kernel(const GemvArgs a) {
+// RB: rows the registers have room for (a.R <= RB); a row's arithmetic is the
+// same in each.
+template <int RB, int EPI>
+__global__ void __launch_bounds__(kGemvThreads) gemv_f32_kernel(const GemvArgs a) {
     if (a.stop && *a.stop) return;   // a draft pass after the dynamic exit
-    constexpr bool PAIR = (EPI == EPI_SWIGLU);
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ float red[kGemvWarps * kMaxRows + kMaxRows];
+    constexpr int NW = EPI == EPI_SWIGLU ? 4 : 2;           // weight rows of a warp
+    constexpr int IT = kGemvChunk / 128;                    // float4 steps of a chunk
+    __shared__ __align__(16) float act[RB][kGemvChunk];
+    __shared__ float inv[kMaxRows];
+    __shared__ float val[kFeatures][kMaxRows];              // squares of the new residual, or logits
     __shared__ int is_last;
-
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int g = lane >> 2, t = lane & 3;
-    const int kbeg = blockIdx.y * a.kc;
-    const int kvalid = min(a.kc, a.K - kbeg);
-    const int pitch = a.kc + 4;
-    float* act = reinterpret_cast<float*>(smem);
-    stage_activations<float>(a, act, pitch, kbeg, red);
-
-    const int n_base = blockIdx.x * kRowsPerCta + warp * 16;
-    float acc[NT][4], accu[NT][4];
+    const int R = a.R, n0 = blockIdx.x * kFeatures + 2 * warp;
+    const float* W = reinterpret_cast<const float*>(a.W);
+    const float* in = reinterpret_cast<const float*>(a.in);
+    const float* gain = reinterpret_cast<const float*>(a.norm_gain);
+    const float* row[NW];
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[nt][i] = accu[nt][i] = 0.f;
-    float* tile = reinterpret_cast<float*>(smem + sizeof(float) * (size_t)a.R * pitch) + warp * 2 * 16 * 16;
-    fma_rows<NT, PAIR>(reinterpret_cast<const float*>(a.W), a.K, a.N, n_base, kbeg, act, pitch, a.R, a.kc,
-                       kvalid, tile, acc, accu);
-
-    const int group = blockIdx.x;
-    if (a.ksplit == 1) {
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int n = n_base + g + 8 * (i >> 1);
-                const int r = nt * 8 + 2 * t + (i & 1);
-                if (n < a.N && r < a.R) {
-                    if (EPI == EPI_LMHEAD) a.logits[(size_t)r * a.logits_ld + n] = acc[nt][i];
-                    else apply_epilogue<float, EPI>(a, n, r, acc[nt][i], accu[nt][i]);
-                }
-            }
-    } else {
-        const int NP = PAIR ? 2 * a.N : a.N;
-        float* mine = a.partial + (size_t)blockIdx.y * a.R * NP;
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int n = n_base + g + 8 * (i >> 1);
-                const int r = nt * 8 + 2 * t + (i & 1);
-                if (n < a.N && r < a.R) {
-                    mine[(size_t)r * NP + n] = acc[nt][i];
-                    if (PAIR) mine[(size_t)r * NP + a.N + n] = accu[nt][i];
-                }
-            }
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) is_last = (atomicAdd(&a.counters[2 + group], 1) == a.ksplit - 1);
-        __syncthreads();
-        if (!is_last) return;
-        __threadfence();
-        const int row0 = group * kRowsPerCta;
-        for (int idx = tid; idx < kRowsPerCta * a.R; idx += blockDim.x) {
-            const int r = idx / kRowsPerCta;
-            const int n = row0 + (idx - r * kRowsPerCta);
-            if (n >= a.N) continue;
-            float v = 0.f, vu = 0.f;
-            for (int sl = 0; sl < a.ksplit; ++sl) {
-                const float* pp = a.partial + ((size_t)sl * a.R + r) * NP;
-                v += __ldcg(pp + n);
-                if (PAIR) vu += __ldcg(pp + a.N + n);
-            }
-            if (EPI == EPI_LMHEAD) a.logits[(size_t)r * a.logits_ld + n] = v;
-            else apply_epilogue<float, EPI>(a, n, r, v, vu);
-        }
-        if (tid == 0) a.counters[2 + group] = 0;
+    for (int f = 0; f < NW; ++f) {
+        const int n = min(n0 + (f & 1), a.N - 1);            // a feature past N repeats the last one, unused
+        row[f] = W + (size_t)(n + (f >= 2 ? a.N : 0)) * a.K;
     }
-    if (EPI == EPI_RESID) residual_sumsq(a, group);
-    if (EPI == EPI_LMHEAD) {
-        group_argmax(a, group);
-        __threadfence();
+    grid_launch_dependents();   // the next launch may start: it waits for this one before it reads its input
+    float4 w[IT][NW];
+    auto load_weights = [&](int k0) {
+        const int kq = min(kGemvChunk, a.K - k0) / 4;
+#pragma unroll
+        for (int t = 0; t < IT; ++t)
+#pragma unroll
+            for (int f = 0; f < NW; ++f)
+                if (lane + 32 * t < kq) w[t][f] = *reinterpret_cast<const float4*>(row[f] + k0 + 4 * (lane + 32 * t));
+    };
+    load_weights(0);            // before the previous launch is done
+    grid_dependency_wait();
+    if (gain != nullptr && tid < R) {
+        float s = 0.f;
+#pragma unroll 8
+        for (int g = 0; g < a.ss_groups; ++g) s += a.ss_in[g * kMaxRows + tid];
+        inv[tid] = rsqrtf(s / (float)a.K + a.eps);
+    }
+    float acc[NW][RB];
+#pragma unroll
+    for (int f = 0; f < NW; ++f)
+#pragma unroll
+        for (int r = 0; r < RB; ++r) acc[f][r] = 0.f;
+    for (int k0 = 0; k0 < a.K; k0 += kGemvChunk) {           // K is a multiple of 8
+        const int kq = min(kGemvChunk, a.K - k0) / 4;
+        if (k0 > 0) load_weights(k0);
+        __syncthreads();   // inv is written; the previous chunk's rows are read
+        for (int idx = tid; idx < R * kq; idx += kGemvThreads) {
+            const int r = idx / kq, k = 4 * (idx - r * kq);
+            float4 x = *reinterpret_cast<const float4*>(in + (size_t)r * a.in_ld + k0 + k);
+            if (gain != nullptr) {
+                const float4 g = *reinterpret_cast<const float4*>(gain + k0 + k);
+                const float s = inv[r];
+                x = make_float4((x.x * s) * g.x, (x.y * s) * g.y, (x.z * s) * g.z, (x.w * s) * g.w);
+            }
+            *reinterpret_cast<float4*>(&act[r][k]) = x;
+        }
         __syncthreads();
-        if (tid == 0) is_last = (atomicAdd(&a.counters[1], 1) == (int)(gridDim.x * gridDim.y) - 1);
+#pragma unroll
+        for (int t = 0; t < IT; ++t) {
+            if (lane + 32 * t >= kq) continue;
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+                if (r >= R) continue;
+                const float4 x = *reinterpret_cast<const float4*>(&act[r][4 * (lane + 32 * t)]);
+#pragma unroll
+                for (int f = 0; f < NW; ++f)
+                    acc[f][r] = fmaf(w[t][f].w, x.w,
+                                     fmaf(w[t][f].z, x.z, fmaf(w[t][f].y, x.y, fmaf(w[t][f].x, x.x, acc[f][r]))));
+            }
+        }
+    }
+    // lane r takes row r's sums
+    float v[NW];
+#pragma unroll
+    for (int f = 0; f < NW; ++f) v[f] = 0.f;
+#pragma unroll
+    for (int r = 0; r < RB; ++r) {
+        if (r >= R) continue;
+#pragma unroll
+        for (int f = 0; f < NW; ++f) {
+            const float s = warp_sum(acc[f][r]);
+            if (lane == r) v[f] = s;
+        }
+    }
+    if (lane < R) {
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            const int n = n0 + f, r = lane;
+            const bool ok = n < a.N;
+            if constexpr (EPI == EPI_STORE) {
+                if (ok) a.out[(size_t)r * a.out_ld + n] = v[f];
+            } else if constexpr (EPI == EPI_SWIGLU) {
+                if (ok) reinterpret_cast<float*>(a.act)[(size_t)r * a.act_ld + n] = silu(v[f]) * v[f + 2];
+            } else if constexpr (EPI == EPI_RESID) {
+                float nx = 0.f;
+                if (ok) {
+                    float* x = a.resid + (size_t)r * a.resid_ld + n;
+                    nx = *x + v[f];
+                    *x = nx;
+                    if (a.capture) a.capture[(size_t)r * a.capture_ld + n] = nx;
+                }
+                val[2 * warp + f][r] = nx * nx;
+            } else {
+                if (ok) a.logits[(size_t)r * a.logits_ld + n] = v[f];
+                val[2 * warp + f][r] = ok ? v[f] : -INFINITY;
+            }
+        }
+    }
+    if constexpr (EPI == EPI_RESID) {
+        // the sum of squares of these 16 features, in feature order
+        __syncthreads();
+        if (tid < R) {
+            float s = 0.f;
+#pragma unroll
+            for (int f = 0; f < kFeatures; ++f) s += val[f][tid];
+            a.ss_out[blockIdx.x * kMaxRows + tid] = s;
+        }
+    }
+    if constexpr (EPI == EPI_LMHEAD) {
+        __syncthreads();
+        if (tid < R) {
+            float bv = -INFINITY;
+            int bi = INT_MAX;
+#pragma unroll
+            for (int f = 0; f < kFeatures; ++f) {
+                const int n = blockIdx.x * kFeatures + f;
+                if (n < a.N && better(val[f][tid], n, bv, bi)) {
+                    bv = val[f][tid];
+                    bi = n;
+                }
+            }
+            a.amax_val[blockIdx.x * kMaxRows + tid] = bv;
+            a.amax_idx[blockIdx.x * kMaxRows + tid] = bi;
+            __threadfence();
+        }
+        __syncthreads();
+        if (tid == 0) is_last = (atomicAdd(&a.counters[0], 1) == (int)gridDim.x - 1);
         __syncthreads();
         if (!is_last) return;
         __threadfence();
         final_argmax(a, gridDim.x);
-        if (tid == 0) a.counters[1] = 0;
+        if (tid == 0) a.counters[0] = 0;
     }
 }
 
@@ -456,24 +303,24 @@ bool make_wide_kv_map(CUtensorMap* map, const void* base, uint64_t rows, uint32_
 
 template <int EPI>
 static cudaError_t launch_f32(const GemvArgs& a, cudaStream_t s) {
-    const int pitch = a.kc + 4;
-    const size_t smem = sizeof(float) * ((size_t)a.R * pitch + kGemvWarps * 2 * 16 * 16);
-    dim3 grid(gemv_grid_x(a.N), a.ksplit);
-    auto run = [&](auto kern) -> cudaError_t {
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        kern<<<grid, 128, smem, s>>>(a);
-        return cudaGetLastError();
-    };
-    if (a.R <= 8) return run(gemv_f32_kernel<1, EPI>);
-    return run(gemv_f32_kernel<2, EPI>);
+    const int grid = gemv_groups(a.N);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kGemvThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (a.R == 1) return cudaLaunchKernelEx(&cfg, gemv_f32_kernel<1, EPI>, a);
+    if (a.R <= 8) return cudaLaunchKernelEx(&cfg, gemv_f32_kernel<8, EPI>, a);
+    return cudaLaunchKernelEx(&cfg, gemv_f32_kernel<16, EPI>, a);
 }
 
-cudaError_t launch_gemv(int dtype, int epi, const GemvArgs& a, cudaStream_t s) {
+cudaError_t launch_gemv(int epi, const GemvArgs& a, cudaStream_t s) {
     // fp32 models only; bf16 projections run in the chain kernel
-    if (a.R < 1 || a.R > kMaxRows || a.dtype != dtype || dtype != 0) return cudaErrorInvalidValue;
+    if (a.R < 1 || a.R > kMaxRows) return cudaErrorInvalidValue;
     switch (epi) {
         case EPI_STORE: return launch_f32<EPI_STORE>(a, s);
         case EPI_RESID: return launch_f32<EPI_RESID>(a, s);

@@ -11,45 +11,36 @@
 namespace ks {
 
 // ------------------------------------------------------------------ GEMV
-// Y[r][n] = sum_k W[n][k] * A[r][k] for r < R rows ("skinny GEMM"), with a
-// fused prologue (optional RMSNorm of an fp32 residual input) and epilogue.
+// fp32 models: Y[r][n] = sum_k W[n][k] * A[r][k] for r < R rows ("skinny
+// GEMM"), with a fused prologue (optional RMSNorm of a residual input) and
+// epilogue.
 enum GemvEpi { EPI_STORE = 0, EPI_RESID = 1, EPI_SWIGLU = 2, EPI_LMHEAD = 3 };
 
 struct GemvArgs {
-    int dtype;              // KS_DTYPE_F32 / KS_DTYPE_BF16 (selects kernel and split plan)
-    const void* W;          // [N (or 2N for SwiGLU)][K], row stride K, model dtype
+    const void* W;          // [N (or 2N for SwiGLU)][K], row stride K
     int N;                  // output features (SwiGLU: d_ff; rows n and N + n pair up)
     int K;
     int R;                  // activation rows, 1..16
-    int ksplit;             // K slices (grid.y); set by gemv_plan
-    int kc;                 // K per slice (multiple of 64)
-    const void* in;         // fp32: the residual [R][in_ld] when norm_gain != null, else the input;
-                            // bf16: the input in bf16 [R][in_ld] (x * gain when ss_in != null)
+    const void* in;         // [R][in_ld]: the residual when norm_gain != null, else the input
     int in_ld;
-    const void* norm_gain;  // RMSNorm gain [K] (model dtype) or null
+    const void* norm_gain;  // RMSNorm gain [K] or null
     float eps;
-    const float* ss_in;     // with norm_gain: per-64-feature sums of squares [ss_groups][16]
+    const float* ss_in;     // with norm_gain: per-16-feature sums of squares [ss_groups][16]
     int ss_groups;
     float* ss_out;          // EPI_RESID: sums of squares of the new residual [groups][16]
-    __nv_bfloat16* xg_out;  // EPI_RESID (bf16): new residual times next_gain, the next GEMV's input
-    const void* next_gain;  // gain of the next RMSNorm (model dtype)
-    int* err;               // device status word: set to 1 when a bounded wait gives up
     const int* stop;        // draft passes: the pass is skipped when *stop != 0 (null: always run)
-    float* out; int out_ld;                    // EPI_STORE (fp32)
+    float* out; int out_ld;                    // EPI_STORE
     float* resid; int resid_ld;                // EPI_RESID: resid[r][n] += y
     float* capture; long long capture_ld;      // EPI_RESID: optional copy of the new residual
-    void* act; int act_ld;                     // EPI_SWIGLU: silu(gate) * up, model dtype
+    void* act; int act_ld;                     // EPI_SWIGLU: silu(gate) * up
     float* logits; int logits_ld;              // EPI_LMHEAD
     float* amax_val; int* amax_idx;            // EPI_LMHEAD per-group candidates [groups][16]
     int* tokens;                               // EPI_LMHEAD argmax per row
-    float* partial;                            // split-K partials [ksplit][R][N or 2N]
-    int* counters;                             // [0] work queue, [1] finished CTAs, [2 + g] group tickets
+    int* counters;                             // EPI_LMHEAD: [0] finished CTAs, zero between launches
 };
 
-void gemv_plan(GemvArgs& a, int epi);           // choose ksplit / kc from (N, K, dtype) only
-size_t gemv_partial_floats(int N, int K, int R, int epi, int dtype);
-int gemv_grid_x(int N);
-cudaError_t launch_gemv(int dtype, int epi, const GemvArgs& a, cudaStream_t s);
+int gemv_groups(int N);     // CTAs of a launch (argmax candidates, sum-of-squares groups)
+cudaError_t launch_gemv(int epi, const GemvArgs& a, cudaStream_t s);
 // TMA map of a row-major bf16 matrix [rows][K] (K % 8 == 0, 16-byte aligned
 // base), box 256 columns x box_rows rows, no swizzle, zero fill outside.
 bool make_tma_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K, uint32_t box_rows);
@@ -67,7 +58,6 @@ bool make_weight_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t
 // swizzle (an operand's stage), and 128 whole cache rows of hd elements.
 bool make_wide_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K);
 bool make_wide_kv_map(CUtensorMap* map, const void* base, uint64_t rows, uint32_t hd);
-int gemv_groups(int N, int dtype);              // output groups (argmax candidates) of a launch
 
 // ----------------------------------------------------------------- chain
 // bf16 models: a run of consecutive projections (phases) in one persistent

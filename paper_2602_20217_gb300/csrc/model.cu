@@ -192,13 +192,11 @@ __global__ void __launch_bounds__(256) tpt_states_kernel(const float* hist, long
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct Layout {
-    size_t kv, rope, x, ss, xg, qkv, attn_out, act, attn_part, gemv_part, counters, logits, amax_val,
+    size_t kv, rope, x, ss, xg, qkv, attn_out, act, attn_part, counters, logits, amax_val,
         amax_idx, tok, hist, hist_snap, hist_idx, sims, mask, obj, wts, select, chain_ctr, best, tpt_masks,
         tpt_tok, tpt_info, tpt_out, dyn, samp, slice, qbuf, wide, wide_part, wide_ticket, total;
     int wide_rows;   // rows of a wide chunk (0: fp32 models, no wide path)
     int n_chunks_max;
-    size_t gemv_part_floats;
-    int counters_n;
     int hist_slots;
 };
 
@@ -298,19 +296,6 @@ static Layout make_layout(const ks_config* c) {
     const int nsub = 2 * c->n_layers;
     L.n_chunks_max = attn_num_chunks(c->max_seq);
     L.hist_slots = c->hist_steps + 1;
-    size_t gp = 0;
-    gp = std::max(gp, gemv_partial_floats(nqkv, d, R, EPI_STORE, c->dtype));
-    gp = std::max(gp, gemv_partial_floats(d, c->n_q_heads * hd, R, EPI_RESID, c->dtype));
-    gp = std::max(gp, gemv_partial_floats(c->d_ff, d, R, EPI_SWIGLU, c->dtype));
-    gp = std::max(gp, gemv_partial_floats(d, c->d_ff, R, EPI_RESID, c->dtype));
-    gp = std::max(gp, gemv_partial_floats(c->vocab, d, R, EPI_LMHEAD, c->dtype));
-    L.gemv_part_floats = gp;
-    int gx = gemv_grid_x(c->vocab);
-    gx = std::max(gx, gemv_grid_x(nqkv));
-    gx = std::max(gx, gemv_grid_x(c->d_ff));
-    gx = std::max(gx, gemv_grid_x(d));
-    L.counters_n = gx + 2;
-
     size_t off = 0;
     auto take = [&](size_t bytes) {
         size_t o = off;
@@ -325,10 +310,10 @@ static Layout make_layout(const ks_config* c) {
     L.qkv = take(sizeof(float) * (size_t)R * nqkv);
     L.attn_out = take(es * (size_t)R * c->n_q_heads * hd);
     L.act = take(es * (size_t)R * c->d_ff);
-    L.gemv_part = take(sizeof(float) * std::max<size_t>(gp, 1));
-    L.counters = take(sizeof(int) * (size_t)L.counters_n);
-    L.amax_val = take(sizeof(float) * (size_t)gemv_groups(c->vocab, c->dtype) * 16);
-    L.amax_idx = take(sizeof(int) * (size_t)gemv_groups(c->vocab, c->dtype) * 16);
+    // fp32 LM head: finished CTAs, per-group argmax candidates
+    L.counters = take(sizeof(int));
+    L.amax_val = take(sizeof(float) * (size_t)gemv_groups(c->vocab) * 16);
+    L.amax_idx = take(sizeof(int) * (size_t)gemv_groups(c->vocab) * 16);
     // tokens: rows[R+1] | target[R] | result[R+3] | err | prompt/out[max_seq]
     L.tok = take(sizeof(int) * ((size_t)3 * R + 8 + c->max_seq));
     // A prefill's wide chunks use the space of what is dead until they are
@@ -398,7 +383,7 @@ struct ks_model {
     Layout lay;
     // carved pointers
     char* kv;
-    float *rope, *x, *ss, *qkv, *attn_part, *gemv_part, *logits, *amax_val, *hist, *hist_snap, *sims;
+    float *rope, *x, *ss, *qkv, *attn_part, *logits, *amax_val, *hist, *hist_snap, *sims;
     __nv_bfloat16* xg;
     void *attn_out, *act, *select;
     int *counters, *amax_idx, *rows, *target, *result, *err, *seq, *hist_idx;
@@ -540,14 +525,9 @@ static ks_status forward(ks_model* m, const int32_t* tok, int R, int p0, const u
         g.ss_in = m->ss;
         g.ss_groups = ssg;
         g.eps = c.rms_eps;
-        if (bf) {
-            g.in = m->xg;       // x * gain in bf16, scaled by 1 / rms in the epilogue
-            g.in_ld = d;
-        } else {
-            g.in = m->x;        // fp32 kernel normalises while staging
-            g.in_ld = d;
-            g.norm_gain = gain;
-        }
+        g.in = m->x;            // normalised while it is staged
+        g.in_ld = d;
+        g.norm_gain = gain;
     };
     auto resid_output = [&](GemvArgs& g, int after) {
         g.resid = m->x;
@@ -555,20 +535,13 @@ static ks_status forward(ks_model* m, const int32_t* tok, int R, int p0, const u
         g.ss_out = m->ss;
         g.capture = cap_ptr(after);
         g.capture_ld = d;
-        if (bf) {
-            g.xg_out = m->xg;
-            g.next_gain = next_gain(after);
-        }
     };
     auto common = [&](GemvArgs& g, const void* W, int N, int K) {
         g.W = W;
-        g.dtype = dt;
         g.N = N;
         g.K = K;
         g.R = R;
-        g.partial = m->gemv_part;
         g.counters = m->counters;
-        g.err = m->err;
         g.stop = stop;
     };
     KS_TRY(launch(m, K_EMBED, [&]() -> cudaError_t {
@@ -705,16 +678,14 @@ static ks_status forward(ks_model* m, const int32_t* tok, int R, int p0, const u
             norm_input(g, m->attn_norm[l]);
             g.out = m->qkv;
             g.out_ld = nqkv;
-            gemv_plan(g, EPI_STORE);
-            KS_TRY(launch(m, K_QKV, [&] { return launch_gemv(dt, EPI_STORE, g, s); }, "qkv"));
+            KS_TRY(launch(m, K_QKV, [&] { return launch_gemv(EPI_STORE, g, s); }, "qkv"));
             KS_TRY(attention(l));
             GemvArgs o{};
             common(o, m->w_o[l], d, c.n_q_heads * hd);
             o.in = m->attn_out;
             o.in_ld = c.n_q_heads * hd;
             resid_output(o, 2 * l + 1);
-            gemv_plan(o, EPI_RESID);
-            KS_TRY(launch(m, K_OPROJ, [&] { return launch_gemv(dt, EPI_RESID, o, s); }, "o-proj"));
+            KS_TRY(launch(m, K_OPROJ, [&] { return launch_gemv(EPI_RESID, o, s); }, "o-proj"));
         }
         if (run_mlp) {
             GemvArgs gu{};
@@ -722,15 +693,13 @@ static ks_status forward(ks_model* m, const int32_t* tok, int R, int p0, const u
             norm_input(gu, m->mlp_norm[l]);
             gu.act = m->act;
             gu.act_ld = c.d_ff;
-            gemv_plan(gu, EPI_SWIGLU);
-            KS_TRY(launch(m, K_GATEUP, [&] { return launch_gemv(dt, EPI_SWIGLU, gu, s); }, "gate-up"));
+            KS_TRY(launch(m, K_GATEUP, [&] { return launch_gemv(EPI_SWIGLU, gu, s); }, "gate-up"));
             GemvArgs dn{};
             common(dn, m->w_down[l], d, c.d_ff);
             dn.in = m->act;
             dn.in_ld = c.d_ff;
             resid_output(dn, 2 * l + 2);
-            gemv_plan(dn, EPI_RESID);
-            KS_TRY(launch(m, K_DOWN, [&] { return launch_gemv(dt, EPI_RESID, dn, s); }, "down"));
+            KS_TRY(launch(m, K_DOWN, [&] { return launch_gemv(EPI_RESID, dn, s); }, "down"));
         }
     }
     if (argmax) {
@@ -742,8 +711,7 @@ static ks_status forward(ks_model* m, const int32_t* tok, int R, int p0, const u
         lm.amax_val = m->amax_val;
         lm.amax_idx = m->amax_idx;
         lm.tokens = argmax;
-        gemv_plan(lm, EPI_LMHEAD);
-        KS_TRY(launch(m, K_LMHEAD, [&] { return launch_gemv(dt, EPI_LMHEAD, lm, s); }, "lm-head"));
+        KS_TRY(launch(m, K_LMHEAD, [&] { return launch_gemv(EPI_LMHEAD, lm, s); }, "lm-head"));
     }
     m->last_pass_rows = R;
     return KS_OK;
@@ -936,7 +904,6 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
     m->attn_out = b + lay.attn_out;
     m->act = b + lay.act;
     m->attn_part = reinterpret_cast<float*>(b + lay.attn_part);
-    m->gemv_part = reinterpret_cast<float*>(b + lay.gemv_part);
     m->counters = reinterpret_cast<int*>(b + lay.counters);
     m->logits = reinterpret_cast<float*>(b + lay.logits);
     m->amax_val = reinterpret_cast<float*>(b + lay.amax_val);
@@ -1063,7 +1030,7 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
         e = cudaStreamSynchronize(m->stream);
         if (e != cudaSuccess) return fail(e, "rope upload");
     }
-    e = cudaMemsetAsync(m->counters, 0, sizeof(int) * lay.counters_n, m->stream);
+    e = cudaMemsetAsync(m->counters, 0, sizeof(int), m->stream);
     if (e != cudaSuccess) return fail(e, "counter reset");
     // The bf16 attention streams whole 16-key tiles; keys past a row's
     // position are masked (softmax weight exactly 0), which needs finite
@@ -1552,13 +1519,10 @@ static ks_status lm_head_rows(ks_model* m, int R, int32_t* tokens) {
     }
     GemvArgs g{};
     g.W = m->lm_head;
-    g.dtype = m->dtype;
     g.N = c.vocab;
     g.K = d;
     g.R = R;
-    g.partial = m->gemv_part;
     g.counters = m->counters;
-    g.err = m->err;
     g.ss_in = m->ss;
     g.ss_groups = (d + kSsGroup - 1) / kSsGroup;
     g.eps = c.rms_eps;
@@ -1570,8 +1534,7 @@ static ks_status lm_head_rows(ks_model* m, int R, int32_t* tokens) {
     g.amax_val = m->amax_val;
     g.amax_idx = m->amax_idx;
     g.tokens = tokens;
-    gemv_plan(g, EPI_LMHEAD);
-    return launch(m, K_LMHEAD, [&] { return launch_gemv(m->dtype, EPI_LMHEAD, g, s); }, "tpt lm-head");
+    return launch(m, K_LMHEAD, [&] { return launch_gemv(EPI_LMHEAD, g, s); }, "tpt lm-head");
 }
 
 // LM head argmax of many rows (bf16 models): buffers in the space of the
