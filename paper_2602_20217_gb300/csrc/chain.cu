@@ -18,18 +18,20 @@
 //    2-D TMA weight boxes into a ring of shared-memory stages;
 //  * warp 5 (activations): follows the same stage sequence; before a stage
 //    it waits until the block of the previous phase's output that the stage
-//    reads is complete, then issues the stage's activation boxes;
+//    reads is complete (its lanes look at all blocks at once: one block and one
+//    round trip per stage held a phase's first item up by 1.4 us a stage), then
+//    issues the stage's activation boxes;
 //  * warps 0-3 (consumers): mma.sync m16n8k16 with weights as A and the R
 //    activation rows as B (columns independent: batch invariant), each warp
-//    a quarter of every stage's columns,
+//    a quarter of every stage's columns and at its own pace,
 //    then hand each item's per-warp sums to
 //  * warp 6 (epilogue): adds them in warp order (fixed), computes the rows'
 //    1/rms at its first item of a normed phase (normalised inputs), runs the
-//    fused epilogue, and after the CTA's last item of a phase adds its item count
-//    to the phase's done-counter (one release per CTA and phase).  LM head:
-//    each CTA keeps its best (logit, id) per row and merges it into a 64-bit
-//    key with atomicMax (value first, then the lower id: any merge order gives
-//    the same argmax); the CTA whose count completes the phase reads it.
+//    fused epilogue, and publishes the row group to the next phase.  LM head:
+//    each CTA keeps its best (logit, id) per row and, after its last item,
+//    merges it into a 64-bit key with atomicMax (value first, then the lower
+//    id: any merge order gives the same argmax) and counts its items; the CTA
+//    whose count completes the phase reads the keys.
 //    Partials are double buffered, so consumers never wait for an epilogue.
 // A stage is full when both loaders have arrived and all bytes have landed.
 // A CTA's first unit of each phase is fixed by its index; further units are
@@ -100,10 +102,10 @@ KS_DEV Phase decode(const ChainArgs& a, int k) {
         }
     }
     p.n_items = (p.N + 15) >> 4;
-    const int cols = p.kind == CH_GU ? 512 : 1024;   // k columns per stage
-    p.tpi = (p.K + cols - 1) / cols;
+    const int shift = p.kind == CH_GU ? 9 : 10;      // k columns per stage: 512 or 1024
+    p.tpi = (p.K + (1 << shift) - 1) >> shift;
     p.n_sl = ((p.kind == CH_O || p.kind == CH_DOWN) && p.n_items <= kSliceMaxItems && p.tpi >= 8) ? 2 : 1;
-    p.sl_len = (p.tpi + p.n_sl - 1) / p.n_sl;
+    p.sl_len = (p.tpi + p.n_sl - 1) >> (p.n_sl - 1);
     p.n_units = p.n_items * p.n_sl;
     return p;
 }
@@ -123,10 +125,8 @@ KS_DEV int block_rowgroups(int n_out, int cols, int b) {   // row groups of bloc
 KS_DEV const CUtensorMap* amap_of(const ChainArgs& a, int kind) {
     return &a.amap[kind == CH_GU ? 1 : kind == CH_O ? 2 : kind == CH_DOWN ? 3 : 0];
 }
-// K % 256 == 0: the activation map is 3-D and a stage is one copy
-KS_DEV bool stage_maps(const Phase& P) { return (P.K & 255) == 0; }
-// K % 64 == 0: the weight map is 3-D and a stage's weights are one copy
-KS_DEV bool weight_3d(const Phase& P) { return (P.K & 63) == 0; }
+// K % 64 == 0: the maps are 3-D and a stage's weights or activations one copy
+KS_DEV bool maps_3d(const Phase& P) { return (P.K & 63) == 0; }
 
 // Independent accumulator chains per consumer warp: the MMAs of a stage go
 // round-robin to kChains accumulators, so consecutive MMAs do not wait on each
@@ -136,38 +136,53 @@ KS_DEV bool weight_3d(const Phase& P) { return (P.K & 63) == 0; }
 constexpr int kChains = 2;
 
 // One stage of one consumer warp: its quarter of the stage's columns.
+// Weights and activations lie in 64-column chunks (16 and R rows of 128 bytes)
+// under the 128-byte swizzle, which goes by shared-memory address: 16-byte unit
+// u of the row at byte offset o (from a multiple of 1024) is at unit
+// u ^ ((o >> 7) & 7).  ldmatrix reads eight rows of one unit at a time, eight
+// different bank groups; 16-byte loads per lane in the MMA's row order met two
+// rows in the same banks, and with a barrier of the four warps per stage a
+// stage took 1.3 us from shared memory: no catching up after a wait at HBM's
+// pace of 1.47 us.  A decode layer (Llama-3-8B shape, 4k context) went from
+// 100.5 to 95.2 us, a verify layer of 5 rows from 119 to 108, of 11 from 175 to 133.
 template <int NT, bool PAIR>
-KS_DEV void mma_stage(const __nv_bfloat16* st, int R, int warp, int lane, float (&acc)[kChains][NT][4],
+KS_DEV void mma_stage(uint32_t st, int R, int warp, int lane, float (&acc)[kChains][NT][4],
                       float (&accu)[kChains][NT][4]) {
-    constexpr int kNB = PAIR ? 2 : 4;              // 256-column activation boxes per stage
-    constexpr int kWarpCols = 256 * kNB / 4;
-    const int g = lane >> 2, t4 = lane & 3;
-    const int wb = (warp * kWarpCols) / 256, wc = (warp * kWarpCols) % 256;
-    // weights: chunk c (64 columns) of 16 rows at c * 2 KB, row r at r * 128 B,
-    // 16-byte unit u at (u ^ (r & 7)) * 16; rows g and g + 8 share the XOR
-    const unsigned char* wbase = reinterpret_cast<const unsigned char*>(st) + g * 128;
-    const __nv_bfloat16* ap = st + 4 * kBoxElems + wb * (256 * R) + g * 256 + wc + 8 * t4;
-    const uint4 z = make_uint4(0, 0, 0, 0);
+    constexpr int kWarpCols = PAIR ? 128 : 256;
+    // weights: matrix l >> 3 of a 16 x 16 step is rows (l >> 3 & 1) * 8 .., unit l >> 4
+    const int wrow = (lane & 7) + ((lane >> 3) & 1) * 8;
+    const uint32_t wbase = st + wrow * 128;
+    const int wkey = lane & 7, wunit = lane >> 4;
+    // activations: matrix l >> 3 of a 32-column step is its unit; rows past R repeat row 0 (their
+    // columns of the product are not used)
+    const int aunit = lane >> 3;
+    int arow[NT];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+        const int r = nt * 8 + (lane & 7);
+        arow[nt] = r < R ? r : 0;
+    }
+    const uint32_t abase = st + kWBytes;
 #pragma unroll
     for (int ks = 0; ks < kWarpCols / 32; ++ks) {
         const int j0 = warp * kWarpCols + 32 * ks;               // first column of the step
-        const int off = (j0 >> 6) * kChunkBytes + (((((j0 & 63) >> 3) + t4) ^ g) << 4);
-        const uint4 w0 = lds128(wbase + off);
-        const uint4 w1 = lds128(wbase + off + 8 * 128);
-        uint4 u0 = z, u1 = z;
-        if (PAIR) {   // up rows: the second half of the stage (8 chunks on)
-            u0 = lds128(wbase + 8 * kChunkBytes + off);
-            u1 = lds128(wbase + 8 * kChunkBytes + off + 8 * 128);
+        const int c = j0 >> 6, u0 = (j0 & 63) >> 3;
+        uint32_t w[2][4], u[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t off = wbase + c * kChunkBytes + (((u0 + 2 * h + wunit) ^ wkey) << 4);
+            ldsm_x4(w[h], off);
+            if (PAIR) ldsm_x4(u[h], off + 8 * kChunkBytes);      // up rows: the second half of the stage
         }
-        const int c0 = (2 * ks) % kChains, c1 = (2 * ks + 1) % kChains;   // constants once unrolled
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
-            const uint4 bv = (nt * 8 + g < R) ? lds128(ap + nt * 8 * 256 + 32 * ks) : z;
-            mma_bf16(acc[c0][nt], w0.x, w1.x, w0.y, w1.y, bv.x, bv.y);
-            mma_bf16(acc[c1][nt], w0.z, w1.z, w0.w, w1.w, bv.z, bv.w);
-            if (PAIR) {
-                mma_bf16(accu[c0][nt], u0.x, u1.x, u0.y, u1.y, bv.x, bv.y);
-                mma_bf16(accu[c1][nt], u0.z, u1.z, u0.w, u1.w, bv.z, bv.w);
+            const int q = c * R + arow[nt];                      // 128-byte row of the activations
+            uint32_t b[4];
+            ldsm_x4(b, abase + q * 128 + (((u0 + aunit) ^ (q & 7)) << 4));
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                mma_bf16(acc[h][nt], w[h][0], w[h][1], w[h][2], w[h][3], b[2 * h], b[2 * h + 1]);
+                if (PAIR) mma_bf16(accu[h][nt], u[h][0], u[h][1], u[h][2], u[h][3], b[2 * h], b[2 * h + 1]);
             }
         }
     }
@@ -276,7 +291,7 @@ KS_DEV void row_scales(const ChainArgs& a, int lane, float* out) {
     float s[kRows];
 #pragma unroll
     for (int r = 0; r < kRows; ++r) s[r] = 0.f;
-#pragma unroll 2
+#pragma unroll 8
     for (int q = lane; q < groups; q += 32) {
         const float4* src = reinterpret_cast<const float4*>(a.ss + (size_t)q * kMaxRows);
 #pragma unroll
@@ -300,19 +315,23 @@ KS_DEV void row_scales(const ChainArgs& a, int lane, float* out) {
     __syncwarp();
 }
 
-// One thread per CTA, as the CTA leaves: the last CTA of the launch to leave
-// resets the queues and counters of its counter set for a later launch.
+// The whole CTA, as it leaves: the last CTA of the launch to leave resets the
+// queues and counters of its counter set for a later launch (with all its
+// threads: the launch is complete, and its dependents may go on, only then).
 KS_DEV void count_out(int n_phases, int* queue, int* done, int* exits, int* blocks) {
+    __shared__ int last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(exits, 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
     __threadfence();
-    if (atomicAdd(exits, 1) == (int)gridDim.x - 1) {
-        __threadfence();
-        for (int k = 0; k < n_phases; ++k) {
-            queue[k] = 0;
-            done[k] = 0;
-            for (int b = 0; b < kMaxBlocks; ++b) blocks[k * kMaxBlocks + b] = 0;
-        }
+    for (int i = threadIdx.x; i < n_phases * kMaxBlocks; i += kThreads) blocks[i] = 0;
+    for (int i = threadIdx.x; i < n_phases; i += kThreads) queue[i] = 0;
+    if (threadIdx.x == 0) {
+        *done = 0;
         *exits = 0;
-        __threadfence();
     }
 }
 
@@ -343,9 +362,9 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
     const int R = a.R, S = a.stages;
     const int stage_elems = 4 * kBoxElems + 4 * 256 * R;
     int* queue = a.counters;
-    int* done = a.counters + kChainMaxPhases;
-    int* exits = a.counters + 2 * kChainMaxPhases;
-    int* blocks = a.counters + 2 * kChainMaxPhases + 1;   // [phase][kMaxBlocks]
+    int* done = a.counters + kChainMaxPhases;             // LM head items finished
+    int* exits = a.counters + kChainMaxPhases + 1;
+    int* blocks = a.counters + kChainMaxPhases + 2;       // [phase][kMaxBlocks]
 
     if (tid == 0) {
         // A job whose status word already holds an error is void (the word
@@ -369,7 +388,7 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
     if (tid < kMaxRows) ones[tid] = 1.f;
     __syncthreads();
     if (void_job) {   // still counted out, so the launch's counters are reset
-        if (tid == 0) count_out(a.n_phases, queue, done, exits, blocks);
+        count_out(a.n_phases, queue, done, exits, blocks);
         return;
     }
 
@@ -396,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                 __nv_bfloat16* st = ring + (size_t)slot * stage_elems;
                 const CUtensorMap* wm = &a.wmap[k];
                 unsigned char* sb = reinterpret_cast<unsigned char*>(st);
-                if (weight_3d(P)) {
+                if (maps_3d(P)) {
                     if (P.kind == CH_GU) {   // 8 gate chunks, then 8 up chunks
                         tma_3d(sb, wm, 0, it * 16, 8 * kt, &full[slot]);
                         tma_3d(sb + 8 * kChunkBytes, wm, 0, P.N + it * 16, 8 * kt, &full[slot]);
@@ -445,7 +464,7 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                 // slice-major: every item's first K-slice comes before any
                 // second one, so the units taken first (one per CTA) read the
                 // previous phase's first blocks, which complete first
-                const int sl = it / P.n_items, item = it - sl * P.n_items;
+                const int sl = it >= P.n_items, item = sl ? it - P.n_items : it;
                 const int kt0 = sl * P.sl_len, kt1 = min(P.tpi, kt0 + P.sl_len);
                 for (int kt = kt0; kt < kt1 && ok; ++kt)
                     ok = issue(k, P, item, kt, sl, kt == kt1 - 1 && next >= P.n_units);
@@ -469,16 +488,18 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
         }
     } else if (warp == kWarpA) {
         // ---------------------------------------------- activation loader
+        // Every lane waits for a stage's record itself: when lane 0 waited and
+        // a shuffle told the others (which orders no memory), they read the
+        // record unsynchronised, and a lane that saw the slot's previous stage
+        // could leave for the exit barrier alone, with lane 0 left for ever at
+        // the next warp-wide operation.
         grid_dependency_wait();   // the first phase's input comes from the previous kernel
-        int cur = -1, ready = 0;
+        int cur = -1, ready = 0, prev_n = 0;
+        Phase P;
         bool ok = true;
         for (int t = 0;; ++t) {
             const int slot = t % S;
-            // lane 0 waits; the shuffle broadcasts the outcome and orders the
-            // other lanes' reads of the slot after it
-            bool got = true;
-            if (lane == 0) got = mbar_wait(&pub[slot], (uint32_t)((t / S) & 1), kWaitLimitNs);
-            if (!__shfl_sync(0xffffffffu, (int)got, 0)) {
+            if (!__all_sync(0xffffffffu, mbar_wait(&pub[slot], (uint32_t)((t / S) & 1), kWaitLimitNs))) {
                 ok = false;
                 break;
             }
@@ -488,60 +509,71 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                 break;
             }
             const int kt = slot_kt[slot];
-            if (k >= a.n_phases || kt < 0) {   // self-check of the stage record
-                if (lane == 0) set_err(a.err, kErrCheckA);
-                ok = false;
-                break;
-            }
-            const Phase P = decode(a, k);
-            if (kt >= P.tpi) {
+            if (k >= a.n_phases || kt < 0) {   // self-check of the stage record (the same in every lane)
                 if (lane == 0) set_err(a.err, kErrCheckA);
                 ok = false;
                 break;
             }
             if (k != cur) {
                 cur = k;
+                P = decode(a, k);
+                prev_n = k > 0 ? decode(a, k - 1).N : 0;
                 ready = 0;      // blocks of phase k - 1 known to be complete
             }
+            if (kt >= P.tpi) {
+                if (lane == 0) set_err(a.err, kErrCheckA);
+                ok = false;
+                break;
+            }
             if (k > 0 && kt >= ready) {
-                // wait for the block of phase k - 1 that this stage reads
-                const int n_prev = decode(a, k - 1).N;
-                bool dep = true;
-                if (lane == 0)
-                    dep = wait_at_least(&blocks[(k - 1) * kMaxBlocks + kt],
-                                        block_rowgroups(n_prev, stage_cols(P.kind), kt), kWaitLimitNs);
-                if (!__shfl_sync(0xffffffffu, (int)dep, 0)) {
-                    ok = false;
-                    break;
+                // wait for the block of phase k - 1 that this stage reads; the
+                // lanes look at the blocks from `ready` on together, so that
+                // one round trip finds all that are complete
+                const uint64_t t0 = global_ns();
+                for (;;) {
+                    const int b = ready + lane;
+                    const bool done_b = b < P.tpi && ld_relaxed(&blocks[(k - 1) * kMaxBlocks + b]) >=
+                                                         block_rowgroups(prev_n, stage_cols(P.kind), b);
+                    const uint32_t open = ~__ballot_sync(0xffffffffu, done_b);
+                    ready += open == 0 ? 32 : __ffs(open) - 1;
+                    if (ready > kt) break;
+                    if (__any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) {
+                        ok = false;
+                        break;
+                    }
                 }
+                if (!ok) break;
+                fence_acq_rel();             // the counters were read relaxed: order the rows behind them
                 fence_proxy_async_global();
-                if (kt == ready) ++ready;   // stages of an item come in order
+                __syncwarp();
             }
             if (lane == 0) {
-                const int nb = (P.kind == CH_GU) ? 2 : 4;
-                const int cols = 256 * nb;
-                mbar_expect_tx(&full[slot], (uint32_t)(nb * 256 * R * 2));
-                __nv_bfloat16* dst = ring + (size_t)slot * stage_elems + 4 * kBoxElems;
+                const int chunks = P.kind == CH_GU ? 8 : 16;
+                mbar_expect_tx(&full[slot], (uint32_t)(chunks * 128 * R));
+                unsigned char* dst = reinterpret_cast<unsigned char*>(ring + (size_t)slot * stage_elems) + kWBytes;
                 const CUtensorMap* am = amap_of(a, P.kind);
-                if (stage_maps(P)) tma_3d(dst, am, 0, 0, nb * kt, &full[slot]);
-                else for (int b = 0; b < nb; ++b) tma_2d(dst + b * 256 * R, am, kt * cols + 256 * b, 0, &full[slot]);
+                if (maps_3d(P)) tma_3d(dst, am, 0, 0, chunks * kt, &full[slot]);
+                else for (int c = 0; c < chunks; ++c) tma_2d(dst + c * 128 * R, am, (chunks * kt + c) * 64, 0, &full[slot]);
             }
             __syncwarp();
         }
         if (!ok && lane == 0) set_err(a.err, kErrWait);
     } else if (warp < 4) {
         // ------------------------------------------------------ consumers
+        // The warps go their own pace: a stage is read when its barrier says
+        // so and freed by all four, and their sums meet through the partials
+        // buffers.  One whose bounded wait gives up leaves by itself; the
+        // others' waits then end the same way.
         float acc[kChains][NT][4], accu[kChains][NT][4];
         bool failed = false;
-        // A wait of one consumer warp that gives up is acted on by all four
-        // together at the next stage's barrier (they must leave the loop
-        // together: a warp left behind at the named barrier would wait forever).
-        bool gave_up = false;
         int n_items = 0;   // items finished by this CTA (selects the partials buffer)
+        int cur = -1;
+        Phase P;
         for (int t = 0;; ++t) {
             const int slot = t % S;
-            const bool ok = !gave_up && mbar_wait(&full[slot], (uint32_t)((t / S) & 1), kWaitLimitNs);
-            if (consumers_or(!ok)) {
+            // the vote also brings the lanes together: they leave the wait's
+            // loop one by one, and ldmatrix and mma need the whole warp
+            if (!__all_sync(0xffffffffu, mbar_wait(&full[slot], (uint32_t)((t / S) & 1), kWaitLimitNs))) {
                 failed = true;
                 break;
             }
@@ -563,7 +595,10 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                 failed = true;
                 break;
             }
-            const Phase P = decode(a, k);
+            if (k != cur) {
+                cur = k;
+                P = decode(a, k);
+            }
             if (kt >= P.tpi || it >= P.n_items || sl < 0 || sl >= P.n_sl) {
                 if (lane == 0) set_err(a.err, kErrCheckC);
                 failed = true;
@@ -578,7 +613,7 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
 #pragma unroll
                         for (int i = 0; i < 4; ++i) acc[c][nt][i] = accu[c][nt][i] = 0.f;
             }
-            const __nv_bfloat16* st = ring + (size_t)slot * stage_elems;
+            const uint32_t st = smem_u32(ring + (size_t)slot * stage_elems);
             if (P.kind == CH_GU) mma_stage<NT, true>(st, R, warp, lane, acc, accu);
             else mma_stage<NT, false>(st, R, warp, lane, acc, accu);
             __syncwarp();
@@ -597,9 +632,10 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                         acc[0][nt][i] += acc[c][nt][i];
                         accu[0][nt][i] += accu[c][nt][i];
                     }
-            if (n_items >= 2 && !mbar_wait(&red_free[b], (uint32_t)(((n_items >> 1) - 1) & 1), kWaitLimitNs)) {
-                gave_up = true;   // leave at the next barrier, with the other warps
-                continue;
+            if (n_items >= 2 &&
+                !__all_sync(0xffffffffu, mbar_wait(&red_free[b], (uint32_t)(((n_items >> 1) - 1) & 1), kWaitLimitNs))) {
+                failed = true;
+                break;
             }
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt)
@@ -632,12 +668,14 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                 run_v[nt][c] = -INFINITY;
                 run_i[nt][c] = INT_MAX;
             }
-        int items_in_phase = 0;   // items of the current phase finished by this CTA
+        int lm_items = 0;         // LM head items finished by this CTA
+        int cur = -1, next_cols = 0;   // the phase P describes, the columns of the next one's stages
+        Phase P;
         int scale_k = -1;         // the phase whose row scales `scale` holds
         bool ok = true;
         for (int n = 0;; ++n) {
             const int b = n & 1;
-            if (!mbar_wait(&red_full[b], (uint32_t)((n >> 1) & 1), kWaitLimitNs)) {
+            if (!__all_sync(0xffffffffu, mbar_wait(&red_full[b], (uint32_t)((n >> 1) & 1), kWaitLimitNs))) {
                 ok = false;
                 break;
             }
@@ -645,12 +683,16 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
             if (k < 0) break;
             const int it = red_it[b];
             const bool last_item = red_last[b] != 0;
-            if (k >= a.n_phases || it < 0 || it >= decode(a, k).n_items) {   // self-check
+            if (k < a.n_phases && k != cur) {
+                cur = k;
+                P = decode(a, k);
+                next_cols = k + 1 < a.n_phases ? stage_cols(decode(a, k + 1).kind) : 0;
+            }
+            if (k >= a.n_phases || it < 0 || it >= P.n_items) {   // self-check
                 set_err(a.err, kErrCheckE);
                 ok = false;
                 break;
             }
-            const Phase P = decode(a, k);
             // the four warps' K quarters, added in warp order
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt)
@@ -691,6 +733,7 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                     if (last) *tk = 0;   // every slice has arrived: ready for the next use
                 }
                 complete = __shfl_sync(0xffffffffu, last, 0) != 0;
+                __syncwarp();   // the other lanes' reads come after lane 0's ticket
                 if (complete) {
                     __threadfence();
 #pragma unroll
@@ -714,7 +757,7 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
             }
             if (complete) {
                 epilogue<NT>(a, P, k, it, acc, accu, normed_input(P.kind) ? scale : ones, run_v, run_i);
-                ++items_in_phase;
+                lm_items += P.kind == CH_LM;
             }
             if (complete && k + 1 < a.n_phases) {
                 // publish this row group to the next phase's stages that read it
@@ -722,33 +765,27 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                 __syncwarp();
                 if (lane == 0) {
                     __threadfence();
-                    atomicAdd(&blocks[k * kMaxBlocks + (it * 16) / stage_cols(decode(a, k + 1).kind)], 1);
+                    atomicAdd(&blocks[k * kMaxBlocks + (it * 16) / next_cols], 1);
                 }
             }
-            if (last_item) {
-                // this CTA has no more items in the phase: publish them all
-                // with one release (the next phase reads them by TMA)
-                if (P.kind == CH_LM) {
-                    // merge this CTA's per-row best into the global keys
-                    const int g = lane >> 2, t4 = lane & 3;
+            if (last_item && P.kind == CH_LM) {
+                // this CTA's last LM head item: merge its per-row best into the
+                // global keys, then count its items
+                const int g = lane >> 2, t4 = lane & 3;
 #pragma unroll
-                    for (int nt = 0; nt < NT; ++nt)
+                for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-                        for (int c = 0; c < 2; ++c) {
-                            const int r = nt * 8 + 2 * t4 + c;
-                            if (g == 0 && r < R && run_i[nt][c] != INT_MAX)
-                                atomicMax(&a.best[r], argmax_key(run_v[nt][c], run_i[nt][c]));
-                        }
-                }
-                fence_proxy_async_global();
+                    for (int c = 0; c < 2; ++c) {
+                        const int r = nt * 8 + 2 * t4 + c;
+                        if (g == 0 && r < R && run_i[nt][c] != INT_MAX)
+                            atomicMax(&a.best[r], argmax_key(run_v[nt][c], run_i[nt][c]));
+                    }
                 __syncwarp();
                 int fin = 0;
                 if (lane == 0) {
                     __threadfence();
-                    const int prev = atomicAdd(&done[k], items_in_phase);
-                    fin = (P.kind == CH_LM && prev + items_in_phase == P.n_items);
+                    fin = atomicAdd(done, lm_items) + lm_items == P.n_items;
                 }
-                items_in_phase = 0;
                 if (__shfl_sync(0xffffffffu, fin, 0)) {
                     // every CTA has merged: read the keys (and leave them zero)
                     __threadfence();
@@ -764,12 +801,12 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
 
     // the last CTA to leave resets the queues and counters for the next launch
     __syncthreads();
-    if (tid == 0) count_out(a.n_phases, queue, done, exits, blocks);
+    count_out(a.n_phases, queue, done, exits, blocks);
 }
 
 }  // namespace
 
-size_t chain_counter_ints() { return 2 * (size_t)kChainMaxPhases + 1 + (size_t)kChainMaxPhases * kMaxBlocks; }
+size_t chain_counter_ints() { return (size_t)kChainMaxPhases + 2 + (size_t)kChainMaxPhases * kMaxBlocks; }
 
 cudaError_t launch_chain(const ChainArgs& args, cudaStream_t s) {
     if (args.R < 1 || args.R > kMaxRows || args.n_phases < 1 || args.n_phases > kChainMaxPhases ||

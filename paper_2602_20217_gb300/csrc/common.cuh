@@ -24,6 +24,13 @@ KS_DEV uint4 lds128(const void* p) {
     return *reinterpret_cast<const uint4*>(p);
 }
 
+// Four 8 x 8 b16 matrices, lane l giving the row address l & 7 of matrix l >> 3.
+KS_DEV void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+
 // D = A * B + D, m16n8k16, bf16 inputs, fp32 accumulators.
 // A (16x16, row-major) fragment a0..a3, B (16x8, column-major) fragment b0..b1.
 KS_DEV void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,

@@ -228,52 +228,25 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return encode;
 }
 
-bool make_tma_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K, uint32_t box_rows) {
-    auto encode = tensor_map_encoder();
-    if (!encode || K % 8 != 0 || (reinterpret_cast<uintptr_t>(base) & 15) != 0) return false;
-    const cuuint64_t dims[2] = {K, rows};
-    const cuuint64_t strides[1] = {K * 2};
-    const cuuint32_t box[2] = {256, box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-bool make_weight_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K, uint32_t chunks) {
+bool make_chunk_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K, uint32_t box_rows,
+                    uint32_t chunks) {
     auto encode = tensor_map_encoder();
     if (!encode || K % 8 != 0 || (reinterpret_cast<uintptr_t>(base) & 15) != 0) return false;
     const cuuint32_t estr[3] = {1, 1, 1};
     if (K % 64 == 0) {
-        // {64 columns, rows, K / 64 chunks}: a box is `chunks` chunks of 16 rows
+        // {64 columns, rows, K / 64 chunks}: a box is `chunks` chunks of box_rows rows
         const cuuint64_t dims[3] = {64, rows, K / 64};
         const cuuint64_t strides[2] = {K * 2, 128};
-        const cuuint32_t box[3] = {64, 16, chunks};
+        const cuuint32_t box[3] = {64, box_rows, chunks};
         return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     }
     const cuuint64_t dims[2] = {K, rows};
     const cuuint64_t strides[1] = {K * 2};
-    const cuuint32_t box[2] = {64, 16};
+    const cuuint32_t box[2] = {64, box_rows};
     return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-bool make_stage_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K, uint32_t box_rows,
-                    uint32_t chunks) {
-    if (K % 256 != 0) return make_tma_map(map, base, rows, K, box_rows);
-    auto encode = tensor_map_encoder();
-    if (!encode || (reinterpret_cast<uintptr_t>(base) & 15) != 0) return false;
-    // [rows][K] viewed as {256 columns, rows, K / 256 chunks}: one box holds
-    // `chunks` consecutive 256-column chunks of box_rows rows, chunk-major
-    const cuuint64_t dims[3] = {256, rows, K / 256};
-    const cuuint64_t strides[2] = {K * 2, 512};
-    const cuuint32_t box[3] = {256, box_rows, chunks};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

@@ -41,19 +41,13 @@ struct GemvArgs {
 
 int gemv_groups(int N);     // CTAs of a launch (argmax candidates, sum-of-squares groups)
 cudaError_t launch_gemv(int epi, const GemvArgs& a, cudaStream_t s);
-// TMA map of a row-major bf16 matrix [rows][K] (K % 8 == 0, 16-byte aligned
-// base), box 256 columns x box_rows rows, no swizzle, zero fill outside.
-bool make_tma_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K, uint32_t box_rows);
-// Map for the chain kernel's stages: when K % 256 == 0 a 3-D view
-// {256, rows, K / 256} whose box {256, box_rows, chunks} is a whole stage (one
-// copy); otherwise the 2-D map above (one copy per 256-column chunk).
-bool make_stage_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K, uint32_t box_rows,
+// Map of a row-major bf16 matrix [rows][K] (K % 8 == 0, 16-byte aligned base)
+// for the chain kernel's stages and the attention tiles: 64-column chunks of
+// box_rows rows with the 128-byte swizzle, zero fill outside.  K % 64 == 0: 3-D
+// view {64, rows, K / 64}, box of `chunks` chunks (one copy per stage);
+// otherwise 2-D, box {64, box_rows} (one copy per chunk).
+bool make_chunk_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K, uint32_t box_rows,
                     uint32_t chunks);
-// Weight map for the chain kernel: 64-column chunks of 16 rows with the
-// 128-byte swizzle (16-byte unit u of row r lands at unit u ^ (r & 7)).
-// K % 64 == 0: 3-D view {64, rows, K / 64}, box of `chunks` chunks (one copy
-// per stage); otherwise 2-D, box {64, 16} (one copy per chunk).
-bool make_weight_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K, uint32_t chunks);
 // Maps of the wide kernels: boxes of 64 columns x 128 rows with the 128-byte
 // swizzle (an operand's stage), and 128 whole cache rows of hd elements.
 bool make_wide_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K);
@@ -71,7 +65,7 @@ enum ChainKind { CH_QKV = 0, CH_O = 1, CH_GU = 2, CH_DOWN = 3, CH_LM = 4 };
 
 constexpr int kChainSliceMaxItems = 640;   // residual phases with at most this many row groups are K-sliced
 struct ChainArgs {
-    CUtensorMap wmap[kChainMaxPhases];  // weights of each phase (make_weight_map)
+    CUtensorMap wmap[kChainMaxPhases];  // weights of each phase (make_chunk_map, 16 rows)
     CUtensorMap amap[4];        // inputs for this R: xg (4-chunk stages), xg (2-chunk), attn_out, act
     int n_phases;
     int R;                      // rows, 1..16
@@ -165,7 +159,7 @@ cudaError_t launch_wide_attention(int hd, const WideAttnArgs& a, cudaStream_t s)
 struct AttnArgs {
     // bf16: TMA map of the whole KV cache viewed as rows of hd elements
     // ([L][K, V][hk][max_seq] rows; 16-row boxes of hd / 64 swizzled 64-column
-    // chunks, make_weight_map), and the first row of this layer's K and V
+    // chunks, make_chunk_map), and the first row of this layer's K and V
     CUtensorMap kvmap;
     int kv_row_k, kv_row_v;
     __nv_bfloat16* q;       // bf16: prepared queries [hk][G R][hd] (QK-norm, RoPE, log2(e)/sqrt(hd))

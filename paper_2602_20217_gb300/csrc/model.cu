@@ -958,21 +958,21 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
         m->map_gu.resize(L);
         m->map_down.resize(L);
         for (int l = 0; l < L && ok; ++l) {
-            ok = ok && make_weight_map(&m->map_qkv[l], m->w_qkv[l], nqkv, d, 16);
-            ok = ok && make_weight_map(&m->map_o[l], m->w_o[l], d, hqd, 16);
-            ok = ok && make_weight_map(&m->map_gu[l], m->w_gate_up[l], 2 * (uint64_t)F, d, 8);
-            ok = ok && make_weight_map(&m->map_down[l], m->w_down[l], d, F, 16);
+            ok = ok && make_chunk_map(&m->map_qkv[l], m->w_qkv[l], nqkv, d, 16, 16);
+            ok = ok && make_chunk_map(&m->map_o[l], m->w_o[l], d, hqd, 16, 16);
+            ok = ok && make_chunk_map(&m->map_gu[l], m->w_gate_up[l], 2 * (uint64_t)F, d, 16, 8);
+            ok = ok && make_chunk_map(&m->map_down[l], m->w_down[l], d, F, 16, 16);
         }
-        ok = ok && make_weight_map(&m->map_lm, m->lm_head, cfg->vocab, d, 16);
+        ok = ok && make_chunk_map(&m->map_lm, m->lm_head, cfg->vocab, d, 16, 16);
         // [L][K, V][hk][max_seq] rows of hd elements; a box is one 16-key tile
-        ok = ok && make_weight_map(&m->map_kv, m->kv,
-                                   2 * (uint64_t)L * cfg->n_kv_heads * (uint64_t)cfg->max_seq, cfg->head_dim,
+        ok = ok && make_chunk_map(&m->map_kv, m->kv,
+                                   2 * (uint64_t)L * cfg->n_kv_heads * (uint64_t)cfg->max_seq, cfg->head_dim, 16,
                                    cfg->head_dim / 64);
         for (int r = 0; r < R; ++r) {
-            ok = ok && make_stage_map(&m->map_xg[r], m->xg, R, d, r + 1, 4);
-            ok = ok && make_stage_map(&m->map_xg2[r], m->xg, R, d, r + 1, 2);
-            ok = ok && make_stage_map(&m->map_attn_out[r], m->attn_out, R, hqd, r + 1, 4);
-            ok = ok && make_stage_map(&m->map_act[r], m->act, R, F, r + 1, 4);
+            ok = ok && make_chunk_map(&m->map_xg[r], m->xg, R, d, r + 1, 16);
+            ok = ok && make_chunk_map(&m->map_xg2[r], m->xg, R, d, r + 1, 8);
+            ok = ok && make_chunk_map(&m->map_attn_out[r], m->attn_out, R, hqd, r + 1, 16);
+            ok = ok && make_chunk_map(&m->map_act[r], m->act, R, F, r + 1, 16);
         }
         m->wide_qkv.resize(L);
         m->wide_o.resize(L);

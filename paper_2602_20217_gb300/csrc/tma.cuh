@@ -64,34 +64,12 @@ KS_DEV bool mbar_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
         else if ((i & 63) == 0 && global_ns() - t0 > limit_ns) return false;
     }
 }
-// Barrier of the four consumer warps (named barrier 1) that also ORs a flag.
-KS_DEV bool consumers_or(bool v) {
-    uint32_t r;
-    asm volatile(
-        "{ .reg .pred p, q; setp.ne.u32 p, %1, 0; bar.red.or.pred q, 1, 128, p; selp.u32 %0, 1, 0, q; }"
-        : "=r"(r)
-        : "r"((uint32_t)v)
-        : "memory");
-    return r != 0;
-}
-KS_DEV void consumers_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-
-KS_DEV int ld_acquire(const int* p) {
+KS_DEV int ld_relaxed(const int* p) {
     int v;
-    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-// Wait until *p >= target (another CTA of the same grid raises it); false
-// after limit_ns.
-KS_DEV bool wait_at_least(const int* p, int target, uint64_t limit_ns) {
-    if (ld_acquire(p) >= target) return true;
-    const uint64_t t0 = global_ns();
-    for (;;) {
-        __nanosleep(64);
-        if (ld_acquire(p) >= target) return true;
-        if (global_ns() - t0 > limit_ns) return false;
-    }
-}
+KS_DEV void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 // Order this thread's earlier generic-proxy writes/reads before its later
 // asynchronous-proxy (TMA) operations on global memory.
 KS_DEV void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
