@@ -210,16 +210,45 @@ __global__ void __launch_bounds__(128) attn_prep_kernel(const __grid_constant__ 
     // The attention kernel may launch now: before its own dependency wait it
     // only loads keys written by earlier passes.
     grid_launch_dependents();
-    grid_dependency_wait();          // the projections of this pass
     constexpr int NPL = HD / 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r = blockIdx.x, v = blockIdx.y * 4 + warp;
     const int G = a.hq / a.hk, M = G * a.R, pos = a.p0 + r;
     const float* row = a.qkv + (size_t)r * a.qkv_ld;
+    // the RoPE row and the norm's gain do not depend on this pass: loaded
+    // while the projections finish
+    const __nv_bfloat16* gain = reinterpret_cast<const __nv_bfloat16*>(v < a.hq ? a.q_norm : a.k_norm);
+    float2 cs[NPL / 2];
+    float gn[NPL];
+#pragma unroll
+    for (int i = 0; i < NPL / 2; ++i)
+        cs[i] = reinterpret_cast<const float2*>(a.rope + (size_t)pos * HD)[lane + 32 * i];
+#pragma unroll
+    for (int i = 0; i < NPL; ++i) gn[i] = gain != nullptr ? __bfloat162float(gain[lane + 32 * i]) : 1.f;
+    grid_dependency_wait();          // the projections of this pass
     float x[NPL];
+    // head vector v: optional RMSNorm, rotate-half RoPE (head_vector's steps)
+    auto vector = [&](const float* src) {
+#pragma unroll
+        for (int i = 0; i < NPL; ++i) x[i] = src[lane + 32 * i];
+        if (gain != nullptr) {
+            float ss = 0.f;
+#pragma unroll
+            for (int i = 0; i < NPL; ++i) ss = fmaf(x[i], x[i], ss);
+            ss = warp_sum(ss);
+            const float inv = rsqrtf(ss / (float)HD + a.eps);
+#pragma unroll
+            for (int i = 0; i < NPL; ++i) x[i] = (x[i] * inv) * gn[i];
+        }
+#pragma unroll
+        for (int i = 0; i < NPL / 2; ++i) {
+            const float u = x[i], w = x[i + NPL / 2];
+            x[i] = u * cs[i].x - w * cs[i].y;
+            x[i + NPL / 2] = w * cs[i].x + u * cs[i].y;
+        }
+    };
     if (v < a.hq) {
-        head_vector<__nv_bfloat16, NPL>(row + v * HD, reinterpret_cast<const __nv_bfloat16*>(a.q_norm), a.eps,
-                                        a.rope, pos, x);
+        vector(row + v * HD);
         const float qscale = kLog2e * rsqrtf((float)HD);
         const int h = v / G, m = r * G + (v - h * G);
         __nv_bfloat16* dst = a.q + ((size_t)h * M + m) * HD;
@@ -227,8 +256,7 @@ __global__ void __launch_bounds__(128) attn_prep_kernel(const __grid_constant__ 
         for (int i = 0; i < NPL; ++i) dst[lane + 32 * i] = __float2bfloat16_rn(x[i] * qscale);
     } else if (v < a.hq + a.hk) {
         const int h = v - a.hq;
-        head_vector<__nv_bfloat16, NPL>(row + (a.hq + h) * HD, reinterpret_cast<const __nv_bfloat16*>(a.k_norm),
-                                        a.eps, a.rope, pos, x);
+        vector(row + (a.hq + h) * HD);
         __nv_bfloat16* kc = reinterpret_cast<__nv_bfloat16*>(a.kcache) + ((size_t)h * a.max_seq + pos) * HD;
         __nv_bfloat16* vc = reinterpret_cast<__nv_bfloat16*>(a.vcache) + ((size_t)h * a.max_seq + pos) * HD;
         const float* vs = row + (a.hq + a.hk + h) * HD;

@@ -13,7 +13,7 @@
 // GPU.  Only the small activation tiles wait for the previous phase.
 //
 // Per CTA (two per SM for up to 8 rows, else one; 7 warps):
-//  * warp 4 (weights): claims work items phase by phase from per-phase
+//  * warp 4 (weights): claims work units phase by phase from per-phase
 //    atomic queues (16 output features over the full K) and issues their
 //    2-D TMA weight boxes into a ring of shared-memory stages;
 //  * warp 5 (activations): follows the same stage sequence; before a stage
@@ -74,18 +74,14 @@ constexpr int kErrCheckW = 2, kErrCheckA = 3, kErrCheckC = 4, kErrCheckE = 5;
 KS_DEV void set_err(int* e, int code) { atomicCAS(e, 0, code); }
 
 struct Phase {
-    int kind, layer, N, K, n_items, tpi;
-    int n_sl, sl_len, n_units;   // K-slices per item (residual phases with few items), stages per slice
+    int kind, layer, N, K, n_items, tpi;   // items of 16 output features, stages per item
 };
 
-// The residual projections W_o and W_down have only d / 16 row groups (256 for
-// d = 4096): fewer items than CTAs.  Long items (8 stages or more: W_down, and
-// W_o at hq * hd >= 8192) are split into two K-slices (fixed by the shape,
-// never by R, so every row has the same arithmetic); the slice that finishes
-// second adds both partial sums in slice order.  Short items stay whole: a
-// slice's partial-sum round trip would cost more than it balances.
-constexpr int kSliceMaxItems = kChainSliceMaxItems;
-
+// W_o and W_down have only d / 16 row groups, fewer than the CTAs or little
+// more, and an item still takes its whole K: cut into two K-slices whose
+// partial sums met in global memory, a layer took 95.2 us (Llama-3-8B shape, 4k
+// context) against 89.9, with more slices up to 123: the partial sums, the
+// ticket and the other slices' read-back all sit on the one epilogue warp.
 KS_DEV Phase decode(const ChainArgs& a, int k) {
     const int code = a.code[k];
     Phase p;
@@ -104,9 +100,6 @@ KS_DEV Phase decode(const ChainArgs& a, int k) {
     p.n_items = (p.N + 15) >> 4;
     const int shift = p.kind == CH_GU ? 9 : 10;      // k columns per stage: 512 or 1024
     p.tpi = (p.K + (1 << shift) - 1) >> shift;
-    p.n_sl = ((p.kind == CH_O || p.kind == CH_DOWN) && p.n_items <= kSliceMaxItems && p.tpi >= 8) ? 2 : 1;
-    p.sl_len = (p.tpi + p.n_sl - 1) >> (p.n_sl - 1);
-    p.n_units = p.n_items * p.n_sl;
     return p;
 }
 KS_DEV bool normed_input(int kind) { return kind == CH_QKV || kind == CH_GU || kind == CH_LM; }
@@ -349,11 +342,10 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
     __shared__ __align__(8) uint64_t pub[kMaxStages];
     __shared__ int slot_k[kMaxStages], slot_it[kMaxStages], slot_kt[kMaxStages];
     __shared__ int slot_last[kMaxStages];   // the stage ends this CTA's last item of its phase
-    __shared__ int slot_sl[kMaxStages];     // the item's K-slice
     __shared__ float ones[kMaxRows];        // the input scale of phases without a norm
     __shared__ float scale[kMaxRows];       // 1 / rms of the rows (epilogue warp only)
     __shared__ float red[2][4][2][NT * 4][32];   // [buffer][consumer warp][gate, up][fragment][lane]
-    __shared__ int red_k[2], red_it[2], red_last[2], red_sl[2];
+    __shared__ int red_k[2], red_it[2], red_last[2];
     __shared__ __align__(8) uint64_t red_full[2];   // 4 consumer warps arrive
     __shared__ __align__(8) uint64_t red_free[2];   // the epilogue warp arrives
     __shared__ int void_job;
@@ -397,11 +389,10 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
         if (lane == 0) {
             bool ok = true;
             int t = 0;
-            auto issue = [&](int k, const Phase& P, int it, int kt, int sl, bool last_item) -> bool {
+            auto issue = [&](int k, const Phase& P, int it, int kt, bool last_item) -> bool {
                 const int slot = t % S;
                 // self-check: every box coordinate below follows from these ranges
-                if (k < 0 || k >= a.n_phases || it < 0 || it >= P.n_items || kt < 0 || kt >= P.tpi || sl < 0 ||
-                    sl >= P.n_sl) {
+                if (k < 0 || k >= a.n_phases || it < 0 || it >= P.n_items || kt < 0 || kt >= P.tpi) {
                     set_err(a.err, kErrCheckW);
                     return false;
                 }
@@ -410,7 +401,6 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                 slot_it[slot] = it;
                 slot_kt[slot] = kt;
                 slot_last[slot] = last_item;
-                slot_sl[slot] = sl;
                 mbar_expect_tx(&full[slot], kWBytes);
                 __nv_bfloat16* st = ring + (size_t)slot * stage_elems;
                 const CUtensorMap* wm = &a.wmap[k];
@@ -435,39 +425,34 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                 ++t;
                 return true;
             };
-            // Work assignment per phase: the CTA's first unit is fixed by its
-            // index (unit blockIdx.x, if the phase has that many), so phases
-            // with about one unit per CTA (W_o, W_down, QKV) spread over every
-            // CTA; further units come from the phase's atomic queue, offset by
+            // Work assignment per phase: the CTA's first item is fixed by its
+            // index (item blockIdx.x, if the phase has that many), so phases
+            // with about one item per CTA (W_o, W_down, QKV) spread over every
+            // CTA; further items come from the phase's atomic queue, offset by
             // the grid size.  This launch's queues were zeroed by the launch
             // before the previous one (counter sets alternate), which has
             // completed.  Weight boxes need no input, so the first S stages
             // go out while the previous kernel runs.  No deadlock: every CTA
             // of the grid is co-resident once the kernels before it finish,
-            // and a CTA finishes its units of a phase before it waits for the
+            // and a CTA finishes its items of a phase before it waits for the
             // next phase's inputs.
             const int grid = (int)gridDim.x;
             int k = 0;
             Phase P = decode(a, 0);
             int it = (int)blockIdx.x;
-            while (ok) {   // `it` counts units: K-slice it / n_items, item it % n_items
-                if (it >= P.n_units) {
+            while (ok) {
+                if (it >= P.n_items) {
                     if (++k >= a.n_phases) break;
                     P = decode(a, k);
                     it = (int)blockIdx.x;
                     continue;
                 }
                 // claimed ahead: its latency hides behind the stream (the
-                // ticket is first needed at the unit's last stage, so its
-                // round trip overlaps the unit's other stages)
-                const int next = P.n_units > grid ? grid + atomicAdd(&queue[k], 1) : INT_MAX;
-                // slice-major: every item's first K-slice comes before any
-                // second one, so the units taken first (one per CTA) read the
-                // previous phase's first blocks, which complete first
-                const int sl = it >= P.n_items, item = sl ? it - P.n_items : it;
-                const int kt0 = sl * P.sl_len, kt1 = min(P.tpi, kt0 + P.sl_len);
-                for (int kt = kt0; kt < kt1 && ok; ++kt)
-                    ok = issue(k, P, item, kt, sl, kt == kt1 - 1 && next >= P.n_units);
+                // ticket is first needed at the item's last stage, so its
+                // round trip overlaps the item's other stages)
+                const int next = P.n_items > grid ? grid + atomicAdd(&queue[k], 1) : INT_MAX;
+                for (int kt = 0; kt < P.tpi && ok; ++kt)
+                    ok = issue(k, P, it, kt, kt == P.tpi - 1 && next >= P.n_items);
                 it = next;
             }
             if (ok) {  // sentinel stage: no more work
@@ -578,7 +563,7 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                 break;
             }
             const int k = slot_k[slot];
-            const int it = slot_it[slot], kt = slot_kt[slot], sl = slot_sl[slot];
+            const int it = slot_it[slot], kt = slot_kt[slot];
             const bool last_item = slot_last[slot] != 0;
             const int b = n_items & 1;
             if (k < 0) {
@@ -599,13 +584,12 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                 cur = k;
                 P = decode(a, k);
             }
-            if (kt >= P.tpi || it >= P.n_items || sl < 0 || sl >= P.n_sl) {
+            if (kt >= P.tpi || it >= P.n_items) {
                 if (lane == 0) set_err(a.err, kErrCheckC);
                 failed = true;
                 break;
             }
-            const int kt0 = sl * P.sl_len, kt1 = min(P.tpi, kt0 + P.sl_len);
-            if (kt == kt0) {
+            if (kt == 0) {
 #pragma unroll
                 for (int c = 0; c < kChains; ++c)
 #pragma unroll
@@ -618,7 +602,7 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
             else mma_stage<NT, false>(st, R, warp, lane, acc, accu);
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[slot]);   // this warp is done with the stage
-            if (kt != kt1 - 1) continue;
+            if (kt != P.tpi - 1) continue;
 
             // item done: add the chains in chain order and hand this warp's
             // sums to the epilogue warp through partials buffer b (double
@@ -648,7 +632,6 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                 red_k[b] = k;
                 red_it[b] = it;
                 red_last[b] = last_item;
-                red_sl[b] = sl;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&red_full[b]);
@@ -710,44 +693,9 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                         acc[nt][i] += red[b][w][0][nt * 4 + i][lane];
                         if (P.kind == CH_GU) accu[nt][i] += red[b][w][1][nt * 4 + i][lane];
                     }
-            const int sl = red_sl[b];
             __syncwarp();
             if (lane == 0) mbar_arrive(&red_free[b]);   // partials read: the buffer is free
-            bool complete = true;
-            if (P.n_sl > 1) {
-                // a K-slice: leave its sums in global memory; the slice that
-                // completes the item adds all of them in slice order
-                const int g = lane >> 2, t4 = lane & 3;
-                float* part = a.slice_part + ((size_t)(k & 1) * kSliceMaxItems + it) * (2 * 256);
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        part[sl * 256 + (g + 8 * (i >> 1)) * 16 + nt * 8 + 2 * t4 + (i & 1)] = acc[nt][i];
-                __syncwarp();
-                int last = 0;
-                if (lane == 0) {
-                    __threadfence();
-                    int* tk = a.slice_ticket + (k & 1) * kSliceMaxItems + it;
-                    last = atomicAdd(tk, 1) == P.n_sl - 1;
-                    if (last) *tk = 0;   // every slice has arrived: ready for the next use
-                }
-                complete = __shfl_sync(0xffffffffu, last, 0) != 0;
-                __syncwarp();   // the other lanes' reads come after lane 0's ticket
-                if (complete) {
-                    __threadfence();
-#pragma unroll
-                    for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int o = (g + 8 * (i >> 1)) * 16 + nt * 8 + 2 * t4 + (i & 1);
-                            float v = __ldcg(&part[o]);
-                            for (int q = 1; q < P.n_sl; ++q) v += __ldcg(&part[q * 256 + o]);
-                            acc[nt][i] = v;
-                        }
-                }
-            }
-            if (complete && normed_input(P.kind) && k != scale_k) {
+            if (normed_input(P.kind) && k != scale_k) {
                 // This CTA's first item of a normed phase: its last stage
                 // waited for every block of phase k - 1 (an item's stages
                 // cover them all), so every row group's partial sums of
@@ -755,11 +703,9 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) chain_kernel(const __gr
                 scale_k = k;
                 row_scales<NT>(a, lane, scale);
             }
-            if (complete) {
-                epilogue<NT>(a, P, k, it, acc, accu, normed_input(P.kind) ? scale : ones, run_v, run_i);
-                lm_items += P.kind == CH_LM;
-            }
-            if (complete && k + 1 < a.n_phases) {
+            epilogue<NT>(a, P, k, it, acc, accu, normed_input(P.kind) ? scale : ones, run_v, run_i);
+            lm_items += P.kind == CH_LM;
+            if (k + 1 < a.n_phases) {
                 // publish this row group to the next phase's stages that read it
                 fence_proxy_async_global();
                 __syncwarp();

@@ -194,7 +194,7 @@ static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 struct Layout {
     size_t kv, rope, x, ss, xg, qkv, attn_out, act, attn_part, counters, logits, amax_val,
         amax_idx, tok, hist, hist_snap, hist_idx, sims, mask, obj, wts, select, chain_ctr, best, tpt_masks,
-        tpt_tok, tpt_info, tpt_out, dyn, samp, slice, qbuf, wide, wide_part, wide_ticket, total;
+        tpt_tok, tpt_info, tpt_out, dyn, samp, qbuf, wide, wide_part, wide_ticket, total;
     int wide_rows;   // rows of a wide chunk (0: fp32 models, no wide path)
     int n_chunks_max;
     int hist_slots;
@@ -346,8 +346,6 @@ static Layout make_layout(const ks_config* c) {
     L.dyn = take(sizeof(float) * ((size_t)R + kTop1Ctas) + sizeof(int));
     // sampling: q and p distributions, [R][kSampleMaxK] ids and probs plus [R] sizes each
     L.samp = take(2 * ((size_t)R * kSampleMaxK * (sizeof(int) + sizeof(float)) + sizeof(int) * R));
-    // chain kernel K-slices: partial sums [2][640][2][16][16] floats, then tickets [2][640]
-    L.slice = take(sizeof(float) * 2 * kChainSliceMaxItems * 512 + sizeof(int) * 2 * kChainSliceMaxItems);
     // bf16 attention: the pass's prepared queries [hk][G R][hd]
     L.qbuf = take(sizeof(__nv_bfloat16) * (size_t)R * c->n_q_heads * hd);
     // wide path: partial sums of K-sliced tiles and their arrivals (zero between launches)
@@ -400,8 +398,6 @@ struct ks_model {
     int* top1_ticket;
     int* stop;                // dynamic exit: set once a draft token is below tau_conf
     int* n_drafted;           // dynamic exit: draft passes of the step that ran
-    float* slice_part;        // chain kernel: K-slice partial sums
-    int* slice_ticket;
     __nv_bfloat16* qbuf;      // bf16 attention: prepared queries of the pass
     CUtensorMap map_kv;       // bf16 attention: the KV cache as rows of hd elements
     bool last_dynamic = false;
@@ -619,8 +615,6 @@ static ks_status forward(ks_model* m, const int32_t* tok, int R, int p0, const u
         ca.capture_plane = (long long)m->lay.hist_slots * c.max_rows * d;
         ca.err = m->err;
         ca.stop = stop;
-        ca.slice_part = m->slice_part;
-        ca.slice_ticket = m->slice_ticket;
         int nph = 0, klass = K_CHAIN;
         double bytes = 0.0;
         auto flush = [&]() -> ks_status {
@@ -931,8 +925,6 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
     m->top1_ticket = reinterpret_cast<int*>(m->top1_part + kTop1Ctas);
     m->stop = m->rows + (3 * cfg->max_rows + 5);        // spare words of the token block
     m->n_drafted = m->rows + (3 * cfg->max_rows + 6);
-    m->slice_part = reinterpret_cast<float*>(b + lay.slice);
-    m->slice_ticket = reinterpret_cast<int*>(m->slice_part + (size_t)2 * kChainSliceMaxItems * 512);
     m->qbuf = reinterpret_cast<__nv_bfloat16*>(b + lay.qbuf);
     {
         char* sb = b + lay.samp;
@@ -1043,8 +1035,6 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
     if (e != cudaSuccess) return fail(e, "counter reset");
     e = cudaMemsetAsync(b + lay.tok, 0, sizeof(int) * ((size_t)3 * R + 8 + cfg->max_seq), m->stream);  // incl. err
     if (e != cudaSuccess) return fail(e, "token reset");
-    e = cudaMemsetAsync(m->slice_ticket, 0, sizeof(int) * 2 * kChainSliceMaxItems, m->stream);
-    if (e != cudaSuccess) return fail(e, "slice reset");
     e = cudaMemsetAsync(b + lay.wide_ticket, 0, sizeof(int) * kWideTickets, m->stream);
     if (e != cudaSuccess) return fail(e, "ticket reset");
     e = cudaMemsetAsync(b + lay.dyn, 0, sizeof(float) * ((size_t)R + kTop1Ctas) + sizeof(int), m->stream);
@@ -1506,8 +1496,6 @@ static ks_status lm_head_rows(ks_model* m, int R, int32_t* tokens) {
         ca.capture = nullptr;
         ca.err = m->err;
         ca.stop = nullptr;
-        ca.slice_part = m->slice_part;
-        ca.slice_ticket = m->slice_ticket;
         ca.n_phases = 1;
         ca.code[0] = (uint16_t)(4 * L);
         ca.gain[0] = nullptr;
