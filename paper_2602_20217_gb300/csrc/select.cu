@@ -29,19 +29,21 @@ namespace ks {
 constexpr int kCosCtas = 4;
 constexpr int kCosThreads = 256;
 
-// VEC: elements per load, 16 bytes' worth or 1 (rows that are not 16-byte aligned)
-template <typename T, int VEC>
-__global__ void __cluster_dims__(kCosCtas, 1, 1) __launch_bounds__(kCosThreads)
-    cosine_kernel(const T* X, const T* Y, int rows, int d, int64_t pair_stride, const int32_t* row_index, float* out) {
+// VEC: elements per load, 16 bytes' worth or 1 (rows that are not 16-byte
+// aligned).  CTAS: kCosCtas, or 1 for pairs of little work, which a cluster's
+// launch and barriers would only slow down.
+template <typename T, int VEC, int CTAS>
+KS_DEV void cosine_pair(const T* X, const T* Y, int rows, int d, int64_t pair_stride, const int32_t* row_index,
+                        float* out) {
     extern __shared__ float rowcos[];
-    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");   // this CTA runs: its shared memory may be written
-    const int64_t p = blockIdx.x / kCosCtas;
-    const uint32_t rank = cluster_rank();
+    if (CTAS > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");   // this CTA's shared memory may be written
+    const int64_t p = blockIdx.x / CTAS;
+    const uint32_t rank = CTAS > 1 ? cluster_rank() : 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const T* Xp = X + p * pair_stride;
     const T* Yp = Y + p * pair_stride;
-    bool waited = false;
-    for (int i = (int)rank + kCosCtas * warp; i < rows; i += kCosCtas * (kCosThreads / 32)) {
+    bool waited = CTAS == 1;
+    for (int i = (int)rank + CTAS * warp; i < rows; i += CTAS * (kCosThreads / 32)) {
         const int64_t ri = row_index ? row_index[i] : i;
         const T* x = Xp + ri * d;
         const T* y = Yp + ri * d;
@@ -79,17 +81,37 @@ __global__ void __cluster_dims__(kCosCtas, 1, 1) __launch_bounds__(kCosThreads)
         waited = true;
         if (lane == 0) {
             const float c = xy / (sqrtf(xx) * sqrtf(yy));
-            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(&rowcos[i], 0)), "f"(c) : "memory");
+            if (CTAS == 1) rowcos[i] = c;
+            else asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(&rowcos[i], 0)), "f"(c) : "memory");
         }
     }
     if (!waited) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-    cluster_sync();   // the row terms are in the first CTA
+    if (CTAS > 1) cluster_sync();   // the row terms are in the first CTA
+    else __syncthreads();
     if (rank == 0 && threadIdx.x == 0) {
         float s = 0.f;
         for (int i = 0; i < rows; ++i) s += rowcos[i];
         out[p] = s / (float)rows;
     }
 }
+
+template <typename T, int VEC>
+__global__ void __cluster_dims__(kCosCtas, 1, 1) __launch_bounds__(kCosThreads)
+    cosine_kernel(const T* X, const T* Y, int rows, int d, int64_t pair_stride, const int32_t* row_index, float* out) {
+    cosine_pair<T, VEC, kCosCtas>(X, Y, rows, d, pair_stride, row_index, out);
+}
+template <typename T, int VEC>
+__global__ void __launch_bounds__(kCosThreads) cosine_small_kernel(const T* X, const T* Y, int rows, int d,
+                                                                   int64_t pair_stride, const int32_t* row_index,
+                                                                   float* out) {
+    cosine_pair<T, VEC, 1>(X, Y, rows, d, pair_stride, row_index, out);
+}
+
+// Bytes of a pair's rows up to which one CTA takes the pair.  A loop of calls
+// on 64 pairs took, in us per call with one CTA / with a cluster: 9.0 / 9.5 at
+// 32 KB, 8.4 / 9.5 at 160 KB, 8.7 / 9.6 at 256 KB (16 pairs), 10.3 / 9.5 at
+// 300 KB, 10.2 / 9.9 at 320 KB, 20.5 / 12.0 at 1000 KB (128 pairs).
+constexpr int64_t kCosSmall = 256 * 1024;
 
 cudaError_t launch_cosine(const void* X, const void* Y, int dtype, int64_t n_pairs, int rows, int d,
                           int64_t pair_stride, const int32_t* row_index, float* out, cudaStream_t s) {
@@ -100,18 +122,27 @@ cudaError_t launch_cosine(const void* X, const void* Y, int dtype, int64_t n_pai
     const bool aligned = d % vec == 0 && pair_stride % vec == 0 &&
                          ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 15) == 0;
     constexpr int64_t kMost = 1 << 28;   // pairs of a launch: the grid's limit
-    auto run = [&](auto kern, auto x, auto y) {
-        for (int64_t p = 0; p < n_pairs; p += kMost)
-            kern<<<(unsigned)((n_pairs - p < kMost ? n_pairs - p : kMost) * kCosCtas), kCosThreads, smem, s>>>(
-                x + p * pair_stride, y + p * pair_stride, rows, d, pair_stride, row_index, out + p);
+    const bool small = 2 * (int64_t)rows * d * (16 / vec) <= kCosSmall;
+    auto run = [&](auto kern, auto kern_small, auto x, auto y) {
+        for (int64_t p = 0; p < n_pairs; p += kMost) {
+            const unsigned n = (unsigned)(n_pairs - p < kMost ? n_pairs - p : kMost);
+            if (small)
+                kern_small<<<n, kCosThreads, smem, s>>>(x + p * pair_stride, y + p * pair_stride, rows, d, pair_stride,
+                                                        row_index, out + p);
+            else
+                kern<<<n * kCosCtas, kCosThreads, smem, s>>>(x + p * pair_stride, y + p * pair_stride, rows, d,
+                                                             pair_stride, row_index, out + p);
+        }
         return cudaGetLastError();
     };
     if (dtype == KS_DTYPE_BF16) {
         auto x = reinterpret_cast<const __nv_bfloat16*>(X), y = reinterpret_cast<const __nv_bfloat16*>(Y);
-        return aligned ? run(cosine_kernel<__nv_bfloat16, 8>, x, y) : run(cosine_kernel<__nv_bfloat16, 1>, x, y);
+        return aligned ? run(cosine_kernel<__nv_bfloat16, 8>, cosine_small_kernel<__nv_bfloat16, 8>, x, y)
+                       : run(cosine_kernel<__nv_bfloat16, 1>, cosine_small_kernel<__nv_bfloat16, 1>, x, y);
     }
     auto x = reinterpret_cast<const float*>(X), y = reinterpret_cast<const float*>(Y);
-    return aligned ? run(cosine_kernel<float, 4>, x, y) : run(cosine_kernel<float, 1>, x, y);
+    return aligned ? run(cosine_kernel<float, 4>, cosine_small_kernel<float, 4>, x, y)
+                   : run(cosine_kernel<float, 1>, cosine_small_kernel<float, 1>, x, y);
 }
 
 // ----------------------------------------------------------------- knapsack
@@ -372,7 +403,7 @@ struct TptArgs {
 // kept by the tie rule (the first of the largest values in candidate order,
 // gamma ascending, which is what replacing on strictly larger finds).  One
 // thread doing all of it in sequence took 50 us for 8 candidates at D = 10,
-// 90 for 13 of the hidden-state DP.
+// 90 for 13 of the hidden-state DP; now 9.
 __global__ void __launch_bounds__(256) tpt_kernel(const TptArgs a) {
     __shared__ double alpha[kMaxTpt], draft[kMaxTpt];
     __shared__ double best_v[8];

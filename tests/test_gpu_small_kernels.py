@@ -54,7 +54,8 @@ def test_knapsack_capacities(n, budget, most):
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("pairs,rows,d,extra,offset", [(1, 1, 1, 0, 0), (3, 4, 7, 0, 0), (2, 33, 64, 0, 0),
                                                        (5, 32, 128, 0, 1), (2, 31, 130, 2, 0), (4, 65, 512, 8, 0),
-                                                       (2, 100, 4096, 4, 0), (2, 9, 4096, 0, 4)])
+                                                       (2, 100, 4096, 4, 0), (2, 9, 4096, 0, 4),
+                                                       (1, 64, 512, 0, 0), (3, 601, 131, 2, 1)])
 def test_cosine_alignment(dtype, pairs, rows, d, extra, offset):
     import torch
 
