@@ -136,7 +136,8 @@ typedef struct ks_model ks_model;
 /* ------------------------------------------------------------ model (a1-a3) */
 
 /* Bytes of device workspace a model with this config needs (KV cache, RoPE
- * table, activations, split partials, history ring).  0 on an invalid config. */
+ * table, activations, split partials, the buffers of the many-row passes,
+ * history ring).  0 on an invalid config. */
 size_t ks_workspace_bytes(const ks_config* cfg);
 
 /* Validate cfg, borrow the weights and the workspace (dev, 256-byte aligned,
@@ -153,7 +154,8 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
 ks_status ks_model_destroy(ks_model* m);
 
 /* Run the prompt (host int32[n], 1 <= n, n + 1 <= max_seq) through the target
- * in chunks of max_rows rows, fill the KV cache, seed the history with the
+ * (bf16 models: many rows at a time as GEMMs; fp32 ones: in chunks of max_rows
+ * rows), fill the KV cache, seed the history with the
  * last hist_init_rows prompt rows, and set the pending token to the greedy
  * next token, written to *next_token (host).  Resets any previous sequence. */
 ks_status ks_prefill(ks_model* m, const int32_t* tokens, int32_t n, int32_t* next_token);
@@ -346,8 +348,8 @@ ks_status ks_select_tpt(ks_model* m, const ks_latency* lat, int32_t n_candidates
  * matrix cosine to the target's X^(i) is at least as high; states with cosine
  * below tau or j > K / 2 are dropped (Sec. 3.4, pruning; the paper uses tau
  * 0.5); g[i, 0] = X^(i).  Inside f^(i) a history row attends to the target's
- * K/V for earlier positions and to the state's own K/V (the target's cache is
- * restored afterwards).  Each surviving terminal state gives a layer set (by
+ * K/V for earlier positions and to the state's own K/V (the target's cache
+ * holds the same values afterwards).  Each surviving terminal state gives a layer set (by
  * its recorded choices) and an acceptance estimate (Eq. 4: the fraction of
  * rows whose LM-head argmax equals the target's); the Eq. 3 grid over the
  * candidates (executed weight ascending) and gamma = 1..max_gamma picks
@@ -413,7 +415,8 @@ ks_status ks_generate_speculative(ks_model* m, const ks_spec_params* params, int
 /* ------------------------------------------------------------ diagnostics */
 
 /* Copy a window of device state to the caller (for tests):
- * what = 0: logits of the last pass, float[rows][vocab];
+ * what = 0: logits of the last prompt, draft or verify pass, float[rows][vocab] (a layer
+ *           selection's candidate states may or may not replace them);
  *        1: the residual stream rows, float[rows][d];
  *        2: K cache of layer `layer`, [n_kv_heads][positions][head_dim] in the model dtype
  *           for positions [start, start + count), dst laid out [hk][count][hd];

@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(128, kAttnCtasPerSm) attn_bf16_kernel(const __
 // same values everywhere), so none waits for another.  Latency-bound: with all
 // rows of a chunk in one CTA and scalar loads the tiny workload's 5-row verify
 // took 91 us on 6 CTAs; 16-byte loads of K, several V rows in flight and a
-// warp per row take 12.
+// warp per row take 18.
 template <int HD>
 __global__ void __launch_bounds__(128) attn_f32_kernel(const AttnArgs a) {
     if (a.stop && *a.stop) return;   // a draft pass after the dynamic exit

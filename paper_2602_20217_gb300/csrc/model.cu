@@ -3,11 +3,13 @@
 // Sec. 2.1), the history ring (Sec. 3.4), and the speculative loop that
 // re-selects the draft mask with the knapsack (a4, a5).
 //
-// All device memory is the caller's workspace; this file carves it up.  The
-// host loop launches one kernel per matrix product (5 per layer plus the
-// attention split/merge pair) on the caller's stream; draft tokens stay on
-// the device between steps and one stream synchronisation per verify step
-// returns the accepted tokens.
+// All device memory is the caller's workspace; this file carves it up.  On
+// the caller's stream, a decode pass of a bf16 model launches a chain of
+// projections between two attention cores (fp32: one kernel per product); rows
+// in large numbers (prompts, the candidate states of the layer selection) go
+// through the wide GEMMs and attention instead.  Draft tokens stay on the
+// device between steps and one stream synchronisation per verify step returns
+// the accepted tokens.
 #include "../../include/knapspec.h"
 #include "common.cuh"
 #include "internal.h"

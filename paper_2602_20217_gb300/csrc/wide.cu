@@ -4,8 +4,11 @@
 // Y[m][n] = sum_k A[m][k] W[n][k], M rows at a time (up to the caller's chunk).
 // Streaming the weights once per 16 rows, as the decode path does, left the
 // tensor cores idle: a 4096-token prompt read every weight 256 times.  Two
-// layers of the Llama-3-8B shape over 4096 tokens: 90.4 -> 2.9 ms for the whole
-// prefill; two of the Qwen3-32B shape over 9001: 391 -> 13.5 ms.
+// layers of the Llama-3-8B shape over 4096 tokens: 90.5 -> 2.74 ms for the whole
+// prefill; two of the Qwen3-32B shape over 9001: 391 -> 14.3 ms.  What bounds it
+// is the tensor pipe: at 2048 rows the gate/up GEMM of the 8B shape takes 262 us
+// (1835 TFLOP/s, pipe 85 % active), W_down 153, QKV 75 and W_o 55 (fewer tiles
+// than two rounds of all pairs, so the last round and the epilogues show).
 //
 // One CTA pair (cta_group::2) works on a 256 x 256 tile: each CTA stages its
 // 128 rows of A and its half of the tile's 256 weight rows (K-major, 64-column

