@@ -235,7 +235,9 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
                     m = mnew;
                 } else if (__any_sync(0xffffffffu, mnew > m + kRescale)) {
                     // only rows that grew change: a row never depends on its neighbours
-                    const float mm = mnew > m + kRescale ? mnew : m, alpha = fast_exp2(m - mm);
+                    // (one that has still seen no key has neither sum nor O: its factor must not be 2^(-inf + inf))
+                    const float mm = mnew > m + kRescale ? mnew : m;
+                    const float alpha = mm == -INFINITY ? 1.f : fast_exp2(m - mm);
                     m = mm;
                     l *= alpha;
 #pragma unroll 1
@@ -249,8 +251,8 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
                         tmem_st32(o_at + c, o);
                     }
                 }
-                // a state's row may have seen no key yet: P is then 0
-                const float ref = STATES && m == -INFINITY ? 0.f : m;
+                // no key seen yet (a state's row before its state's tile): P is then 0
+                const float ref = m == -INFINITY ? 0.f : m;
                 float sum[4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
