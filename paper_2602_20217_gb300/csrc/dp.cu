@@ -73,8 +73,8 @@ KS_DEV void wide_row(float v, int q, int k, int d, const __nv_bfloat16* gain, __
 }
 
 // grid (n r, ceil(d / 256)): row q belongs to state j0 + q / r.  Invalid
-// states become zeros: their values are never used, but they share key tiles
-// with the others, where 0 * NaN would not vanish.
+// states become zeros: their values are never used, but what lies there could
+// send the attention's check of its key tiles down its slow path.
 __global__ void __launch_bounds__(256) dp_prep_kernel(const float* G, int j0, const int* valid, int r, int d,
                                                       const __nv_bfloat16* gain, float* E, __nv_bfloat16* xg,
                                                       float* ss, int ss_ld) {

@@ -18,6 +18,12 @@
 // see the cache's keys below p0, and each row its own state's rows up to
 // itself, so the key tiles are the cache's and then those of the block's own
 // K/V rows under a band mask.
+// A masked key has P = 0, but 0 times an infinity or a NaN in its V row would
+// still be NaN, for rows that do not see that key: in the tiles that some row
+// does not see whole (the last two or three of a CTA), a warp of its own clears
+// V rows that are not finite before they are used and notes their keys, and the
+// rows that do see such a key get NaN.  It takes half a microsecond a tile,
+// under the softmax of the tile's scores.
 // Queries come prepared (QK-norm, RoPE, log2(e) / sqrt(hd)), the keys and
 // values of these rows are already in the cache.
 //
@@ -28,8 +34,8 @@
 // The decode kernel read the cache once per 16 rows for the same work.
 //
 // Warps: 0-3 and 4-7 the softmax of query tile 0 and 1, 8 the MMAs, 9 the
-// loads.  TMEM: S0, S1 (128 columns each), O0, O1 (hd columns each).  Longest
-// query blocks first.  Every wait is bounded.
+// loads, 10 the check of the masked tiles.  TMEM: S0, S1 (128 columns each), O0,
+// O1 (hd columns each).  Longest query blocks first.  Every wait is bounded.
 #include "common.cuh"
 #include "internal.h"
 #include "umma.cuh"
@@ -43,8 +49,10 @@ namespace {
 constexpr int kQ = 128;                      // rows of a query tile, keys of a key tile
 constexpr int kChunk = kQ * 128;             // bytes of 128 rows x 64 columns
 constexpr int kRing = 4;                     // K and V tiles in flight
-constexpr int kThreads = 320;
+constexpr int kThreads = 352;
 constexpr float kRescale = 8.f;              // log2 of the growth of a maximum that O is rescaled for
+constexpr int kMaskedTiles = 16;             // tiles with masked keys: at most 3, states up to kMaxStateRows: 14
+constexpr int kMaxStateRows = 1280;
 template <int HD>
 constexpr size_t wide_attn_smem() { return 1024 + (size_t)(2 + kRing) * (HD / 64) * kChunk; }
 
@@ -52,6 +60,56 @@ KS_DEV float fast_exp2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+// One warp: the rows (keys) of a V tile that hold an infinity or a NaN are cleared
+// and recorded in bad[4] (a bit per key); false if there are none.
+template <int HD>
+KS_DEV bool clear_bad_keys(unsigned char* tile, uint32_t* bad) {
+    constexpr int CH = HD / 64;
+    const int lane = threadIdx.x & 31;
+    // lane l: 16 bytes of row 4 it + l / 8 in every chunk (the swizzle stays within a row)
+    auto at = [&](int it, int c) { return reinterpret_cast<uint4*>(tile + c * kChunk + it * 512 + lane * 16); };
+    // 0 * x is NaN exactly where x is not finite
+    auto probe = [](uint4 v, __nv_bfloat162 (&s)[4]) {
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            s[e] = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w[e]), __float2bfloat162_rn(0.f), s[e]);
+    };
+    auto found = [](const __nv_bfloat162 (&s)[4]) {
+        uint32_t any = 0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) any |= *reinterpret_cast<const uint32_t*>(&s[e]);
+        return (any & 0x7fff7fffu) != 0;
+    };
+    __nv_bfloat162 s[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) s[e] = __float2bfloat162_rn(0.f);
+#pragma unroll 8
+    for (int it = 0; it < kQ / 4; ++it)
+#pragma unroll
+        for (int c = 0; c < CH; ++c) probe(*at(it, c), s);
+    if (!__any_sync(0xffffffffu, found(s))) return false;
+#pragma unroll 1
+    for (int it = 0; it < kQ / 4; ++it) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[e] = __float2bfloat162_rn(0.f);
+#pragma unroll
+        for (int c = 0; c < CH; ++c) probe(*at(it, c), s);
+        const uint32_t hit = __ballot_sync(0xffffffffu, found(s));
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if ((hit >> (8 * q) & 0xffu) == 0) continue;
+            if (lane == 0) bad[it / 8] |= 1u << (4 * (it % 8) + q);
+            if (lane / 8 == q)
+#pragma unroll
+                for (int c = 0; c < CH; ++c) *at(it, c) = make_uint4(0, 0, 0, 0);
+        }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read the cleared rows
+    __syncwarp();
+    return true;
 }
 
 template <int HD, bool STATES>
@@ -65,9 +123,11 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     unsigned char* qs = smem;
     unsigned char* ring = smem + 2 * TB;
-    __shared__ __align__(8) uint64_t q_full, kv_full[kRing], kv_free[kRing], s_full[2], p_full[2], o_full[2];
+    __shared__ __align__(8) uint64_t q_full, kv_full[kRing], kv_free[kRing], s_full[2], p_full[2], o_full[2], v_ok[2], check;
     __shared__ uint32_t tmem_slot;
     __shared__ int void_job;
+    __shared__ uint32_t bad[kMaskedTiles][4];   // keys of the masked tiles whose V row is not finite
+    __shared__ int any_bad;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int h = (int)blockIdx.x % a.hq, kvh = h / (a.hq / a.hk);
@@ -82,11 +142,16 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
         nt[i] = first >= a.M ? 0 : STATES ? n_cache + last / kQ - own0 + 1 : (a.p0 + last) / kQ + 1;
     }
     const int n = max(nt[0], nt[1]);
+    // the first key tile that some row does not see whole
+    const int m0 = STATES ? a.p0 / kQ : (a.p0 + q0 + 1) / kQ;
 
+    if (tid < kMaskedTiles * 4) (&bad[0][0])[tid] = 0u;
     if (warp == 8) tmem_alloc<1>(&tmem_slot, 512);
     if (tid == 0) {
         void_job = __ldcg(a.err) != 0;
+        any_bad = 0;
         mbar_init(&q_full, 1);
+        mbar_init(&check, 1);
         for (int i = 0; i < kRing; ++i) {
             mbar_init(&kv_full[i], 1);
             mbar_init(&kv_free[i], 1);
@@ -94,7 +159,8 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
         for (int i = 0; i < 2; ++i) {
             mbar_init(&s_full[i], 1);
             mbar_init(&p_full[i], 4);
-            mbar_init(&o_full[i], 1);
+            mbar_init(&o_full[i], 2);   // the MMAs' commit, and an arrival that orders `bad` before it
+            mbar_init(&v_ok[i], 1);     // masked tiles m0 + i, m0 + i + 2, ..
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -152,6 +218,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
                     umma_commit(&s_full[i]);
                 };
                 wait_tile(0);
+                if (m0 == 0) mbar_arrive(&check);
                 if (ok) {
                     for (int i = 0; i < 2; ++i)
                         if (nt[i] > 0) scores(i, 0);
@@ -159,7 +226,9 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
                 }
                 for (int j = 0; j < n && ok; ++j) {
                     wait_tile(2 * j + 1);
+                    if (j + 1 == m0) mbar_arrive(&check);
                     if (j + 1 < n) wait_tile(2 * j + 2);
+                    if (j >= m0) ok = ok && mbar_wait(&v_ok[(j - m0) & 1], (uint32_t)((j - m0) >> 1 & 1), kWaitLimitNs);
                     if (!ok) break;
                     const uint32_t sv = smem_u32(ring + (size_t)((2 * j + 1) % kRing) * TB);
                     for (int i = 0; i < 2; ++i) {
@@ -171,8 +240,12 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
                         for (int k = 0; k < kQ / 16; ++k)   // 16 keys: 8 P columns, 2 KB of V rows
                             umma_ts(tmem + 256 + HD * i, tmem + 128 * i + 8 * k,
                                     umma_desc(sv + 2048 * k, kChunk, 1024), kIdescO, j > 0 || k > 0);
-                        if (j + 1 < nt[i]) scores(i, j + 1);
-                        else umma_commit(&o_full[i]);
+                        if (j + 1 < nt[i]) {
+                            scores(i, j + 1);
+                        } else {
+                            umma_commit(&o_full[i]);
+                            mbar_arrive(&o_full[i]);
+                        }
                     }
                     if (!ok) break;
                     umma_commit(&kv_free[(2 * j + 1) % kRing]);
@@ -180,6 +253,21 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
                 }
                 if (!ok) atomicCAS(a.err, 0, 1);
             }
+        } else if (warp == 10) {
+            // ------------------------------------------- check of the masked tiles
+            // It starts once the V tiles before m0 have landed: a ring slot's parity tells a tile's copy only
+            // from the slot's last one.  From tile m0 on the MMAs wait for it.
+            bool ok = m0 >= n || __all_sync(0xffffffffu, mbar_wait(&check, 0, kWaitLimitNs));
+            for (int j = m0; j < n && ok; ++j) {
+                // every lane reads the tile, so each waits for it itself
+                const int t = 2 * j + 1;
+                ok = __all_sync(0xffffffffu, mbar_wait(&kv_full[t % kRing], (uint32_t)((t / kRing) & 1), kWaitLimitNs));
+                if (!ok) break;
+                if (clear_bad_keys<HD>(ring + (size_t)(t % kRing) * TB, bad[j - m0]) && lane == 0) any_bad = 1;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&v_ok[(j - m0) & 1]);
+            }
+            if (!ok && lane == 0) atomicCAS(a.err, 0, 1);
         } else {
             // -------------------------------------------------------- softmax
             const int i = warp >> 2, quad = warp & 3;
@@ -189,6 +277,16 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
             const uint32_t s_at = lanes + 128 * i, o_at = lanes + 256 + HD * i;
             float m = -INFINITY, l = 0.f;
             bool ok = true;
+            // this row sees the keys lo .. hi of key tile j
+            auto seen = [&](int j, int& lo, int& hi) {
+                lo = 0;
+                hi = pos - kQ * j;
+                if (STATES) {
+                    const int base = (own0 + j - n_cache) * kQ;
+                    lo = j < n_cache ? 0 : row - row % a.state_rows - base;
+                    hi = j < n_cache ? a.p0 - 1 - kQ * j : row - base;
+                }
+            };
             for (int j = 0; j < nt[i]; ++j) {
                 ok = mbar_wait(&s_full[i], (uint32_t)(j & 1), kWaitLimitNs);
                 if (!__all_sync(0xffffffffu, ok)) {
@@ -202,20 +300,10 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
                 tmem_wait_ld();
 #pragma unroll
                 for (int c = 0; c < 4; ++c) tmem_pin(s[c]);
-                // keys lo .. hi of the tile are seen; tiles that every row sees whole need no mask
-                int lo = 0, hi = pos - kQ * j;
-                bool masked = kQ * (j + 1) > a.p0 + q0 + i * kQ + 1;
-                if (STATES) {
-                    if (j < n_cache) {
-                        hi = a.p0 - 1 - kQ * j;
-                        masked = kQ * (j + 1) > a.p0;
-                    } else {
-                        const int base = (own0 + j - n_cache) * kQ;
-                        lo = row - row % a.state_rows - base;
-                        hi = row - base;
-                        masked = true;
-                    }
-                }
+                // tiles that every row sees whole need no mask
+                int lo, hi;
+                seen(j, lo, hi);
+                const bool masked = STATES ? j >= n_cache || kQ * (j + 1) > a.p0 : kQ * (j + 1) > a.p0 + q0 + i * kQ + 1;
                 if (masked) {
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
@@ -284,7 +372,16 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
                 ok = __all_sync(0xffffffffu, ok);
                 if (ok) {
                     umma_fence_after();
-                    const float inv = 1.f / l;
+                    float inv = 1.f / l;
+                    for (int j = any_bad ? m0 : nt[i]; j < nt[i]; ++j) {   // a key with a V row that is not finite: NaN
+                        int lo, hi;
+                        seen(j, lo, hi);
+                        for (int w = 0; w < 4; ++w)
+                            for (uint32_t b = bad[j - m0][w]; b != 0; b &= b - 1) {
+                                const int key = 32 * w + __ffs(b) - 1;
+                                if (key >= lo && key <= hi) inv = __int_as_float(0x7fffffff);
+                            }
+                    }
                     __nv_bfloat16* dst = a.out + (size_t)row * a.hq * HD + h * HD;
 #pragma unroll 1
                     for (int c = 0; c < HD; c += 32) {
@@ -318,7 +415,8 @@ __global__ void __launch_bounds__(kThreads, 1) wide_attn_kernel(const __grid_con
 }  // namespace
 
 cudaError_t launch_wide_attention(int hd, const WideAttnArgs& args, cudaStream_t s) {
-    if (args.M < 1 || args.p0 < 0 || args.err == nullptr || args.hq % args.hk) return cudaErrorInvalidValue;
+    if (args.M < 1 || args.p0 < 0 || args.err == nullptr || args.hq % args.hk || args.state_rows > kMaxStateRows)
+        return cudaErrorInvalidValue;
     WideAttnArgs a = args;
     a.blocks = (a.M + 2 * kQ - 1) / (2 * kQ);
     auto run = [&](auto kern, size_t smem) -> cudaError_t {
