@@ -99,7 +99,7 @@ struct WideArgs {
     int M, N, K;                // rows, output features (WK_SWIGLU: d_ff), inputs
     int tiles_m, tiles_n;       // set by launch_wide
     int full, tail, share;      // set by launch_wide: whole tiles, tiles cut along K, stages per pair of the latter
-    float* part;                // kWidePartFloats partial sums of the cut tiles (null: none is cut)
+    float* part;                // kWidePartFloats partial sums of the cut tiles (used only where wide_cuts(K))
     int* ticket;                // kWideTickets arrivals, zero between launches
     float* capture;             // WK_RESID: rows from capture_from on are also written here, [row - capture_from][N]
     int capture_from;
@@ -128,6 +128,7 @@ struct WideArgs {
 constexpr int kWidePairs = 76;
 constexpr size_t kWidePartFloats = (size_t)2 * kWidePairs * 256 * 256;
 constexpr int kWideTickets = kWidePairs * 16;
+bool wide_cuts(int K);      // a launch over K inputs may cut tiles
 int wide_tiles_n(int kind, int N);
 inline int wide_ss_slots(int d) { return 2 * ((d + 255) / 256); }   // of a WK_RESID launch's ss_out
 cudaError_t launch_wide(int kind, int hd, const WideArgs& a, cudaStream_t s);

@@ -350,8 +350,10 @@ static Layout make_layout(const ks_config* c) {
     L.samp = take(2 * ((size_t)R * kSampleMaxK * (sizeof(int) + sizeof(float)) + sizeof(int) * R));
     // bf16 attention: the pass's prepared queries [hk][G R][hd]
     L.qbuf = take(sizeof(__nv_bfloat16) * (size_t)R * c->n_q_heads * hd);
-    // wide path: partial sums of K-sliced tiles and their arrivals (zero between launches)
-    L.wide_part = take(L.wide_rows ? sizeof(float) * kWidePartFloats : 0);
+    // wide path: partial sums of the tiles cut along K, for models some of whose
+    // projections can have such tiles, and their arrivals (zero between launches)
+    const int deepest = std::max({d, c->n_q_heads * hd, c->d_ff});
+    L.wide_part = take(L.wide_rows && wide_cuts(deepest) ? sizeof(float) * kWidePartFloats : 0);
     L.wide_ticket = take(sizeof(int) * kWideTickets);
     L.total = off;
     return L;

@@ -597,6 +597,9 @@ cudaError_t launch_wide_tokens(const unsigned long long* best, int M, int32_t* t
     return cudaGetLastError();
 }
 
+// launch_wide's rule below for the smallest share it deals out
+bool wide_cuts(int K) { return kMinShare + kMergeStages < (K + kTileK - 1) / kTileK; }
+
 int wide_tiles_n(int kind, int N) { return kind == WK_SWIGLU ? (N + 127) / 128 : (N + kTileN - 1) / kTileN; }
 
 cudaError_t launch_wide_embed(const __nv_bfloat16* embed, const int32_t* tok, int M, int d, int vocab, float* x,
@@ -626,7 +629,7 @@ cudaError_t launch_wide(int kind, int hd, const WideArgs& args, cudaStream_t s) 
     a.tail = 0;
     a.share = 1;
     int pairs = std::min(pairs_max, tiles);
-    if (rest > 0 && a.part != nullptr && a.ticket != nullptr && share + kMergeStages < kblocks) {
+    if (rest > 0 && share + kMergeStages < kblocks) {
         a.full = tiles - rest;
         a.tail = rest;
         a.share = share;
