@@ -141,7 +141,9 @@ typedef struct ks_model ks_model;
 size_t ks_workspace_bytes(const ks_config* cfg);
 
 /* Validate cfg, borrow the weights and the workspace (dev, 256-byte aligned,
- * at least ks_workspace_bytes(cfg) bytes), build the RoPE table, zero the KV
+ * ks_workspace_bytes(cfg) bytes; one that lacks only the room of the many-row
+ * passes' buffers is taken too, and prompts and layer selections of a bf16
+ * model then go through decode passes of max_rows rows), build the RoPE table, zero the KV
  * cache region of the workspace (the attention streams whole 16-key tiles,
  * and keys past a row's position get an exact zero weight only if their
  * values are finite), and return a handle bound to `stream` (a cudaStream_t;

@@ -197,7 +197,7 @@ struct Layout {
     size_t kv, rope, x, ss, xg, qkv, attn_out, act, attn_part, counters, logits, amax_val,
         amax_idx, tok, hist, hist_snap, hist_idx, sims, mask, obj, wts, select, chain_ctr, best, tpt_masks,
         tpt_tok, tpt_info, tpt_out, dyn, samp, qbuf, wide, wide_part, wide_ticket, total;
-    int wide_rows;   // rows of a wide chunk (0: fp32 models, no wide path)
+    int wide_rows;   // rows of a wide chunk (0: no wide path: fp32 models, workspaces without its buffers)
     int n_chunks_max;
     int hist_slots;
 };
@@ -290,7 +290,8 @@ static int dp_wide_rows(const ks_config* c, size_t bytes) {
     return rows;
 }
 
-static Layout make_layout(const ks_config* c) {
+// many_rows: with the buffers of the many-row passes (bf16 models).
+static Layout make_layout(const ks_config* c, bool many_rows = true) {
     Layout L{};
     const size_t es = c->dtype == KS_DTYPE_BF16 ? 2 : 4;
     const int d = c->d_model, hd = c->head_dim, R = c->max_rows;
@@ -321,13 +322,13 @@ static Layout make_layout(const ks_config* c) {
     // A prefill's wide chunks use the space of what is dead until they are
     // done: attention partials, logits and history; only models of few layers
     // need more than these take.
-    L.wide_rows = c->dtype == KS_DTYPE_BF16 ? wide_chunk_rows(c) : 0;
+    L.wide_rows = many_rows && c->dtype == KS_DTYPE_BF16 ? wide_chunk_rows(c) : 0;
     L.wide = off;
     L.attn_part = take(sizeof(float) * (size_t)R * c->n_q_heads * L.n_chunks_max * (hd + 4));
     L.logits = take(sizeof(float) * (size_t)R * c->vocab);
     if (L.wide_rows) off = std::max(off, L.wide + dp_wide_layout(c, kDpWideRows, 0).bytes);   // the DP's, beside the history
     L.hist = take(sizeof(float) * (size_t)(nsub + 1) * L.hist_slots * R * d);
-    off = std::max(off, L.wide + wide_layout(c, L.wide_rows, 0).bytes);
+    if (L.wide_rows) off = std::max(off, L.wide + wide_layout(c, L.wide_rows, 0).bytes);
     L.hist_snap = take(sizeof(float) * (size_t)(nsub + 1) * R * d);  // the prefill's history entry
     L.hist_idx = take(sizeof(int) * (size_t)L.hist_slots * R);
     L.sims = take(sizeof(float) * nsub);
@@ -354,7 +355,7 @@ static Layout make_layout(const ks_config* c) {
     // projections can have such tiles, and their arrivals (zero between launches)
     const int deepest = std::max({d, c->n_q_heads * hd, c->d_ff});
     L.wide_part = take(L.wide_rows && wide_cuts(deepest) ? sizeof(float) * kWidePartFloats : 0);
-    L.wide_ticket = take(sizeof(int) * kWideTickets);
+    L.wide_ticket = take(L.wide_rows ? sizeof(int) * kWideTickets : 0);
     L.total = off;
     return L;
 }
@@ -850,9 +851,12 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
         set_error("ks_model_create: workspace must be 256-byte aligned");
         return KS_ERR_INVALID_ARG;
     }
-    const Layout lay = make_layout(cfg);
+    Layout lay = make_layout(cfg);
+    const size_t want = lay.total;
+    // room for all but the many-row passes' buffers: decode passes take their place
+    if (workspace_bytes < want) lay = make_layout(cfg, false);
     if (workspace_bytes < lay.total) {
-        set_error("ks_model_create: workspace %zu < required %zu", workspace_bytes, lay.total);
+        set_error("ks_model_create: workspace %zu < required %zu", workspace_bytes, want);
         return KS_ERR_WORKSPACE;
     }
     const int L = cfg->n_layers;
@@ -970,24 +974,26 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
             ok = ok && make_chunk_map(&m->map_attn_out[r], m->attn_out, R, hqd, r + 1, 16);
             ok = ok && make_chunk_map(&m->map_act[r], m->act, R, F, r + 1, 16);
         }
-        m->wide_qkv.resize(L);
-        m->wide_o.resize(L);
-        m->wide_gu.resize(L);
-        m->wide_down.resize(L);
-        for (int l = 0; l < L && ok; ++l) {
-            ok = ok && make_wide_map(&m->wide_qkv[l], m->w_qkv[l], nqkv, d);
-            ok = ok && make_wide_map(&m->wide_o[l], m->w_o[l], d, hqd);
-            ok = ok && make_wide_map(&m->wide_gu[l], m->w_gate_up[l], 2 * (uint64_t)F, d);
-            ok = ok && make_wide_map(&m->wide_down[l], m->w_down[l], d, F);
+        if (lay.wide_rows) {
+            m->wide_qkv.resize(L);
+            m->wide_o.resize(L);
+            m->wide_gu.resize(L);
+            m->wide_down.resize(L);
+            for (int l = 0; l < L && ok; ++l) {
+                ok = ok && make_wide_map(&m->wide_qkv[l], m->w_qkv[l], nqkv, d);
+                ok = ok && make_wide_map(&m->wide_o[l], m->w_o[l], d, hqd);
+                ok = ok && make_wide_map(&m->wide_gu[l], m->w_gate_up[l], 2 * (uint64_t)F, d);
+                ok = ok && make_wide_map(&m->wide_down[l], m->w_down[l], d, F);
+            }
+            ok = ok && make_wide_map(&m->wide_lm, m->lm_head, cfg->vocab, d);
+            const WideLayout W = wide_layout(cfg, lay.wide_rows, lay.wide);
+            ok = ok && make_wide_map(&m->wide_xg, b + W.xg, lay.wide_rows, d);
+            ok = ok && make_wide_map(&m->wide_q, b + W.q, lay.wide_rows, hqd);
+            ok = ok && make_wide_map(&m->wide_ao, b + W.ao, lay.wide_rows, hqd);
+            ok = ok && make_wide_map(&m->wide_act, b + W.act, lay.wide_rows, F);
+            ok = ok && make_wide_kv_map(&m->wide_kv, m->kv,
+                                        2 * (uint64_t)L * cfg->n_kv_heads * (uint64_t)cfg->max_seq, cfg->head_dim);
         }
-        ok = ok && make_wide_map(&m->wide_lm, m->lm_head, cfg->vocab, d);
-        const WideLayout W = wide_layout(cfg, lay.wide_rows, lay.wide);
-        ok = ok && make_wide_map(&m->wide_xg, b + W.xg, lay.wide_rows, d);
-        ok = ok && make_wide_map(&m->wide_q, b + W.q, lay.wide_rows, hqd);
-        ok = ok && make_wide_map(&m->wide_ao, b + W.ao, lay.wide_rows, hqd);
-        ok = ok && make_wide_map(&m->wide_act, b + W.act, lay.wide_rows, F);
-        ok = ok && make_wide_kv_map(&m->wide_kv, m->kv, 2 * (uint64_t)L * cfg->n_kv_heads * (uint64_t)cfg->max_seq,
-                                    cfg->head_dim);
         if (!ok) {
             set_error("ks_model_create: TMA descriptor encoding failed");
             delete m;
@@ -1039,7 +1045,7 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
     if (e != cudaSuccess) return fail(e, "counter reset");
     e = cudaMemsetAsync(b + lay.tok, 0, sizeof(int) * ((size_t)3 * R + 8 + cfg->max_seq), m->stream);  // incl. err
     if (e != cudaSuccess) return fail(e, "token reset");
-    e = cudaMemsetAsync(b + lay.wide_ticket, 0, sizeof(int) * kWideTickets, m->stream);
+    if (lay.wide_rows) e = cudaMemsetAsync(b + lay.wide_ticket, 0, sizeof(int) * kWideTickets, m->stream);
     if (e != cudaSuccess) return fail(e, "ticket reset");
     e = cudaMemsetAsync(b + lay.dyn, 0, sizeof(float) * ((size_t)R + kTop1Ctas) + sizeof(int), m->stream);
     if (e != cudaSuccess) return fail(e, "dynamic-exit reset");
@@ -1107,7 +1113,7 @@ ks_status ks_prefill(ks_model* m, const int32_t* tokens, int32_t n, int32_t* nex
     // to 8 cost (four Llama-3-8B layers: 820 us at any length up to 256 against
     // 1385, 1780, 2724 us at 32, 33 and 64 tokens in passes of 16).
     const int passes = (n + R - 1) / R;
-    const bool wide = m->dtype == KS_DTYPE_BF16 && passes * (R > 8 ? 3 : 2) > 7;
+    const bool wide = m->lay.wide_rows > 0 && passes * (R > 8 ? 3 : 2) > 7;
     if (wide) {
         // even wide chunks of whole tiles; the last rows' states go to the
         // snapshot of the history entry, from where the LM head takes them
@@ -1596,7 +1602,7 @@ static ks_status tpt_stage(ks_model* m, const ks_latency* lat, int K, int D, int
     int done = 0;
     // More rows than one pass of the decode kernel takes: the LM head reads
     // its weights once for all of them instead of once per max_rows.
-    if (bf && total > c.max_rows) {
+    if (m->lay.wide_rows > 0 && total > c.max_rows) {
         const WideHead H = wide_head(m);
         for (; H.rows > c.max_rows && done < total; done += std::min(H.rows, total - done)) {
             const int B = std::min(H.rows, total - done);
@@ -1933,7 +1939,7 @@ ks_status ks_select_dp(ks_model* m, const ks_latency* lat, float tau, int32_t ma
     }
     // bf16 models with more state rows than one decode pass takes: wide passes
     // over batches of whole states
-    const int wide_rows = m->dtype == KS_DTYPE_BF16 ? dp_wide_rows(&c, m->lay.hist - m->lay.wide) : 0;
+    const int wide_rows = m->lay.wide_rows > 0 ? dp_wide_rows(&c, m->lay.hist - m->lay.wide) : 0;
     const bool wide = (S - 1) * r > c.max_rows && wide_rows >= r;
     CUtensorMap maps[6];
     if (wide) {
@@ -2018,7 +2024,7 @@ ks_status ks_select_dp(ks_model* m, const ks_latency* lat, float tau, int32_t ma
     // Eq. 4 inputs: the LM head's argmax of every terminal state's rows and of X^(2L)
     const int total = (n_cand + 1) * r;
     int done = 0;
-    if (m->dtype == KS_DTYPE_BF16 && total > c.max_rows) {   // all rows in one wide LM head pass (or few)
+    if (m->lay.wide_rows > 0 && total > c.max_rows) {   // all rows in one wide LM head pass (or few)
         const WideHead H = wide_head(m);
         for (; H.rows > c.max_rows && done < total; done += std::min(H.rows, total - done)) {
             const int rows = std::min(H.rows, total - done);
