@@ -418,7 +418,8 @@ ks_status ks_generate_speculative(ks_model* m, const ks_spec_params* params, int
 
 /* Copy a window of device state to the caller (for tests):
  * what = 0: logits of the last prompt, draft or verify pass, float[rows][vocab] (a layer
- *           selection's candidate states may or may not replace them);
+ *           selection of few rows, or of an fp32 model, replaces them with its candidate
+ *           states'; the many-row passes of bf16 models leave them);
  *        1: the residual stream rows, float[rows][d];
  *        2: K cache of layer `layer`, [n_kv_heads][positions][head_dim] in the model dtype
  *           for positions [start, start + count), dst laid out [hk][count][hd];

@@ -319,14 +319,17 @@ static Layout make_layout(const ks_config* c, bool many_rows = true) {
     L.amax_idx = take(sizeof(int) * (size_t)gemv_groups(c->vocab) * 16);
     // tokens: rows[R+1] | target[R] | result[R+3] | err | prompt/out[max_seq]
     L.tok = take(sizeof(int) * ((size_t)3 * R + 8 + c->max_seq));
+    // the last pass's logits, which a layer selection leaves alone
+    const size_t logits = sizeof(float) * (size_t)R * c->vocab;
+    L.logits = take(logits);
     // A prefill's wide chunks use the space of what is dead until they are
-    // done: attention partials, logits and history; only models of few layers
-    // need more than these take.
+    // done: attention partials and history; only models of few layers need
+    // more than these take.  The selections' wide passes keep the history and
+    // have the space before it, which is widened for them.
     L.wide_rows = many_rows && c->dtype == KS_DTYPE_BF16 ? wide_chunk_rows(c) : 0;
     L.wide = off;
     L.attn_part = take(sizeof(float) * (size_t)R * c->n_q_heads * L.n_chunks_max * (hd + 4));
-    L.logits = take(sizeof(float) * (size_t)R * c->vocab);
-    if (L.wide_rows) off = std::max(off, L.wide + dp_wide_layout(c, kDpWideRows, 0).bytes);   // the DP's, beside the history
+    if (L.wide_rows) off = std::max(align_up(off + logits, 256), L.wide + dp_wide_layout(c, kDpWideRows, 0).bytes);
     L.hist = take(sizeof(float) * (size_t)(nsub + 1) * L.hist_slots * R * d);
     if (L.wide_rows) off = std::max(off, L.wide + wide_layout(c, L.wide_rows, 0).bytes);
     L.hist_snap = take(sizeof(float) * (size_t)(nsub + 1) * R * d);  // the prefill's history entry
@@ -1535,8 +1538,8 @@ static ks_status lm_head_rows(ks_model* m, int R, int32_t* tokens) {
     return launch(m, K_LMHEAD, [&] { return launch_gemv(EPI_LMHEAD, g, s); }, "tpt lm-head");
 }
 
-// LM head argmax of many rows (bf16 models): buffers in the space of the
-// attention partials and logits, which no pass is using then.
+// LM head argmax of many rows (bf16 models): buffers in the space from the
+// attention partials to the history, which no pass is using then.
 struct WideHead {
     __nv_bfloat16* xg;            // [rows][d] x * final gain
     float* ss;                    // [slots][rows] sums of squares
