@@ -181,8 +181,6 @@ KS_DEV void mma_stage(uint32_t st, int R, int warp, int lane, float (&acc)[kChai
     }
 }
 
-// Item epilogue on warp 0 (after the warp-order sum).  Fragment (nt, i) of
-// lane (g, t) is feature it * 16 + g + 8 (i >> 1), row nt * 8 + 2 t + (i & 1).
 // Argmax key of (logit v, token i): larger v first, then the lower id; an
 // unsigned 64-bit max over keys is the argmax in any order of merging.
 KS_DEV unsigned long long argmax_key(float v, int i) {
@@ -216,6 +214,8 @@ struct ResidIn {
     }
 };
 
+// Item epilogue (after the warp-order sum).  Fragment (nt, i) of lane (g, t) is
+// feature it * 16 + g + 8 (i >> 1), row nt * 8 + 2 t + (i & 1).
 template <int NT>
 KS_DEV void epilogue(const ChainArgs& a, const Phase& P, int it, const ResidIn<NT>& in, float (&acc)[NT][4],
                      float (&accu)[NT][4], const float* scale, float (&run_v)[NT][2], int (&run_i)[NT][2]) {

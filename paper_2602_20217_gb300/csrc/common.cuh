@@ -11,19 +11,6 @@ namespace ks {
 
 constexpr int kWarp = 32;
 
-// 16-byte streaming load that bypasses L1 (weights are read exactly once per pass).
-KS_DEV uint4 ldg_stream(const void* p) {
-    uint4 r;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
-                 : "l"(p));
-    return r;
-}
-
-KS_DEV uint4 lds128(const void* p) {
-    return *reinterpret_cast<const uint4*>(p);
-}
-
 // Four 8 x 8 b16 matrices, lane l giving the row address l & 7 of matrix l >> 3.
 KS_DEV void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
