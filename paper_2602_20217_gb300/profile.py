@@ -7,8 +7,9 @@ capture short: a few GB of device memory, a few hundred kernel launches.
 
   python -m paper_2602_20217_gb300.profile --workload llama8b-4k --layers 2 --prompt 512 --steps 3
 
-The speculative steps run inside an NVTX range named "decode", so a profiler
-can skip the prefill (ncu --nvtx --nvtx-include "decode/").
+The prompt runs inside an NVTX range named "prefill" and the speculative steps
+inside one named "decode", so a profiler can take either alone (ncu --nvtx
+--nvtx-include "decode/").
 """
 from __future__ import annotations
 
@@ -42,7 +43,9 @@ def main():
         sh = replace(sh, vocab=args.vocab)
     prompt = synth.prompt_tokens(sh, args.prompt, seed=wl.prompt_seed)
     m = Model(sh, max_seq=args.prompt + (args.steps + 2) * (args.gamma + 1) + 16, seed=wl.weight_seed)
+    torch.cuda.nvtx.range_push("prefill")
     m.prefill(prompt)
+    torch.cuda.nvtx.range_pop()
     if args.timing:
         for k in ks.KLASS.values():   # every class: the projections then run one per launch
             ks.ks_kernel_timing(m.h, k, True)
