@@ -156,10 +156,14 @@ ks_status ks_model_create(const ks_config* cfg, const ks_weights* w, void* works
 ks_status ks_model_destroy(ks_model* m);
 
 /* Run the prompt (host int32[n], 1 <= n, n + 1 <= max_seq) through the target
- * (bf16 models: many rows at a time as GEMMs; fp32 ones: in chunks of max_rows
- * rows), fill the KV cache, seed the history with the
+ * (bf16 models: many rows at a time as GEMMs; short prompts and fp32 models: in
+ * chunks of max_rows rows), fill the KV cache, seed the history with the
  * last hist_init_rows prompt rows, and set the pending token to the greedy
- * next token, written to *next_token (host).  Resets any previous sequence. */
+ * next token, written to *next_token (host).  Resets any previous sequence.
+ * The same prompt gives the same bits again.  The GEMMs add in another order
+ * than decode passes, and their tiling depends on the prompt's length: a
+ * prompt's rows agree with the same tokens decoded, verified or read in a
+ * prompt of another length to bf16 rounding, not bit for bit. */
 ks_status ks_prefill(ks_model* m, const int32_t* tokens, int32_t n, int32_t* next_token);
 
 /* Return to the state right after the last ks_prefill without recomputing the

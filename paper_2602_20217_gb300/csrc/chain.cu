@@ -81,7 +81,11 @@ struct Phase {
 // more, and an item still takes its whole K: cut into two K-slices whose
 // partial sums met in global memory, a layer took 95.2 us (Llama-3-8B shape, 4k
 // context) against 89.9, with more slices up to 123: the partial sums, the
-// ticket and the other slices' read-back all sit on the one epilogue warp.
+// ticket and the other slices' read-back all sit on the one epilogue warp.  Other
+// shapes, 16 decode steps of four layers before (slices) and since (without,
+// and with the query prep's and the residual's loads ahead), ms: width 512 2.13,
+// 2.06; 1024 2.43, 2.36; 2048 3.35, 3.25; 3072 4.31, 3.95; 8B 6.25, 5.84; 32B
+// 11.19, 10.97; two of width 8192 8.77, 8.39.
 KS_DEV Phase decode(const ChainArgs& a, int k) {
     const int code = a.code[k];
     Phase p;

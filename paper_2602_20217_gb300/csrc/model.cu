@@ -1112,13 +1112,17 @@ ks_status ks_prefill(ks_model* m, const int32_t* tokens, int32_t n, int32_t* nex
     // the last rows leave their history and logits; pending = argmax of the last
     const int lastlen = (n <= R) ? n : R;
     const size_t row_bytes = sizeof(float) * (size_t)R * c.d_model;   // a plane's rows of one history entry
-    // A wide pass costs about what three passes of 9 to 16 rows or four of up
-    // to 8 cost (four Llama-3-8B layers: 820 us at any length up to 256 against
-    // 1385, 1780, 2724 us at 32, 33 and 64 tokens in passes of 16).
+    // From where no shape loses by the wide pass, whose time hardly depends on
+    // the length up to 256.  Passes / wide in us, max_rows 16, at 32 and 33
+    // tokens: four layers of the Llama-3-8B shape 891 / 822, 1241 / 823; two of
+    // the Qwen3-32B shape 842 / 631, 1183 / 633; four of width 1536 474 / 457,
+    // 630 / 460; eight of width 512 737 / 652, 979 / 658 (at 17 tokens 637 / 642,
+    // width 1536 419 / 451).  max_rows 8 at 24 and 25 tokens: 8B 1173 / 822, 1517
+    // / 828; width 1536 574 / 454, 726 / 461; at 8 tokens every shape loses.
     const int passes = (n + R - 1) / R;
     const bool wide = m->lay.wide_rows > 0 && passes * (R > 8 ? 3 : 2) > 7;
     if (wide) {
-        // even wide chunks of whole tiles; the last rows' states go to the
+        // chunks of whole tiles, equal but for the last; the last rows' states go to the
         // snapshot of the history entry, from where the LM head takes them
         const int parts = (n + m->lay.wide_rows - 1) / m->lay.wide_rows;
         const int rows = std::min(m->lay.wide_rows, (int)align_up((size_t)(n + parts - 1) / parts, 256));

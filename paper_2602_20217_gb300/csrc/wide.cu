@@ -6,9 +6,10 @@
 // tensor cores idle: a 4096-token prompt read every weight 256 times.  Two
 // layers of the Llama-3-8B shape over 4096 tokens: 90.5 -> 2.74 ms for the whole
 // prefill; two of the Qwen3-32B shape over 9001: 391 -> 14.3 ms.  What bounds it
-// is the tensor pipe: at 2048 rows the gate/up GEMM of the 8B shape takes 262 us
-// (1835 TFLOP/s, pipe 85 % active), W_down 153, QKV 75 and W_o 55 (fewer tiles
-// than two rounds of all pairs, so the last round and the epilogues show).
+// is the tensor pipe: at 2048 rows the gate/up GEMM of the 8B shape takes 264 us
+// (1821 TFLOP/s, pipe 84 % active), W_down 154, QKV 76 and W_o 55 (128 tiles of
+// W_down and W_o, 192 of QKV are 1.7 and 2.5 rounds of the 76 pairs, so the last
+// round and the epilogues show).
 //
 // One CTA pair (cta_group::2) works on a 256 x 256 tile: each CTA stages its
 // 128 rows of A and its half of the tile's 256 weight rows (K-major, 64-column
@@ -35,8 +36,9 @@
 //              (any order gives the same argmax): the LM head of the layer
 //              selection's candidate states, whose logits nobody reads.
 // The tiles that do not fill a last round of all pairs (all of them, for a few
-// hundred rows) are cut along K instead: their stages are dealt out to the
-// pairs in equal contiguous shares.  Every part of a cut tile leaves its sums
+// hundred rows) are cut along K where K is long (more than 7680 inputs) and the
+// tiles are few: their stages are dealt out to the pairs in equal contiguous
+// shares.  Every part of a cut tile leaves its sums
 // in global memory, and per group of 32 rows the part that arrives last (a
 // ticket) adds them in K order, puts the total back into its TMEM columns and
 // runs the epilogue.  No pair waits for another.
@@ -618,8 +620,10 @@ cudaError_t launch_wide(int kind, int hd, const WideArgs& args, cudaStream_t s) 
     a.tiles_n = wide_tiles_n(kind, a.N);
     // The tiles past the last full round of all pairs are cut along K where
     // that is shorter: their stages dealt out evenly, plus the partial sums'
-    // round trip (kMergeStages), against a round of whole tiles.  Whole
-    // prefills of four Llama-3-8B layers with kMergeStages at 16, 48, 112 and
+    // round trip (kMergeStages), against a round of whole tiles.  In the
+    // configured shapes that is W_down at most sizes (Llama-3-8B: up to 512 and
+    // 1280 to 1792 rows, not 768, 1024 or 2048) and W_o of the Qwen3-32B shape at
+    // 1024 and 2048.  Whole prefills of four Llama-3-8B layers with kMergeStages at 16, 48, 112 and
     // never cutting: 882, 850, 827, 943 us at 256 tokens (W_down: 16 tiles of
     // 224 stages), 2700, 2635, 2547, 2529 us at 2048 (128 tiles).
     const int tiles = a.tiles_m * a.tiles_n, kblocks = (a.K + kTileK - 1) / kTileK;

@@ -11,9 +11,10 @@
 //   O += P V           tcgen05.mma with P as the TMEM operand, V as it lies in
 //                      the cache (keys x head_dim: an MN-major operand)
 // The two query tiles alternate: while one is in its softmax, the tensor core
-// works on the other.  O is rescaled only when a row's maximum grew by more
-// than 2^8: the factor 2^(m - m_ref) of the rest stays exact in fp32 and bf16
-// alike (a power of two apart, the relative precision is the same).
+// works on the other (Shah et al., FlashAttention-3, 2024).  O is rescaled only
+// when a row's maximum grew by more than 2^8 (the conditional rescaling known
+// from FlashAttention-4): the factor 2^(m - m_ref) of the rest stays exact in
+// fp32 and bf16 alike (a power of two apart, the relative precision is the same).
 // STATES: the rows are several states of r rows (the hidden-state DP's); all
 // see the cache's keys below p0, and each row its own state's rows up to
 // itself, so the key tiles are the cache's and then those of the block's own
@@ -22,8 +23,10 @@
 // still be NaN, for rows that do not see that key: in the tiles that some row
 // does not see whole (the last two or three of a CTA), a warp of its own clears
 // V rows that are not finite before they are used and notes their keys, and the
-// rows that do see such a key get NaN.  It takes half a microsecond a tile,
-// under the softmax of the tile's scores.
+// rows that do see such a key get NaN.  It works under the softmax of the tile's
+// scores: the DP over 16 sublayers (eight launches of 276 rows) takes 2713 us with
+// it, 2731 with the check in the MMA warp, 2700 without; prompts of 4096 and 9001
+// tokens differ by less than their runs.
 // Queries come prepared (QK-norm, RoPE, log2(e) / sqrt(hd)), the keys and
 // values of these rows are already in the cache.
 //
